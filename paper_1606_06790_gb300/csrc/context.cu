@@ -81,11 +81,6 @@ uint64_t sm64_at(uint64_t s, uint64_t k) { return sm64_mix(s + (k + 1ull) * 0x9E
 
 }  // namespace
 
-// Autotuned tile shape of one grouped-GEMM list.  Every shape gives the same
-// result bit for bit (each output element sums its K terms in the same
-// order), so the first calls of a list try each shape once on real work,
-// timed with CUDA events on the stream, and the fastest is kept until the
-// list's work changes by more than 10 %.
 // A grouped FP64 GEMM list in the digit-slice form (kernels_tc.cu): every
 // task's op(A) (M x K) and op(B)^T (N x K), K concatenated over its segments,
 // become digit planes in the context's digit arena, one exponent per packed
@@ -101,16 +96,12 @@ struct OzList {
   DevBuf dsegs, dtasks, dtiles;
 };
 
-struct GemmTune {
+// Device side of one grouped FP64 GEMM list: its tiles, or its digit-slice form.
+struct GemmDev {
   OzList oz;
   bool oz_use = false;  // list eligible for the digit-slice form (environments, prediction, SVD)
-  DevBuf tiles[GEMM_NSHAPE];
-  int ntiles[GEMM_NSHAPE] = {0, 0, 0, 0};
-  int choice = -1;
-  int state[GEMM_NSHAPE] = {0, 0, 0, 0};  // 0 untried, 1 timing, 2 timed
-  float ms[GEMM_NSHAPE] = {0, 0, 0, 0};
-  cudaEvent_t e0[GEMM_NSHAPE] = {}, e1[GEMM_NSHAPE] = {};
-  double work = -1.0;
+  DevBuf tiles;
+  int ntiles = 0;
 };
 
 // Uniform MPS of Eq. mps2 (observables): the unit's l site tensors A_k
@@ -316,8 +307,8 @@ struct idmrg_ctx {
   // FP32-preconditioned Jacobi: G = V^T V, W = V G (Newton-Schulz), X = B V
   GemmList svdG, svdW, svdX;
   DevBuf dsgk, dsgs, dswk, dsws, dsxk, dsxs;
-  // tile-shape autotuning of every grouped-GEMM list
-  GemmTune tn_g1, tn_g3, tn_gp, tn_env1, tn_env3, tn_svdG, tn_svdW, tn_svdX;
+  // device side of every grouped-GEMM list
+  GemmDev gd_g1, gd_g3, gd_gp, gd_env1, gd_env3, gd_svdG, gd_svdW, gd_svdX;
   int64_t tmaxel_all = 0;
 
   int svd_jobs = 0, svd_max_cols = 0, svd_max_rank = 0, svd_max_sweeps = 0;
@@ -620,66 +611,20 @@ idmrg_status oz_run(idmrg_ctx *c, OzList &Z) {
   return IDMRG_OK;
 }
 
-// tiles of every shape (L.tiles ends with the 64 x 64 ones) plus tasks and
-// segments to the device
-idmrg_status gemm_upload(idmrg_ctx *c, GemmList &L, DevBuf &dk, DevBuf &ds, GemmTune &T) {
+// tiles, tasks and segments of a list (or its digit-slice form) to the device
+idmrg_status gemm_upload(idmrg_ctx *c, GemmList &L, DevBuf &dk, DevBuf &ds, GemmDev &T) {
   T.oz.ok = false;
   if (T.oz_use && c->oz_lists()) return oz_build(c, L, T.oz);
-  for (int sh = GEMM_NSHAPE - 1; sh >= 0; --sh) {
-    L.finish(GEMM_TM[sh], GEMM_TN[sh]);
-    T.ntiles[sh] = (int)L.tiles.size();
-    NOMEM(c->upload(T.tiles[sh], L.tiles));
-  }
-  NOMEM(c->upload(dk, L.tasks) && c->upload(ds, L.segs));
-  const double w = L.flops;
-  if (T.work < 0.0 || fabs(w - T.work) > 0.1 * T.work) {  // new work: tune again
-    T.work = w;
-    T.choice = -1;
-    for (int sh = 0; sh < GEMM_NSHAPE; ++sh) T.state[sh] = 0;
-  }
+  L.finish();
+  T.ntiles = (int)L.tiles.size();
+  NOMEM(c->upload(T.tiles, L.tiles) && c->upload(dk, L.tasks) && c->upload(ds, L.segs));
   return IDMRG_OK;
 }
 
-idmrg_status gemm_run(idmrg_ctx *c, GemmTune &T, DevBuf &dk, DevBuf &ds, const int *active) {
+idmrg_status gemm_run(idmrg_ctx *c, GemmDev &T, DevBuf &dk, DevBuf &ds, const int *active) {
   if (T.oz.ok) return oz_run(c, T.oz);
-  double *const *bufs = (double *const *)c->dbufs.p;
-  int sh = T.choice;
-  if (sh < 0) {
-    bool all = true;
-    for (int k = 0; k < GEMM_NSHAPE; ++k) {
-      if (T.state[k] == 1 && cudaEventQuery(T.e1[k]) == cudaSuccess) {
-        cudaEventElapsedTime(&T.ms[k], T.e0[k], T.e1[k]);
-        T.state[k] = 2;
-      }
-      all &= T.state[k] == 2;
-    }
-    if (all) {
-      int best = 0;
-      for (int k = 1; k < GEMM_NSHAPE; ++k)
-        if (T.ms[k] < T.ms[best]) best = k;
-      T.choice = sh = best;
-    }
-  }
-  if (sh >= 0) {
-    CK(launch_gemm_f64((const GemmTile *)T.tiles[sh].p, T.ntiles[sh], (const GemmTask *)dk.p, (const GemmSeg *)ds.p,
-                       bufs, active, c->st, sh));
-    return IDMRG_OK;
-  }
-  int k = 0;
-  while (k < GEMM_NSHAPE && T.state[k] != 0) ++k;
-  if (k == GEMM_NSHAPE) k = 0;  // every shape in flight: the default
-  const bool timed = T.state[k] == 0;
-  if (timed) {
-    if (!T.e0[k]) CK(cudaEventCreate(&T.e0[k]));
-    if (!T.e1[k]) CK(cudaEventCreate(&T.e1[k]));
-    CK(cudaEventRecord(T.e0[k], c->st));
-  }
-  CK(launch_gemm_f64((const GemmTile *)T.tiles[k].p, T.ntiles[k], (const GemmTask *)dk.p, (const GemmSeg *)ds.p, bufs,
-                     active, c->st, k));
-  if (timed) {
-    CK(cudaEventRecord(T.e1[k], c->st));
-    T.state[k] = 1;
-  }
+  CK(launch_gemm_f64((const GemmTile *)T.tiles.p, T.ntiles, (const GemmTask *)dk.p, (const GemmSeg *)ds.p,
+                     (double *const *)c->dbufs.p, active, c->st));
   return IDMRG_OK;
 }
 
@@ -870,9 +815,9 @@ idmrg_status plan_iteration(idmrg_ctx *c) {
 
   // ---- device buffers for this iteration
   {
-    idmrg_status sg = gemm_upload(c, c->g1, c->dg1k, c->dg1s, c->tn_g1);
+    idmrg_status sg = gemm_upload(c, c->g1, c->dg1k, c->dg1s, c->gd_g1);
     if (sg != IDMRG_OK) return sg;
-    sg = gemm_upload(c, c->g3, c->dg3k, c->dg3s, c->tn_g3);
+    sg = gemm_upload(c, c->g3, c->dg3k, c->dg3s, c->gd_g3);
     if (sg != IDMRG_OK) return sg;
   }
   NOMEM(c->upload(c->dwt, c->wl.tasks) && c->upload(c->dwm, c->wl.terms));
@@ -1643,7 +1588,7 @@ idmrg_status heff_launch_fp64(idmrg_ctx *c, const int *active_dev, const int *ac
   const int kg = c->mixed ? IDMRG_K_HEFF_F64 : IDMRG_K_HEFF_GEMM;  // (FP64 GEMMs)
   c->kbegin(kg);
   {
-    idmrg_status sg_ = gemm_run(c, c->tn_g1, c->dg1k, c->dg1s, active_dev);
+    idmrg_status sg_ = gemm_run(c, c->gd_g1, c->dg1k, c->dg1s, active_dev);
     if (sg_ != IDMRG_OK) return sg_;
   }
   c->kend(kg, 0.0, 0.0);
@@ -1653,7 +1598,7 @@ idmrg_status heff_launch_fp64(idmrg_ctx *c, const int *active_dev, const int *ac
   c->kend(IDMRG_K_HEFF_WSTAGE, wf, 0.0);
   c->kbegin(kg);
   {
-    idmrg_status sg_ = gemm_run(c, c->tn_g3, c->dg3k, c->dg3s, active_dev);
+    idmrg_status sg_ = gemm_run(c, c->gd_g3, c->dg3k, c->dg3s, active_dev);
     if (sg_ != IDMRG_OK) return sg_;
   }
   c->kend(kg, gf, by);
@@ -1793,14 +1738,14 @@ idmrg_status predict(idmrg_ctx *c, int p) {
     NOMEM(sync_bufs(c) == IDMRG_OK);
     NOMEM(c->upload(c->dst, c->stasks) && c->upload(c->dstab, c->stable));
     {
-      idmrg_status sg = gemm_upload(c, c->gp, c->dgpk, c->dgps, c->tn_gp);
+      idmrg_status sg = gemm_upload(c, c->gp, c->dgpk, c->dgps, c->gd_gp);
       if (sg != IDMRG_OK) return sg;
     }
     c->kbegin(IDMRG_K_PREDICT);
     CK(launch_scale_tasks((const ScaleTask *)c->dst.p, (int)c->stasks.size(), c->smax_rows,
                           (const double *)c->dstab.p, c->o.lambda_zero_rel, bufs, c->st));
     {
-    idmrg_status sg_ = gemm_run(c, c->tn_gp, c->dgpk, c->dgps, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_gp, c->dgpk, c->dgps, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
     c->kend(IDMRG_K_PREDICT, c->gp.flops, 0.0);
@@ -1942,12 +1887,8 @@ idmrg_status lanczos(idmrg_ctx *c, int p) {
     c->launches += 4;
     if (r == 0) CK(c->d2h_copy(nrm2.data(), c->lresid.p, 8 * P));  // ||psi~|| for the report
     for (int it = 0; it < inner_cap; ++it) {
-      // the same iteration as a graph once the kernels of its matvec are
-      // fixed (reduced precision, or FP64 with tuned GEMM tiles)
       const bool fp64 = it == 0 || !c->mixed;
-      const bool as_graph = graph_ok && !c->prof &&
-                            (fp64 ? (c->oz_active() || (!c->mixed && c->tn_g1.choice >= 0 && c->tn_g3.choice >= 0))
-                                  : true);
+      const bool as_graph = graph_ok && !c->prof;
       if (as_graph && !iter_graph[fp64]) {
         const uint64_t l0 = c->launches, mm0 = c->mixed_matvecs, fm0 = c->fp64_matvecs;
         cudaGraph_t g = nullptr;
@@ -2236,9 +2177,9 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
         c->ensure(c->slam, 8 * std::max(sv, 1)) && c->ensure(c->seps, 8 * P) && c->ensure(c->sepsb, 8 * P) &&
         c->ensure(c->skept, 4 * P) && c->upload(c->sorder, c->torder) && c->upload(c->sorderq, c->torderq) &&
         c->ensure(c->slamk, 8 * (size_t)P * std::max(1, c->o.m)));
-  for (auto [L, dk, ds, T] : {std::make_tuple(&c->svdG, &c->dsgk, &c->dsgs, &c->tn_svdG),
-                               std::make_tuple(&c->svdW, &c->dswk, &c->dsws, &c->tn_svdW),
-                               std::make_tuple(&c->svdX, &c->dsxk, &c->dsxs, &c->tn_svdX)}) {
+  for (auto [L, dk, ds, T] : {std::make_tuple(&c->svdG, &c->dsgk, &c->dsgs, &c->gd_svdG),
+                               std::make_tuple(&c->svdW, &c->dswk, &c->dsws, &c->gd_svdW),
+                               std::make_tuple(&c->svdX, &c->dsxk, &c->dsxs, &c->gd_svdX)}) {
     idmrg_status sg = gemm_upload(c, *L, *dk, *ds, *T);
     if (sg != IDMRG_OK) return sg;
   }
@@ -2420,17 +2361,17 @@ idmrg_status truncate(idmrg_ctx *c, int p) {
   c->kbegin(PH + 2);
   for (int it = 0; it < 2; ++it) {
     {
-    idmrg_status sg_ = gemm_run(c, c->tn_svdG, c->dsgk, c->dsgs, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_svdG, c->dsgk, c->dsgs, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
     {
-    idmrg_status sg_ = gemm_run(c, c->tn_svdW, c->dswk, c->dsws, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_svdW, c->dswk, c->dsws, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
     CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 1, sw, c->st));
   }
   {
-    idmrg_status sg_ = gemm_run(c, c->tn_svdX, c->dsxk, c->dsxs, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_svdX, c->dsxk, c->dsxs, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
   CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 2, sw, c->st));
@@ -2651,22 +2592,22 @@ idmrg_status update_envs(idmrg_ctx *c, int p) {
   }
   NOMEM(sync_bufs(c) == IDMRG_OK);
   {
-    idmrg_status sg = gemm_upload(c, c->genv1, c->dge1k, c->dge1s, c->tn_env1);
+    idmrg_status sg = gemm_upload(c, c->genv1, c->dge1k, c->dge1s, c->gd_env1);
     if (sg != IDMRG_OK) return sg;
-    sg = gemm_upload(c, c->genv3, c->dge3k, c->dge3s, c->tn_env3);
+    sg = gemm_upload(c, c->genv3, c->dge3k, c->dge3s, c->gd_env3);
     if (sg != IDMRG_OK) return sg;
   }
   NOMEM(c->upload(c->dwet, c->wenv.tasks) && c->upload(c->dwem, c->wenv.terms));
   double *const *bufs = (double *const *)c->dbufs.p;
   c->kbegin(IDMRG_K_ENV);
   {
-    idmrg_status sg_ = gemm_run(c, c->tn_env1, c->dge1k, c->dge1s, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_env1, c->dge1k, c->dge1s, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
   CK(launch_wstage_f64((const WTask *)c->dwet.p, (int)c->wenv.tasks.size(), c->wenv.max_rows,
                        (const WTerm *)c->dwem.p, bufs, nullptr, c->st));
   {
-    idmrg_status sg_ = gemm_run(c, c->tn_env3, c->dge3k, c->dge3s, nullptr);
+    idmrg_status sg_ = gemm_run(c, c->gd_env3, c->dge3k, c->dge3s, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
   c->kend(IDMRG_K_ENV, c->genv1.flops + c->wenv.flops + c->genv3.flops, 0.0);
@@ -2766,8 +2707,8 @@ void obs_left_map(const ObsState &S, int d, int k, const double *O, double alpha
       }
     }
   }
-  g1.finish(32, 32);
-  g2.finish(32, 32);
+  g1.finish();
+  g2.finish();
 }
 
 // out = alpha sum_t A_k[t] in A_k[t]^T
@@ -2798,8 +2739,8 @@ void obs_right_map(const ObsState &S, int d, int k, double alpha, int in_buf, in
              S.aoff[k] + t * plane + (int64_t)B0[rb].first * Dk1 + B1[cb].first, Dk1, B1[cb].second, 2, alpha);
     }
   }
-  g1.finish(32, 32);
-  g2.finish(32, 32);
+  g1.finish();
+  g2.finish();
 }
 
 idmrg_status obs_upload(idmrg_ctx *c, ObsArena &a) {
@@ -2809,7 +2750,7 @@ idmrg_status obs_upload(idmrg_ctx *c, ObsArena &a) {
 
 idmrg_status obs_run(idmrg_ctx *c, ObsArena &a, const ObsList &L) {
   CK(launch_gemm_f64((const GemmTile *)a.dtiles.p + L.tile0, L.ntile, (const GemmTask *)a.dtasks.p,
-                     (const GemmSeg *)a.dsegs.p, (double *const *)c->obs.tab.p, nullptr, c->st, GEMM_32x32));
+                     (const GemmSeg *)a.dsegs.p, (double *const *)c->obs.tab.p, nullptr, c->st));
   c->launches += 1;
   return IDMRG_OK;
 }
@@ -3493,7 +3434,7 @@ idmrg_status idmrg_create_batch(const idmrg_mpo *mpos, int nmpo, const int *m_pe
     return bail(IDMRG_EINVAL);
   c->mixed = opts->prec == IDMRG_TF32X3 || opts->prec == IDMRG_BF16X3;
   c->fp64tc = opts->prec == IDMRG_FP64_TC;
-  for (GemmTune *t : {&c->tn_gp, &c->tn_env1, &c->tn_env3, &c->tn_svdG, &c->tn_svdW, &c->tn_svdX}) t->oz_use = true;
+  for (GemmDev *t : {&c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX}) t->oz_use = true;
   c->bf16 = opts->prec == IDMRG_BF16X3 ? 1 : 0;
   c->inner_factor = c->bf16 ? 1e-2 : 1e-3;
   c->d = d;
@@ -3683,15 +3624,11 @@ void idmrg_destroy(idmrg_ctx *c) {
   for (cudaStream_t x : c->side)
     if (x) cudaStreamDestroy(x);
   if (c->pin_act) cudaFreeHost(c->pin_act);
-  for (GemmTune *t : {&c->tn_g1, &c->tn_g3, &c->tn_gp, &c->tn_env1, &c->tn_env3, &c->tn_svdG, &c->tn_svdW, &c->tn_svdX}) {
-    for (auto &b : t->tiles) rel(b);
+  for (GemmDev *t : {&c->gd_g1, &c->gd_g3, &c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX}) {
+    rel(t->tiles);
     rel(t->oz.dsegs);
     rel(t->oz.dtasks);
     rel(t->oz.dtiles);
-    for (int k = 0; k < GEMM_NSHAPE; ++k) {
-      if (t->e0[k]) cudaEventDestroy(t->e0[k]);
-      if (t->e1[k]) cudaEventDestroy(t->e1[k]);
-    }
   }
   for (cudaEvent_t e : c->ev_act)
     if (e) cudaEventDestroy(e);
@@ -4486,12 +4423,12 @@ extern "C" idmrg_status idmrg_heff_apply_noalloc(idmrg_ctx *c, int p, const doub
                                              c->hbufs[p * NBUF + BUF_L], c->hbufs[p * NBUF + BUF_R],
                                              const_cast<double *>(psi_dev), out_dev, t1, t3);
   CK(cudaGetLastError());
-  CK(launch_gemm_f64((const GemmTile *)c->tn_g1.tiles[GEMM_64x64].p, c->tn_g1.ntiles[GEMM_64x64],
-                     (const GemmTask *)c->dg1k.p, (const GemmSeg *)c->dg1s.p, bufs, active, c->st, GEMM_64x64));
+  CK(launch_gemm_f64((const GemmTile *)c->gd_g1.tiles.p, c->gd_g1.ntiles,
+                     (const GemmTask *)c->dg1k.p, (const GemmSeg *)c->dg1s.p, bufs, active, c->st));
   CK(launch_wstage_f64((const WTask *)c->dwt.p, (int)c->wl.tasks.size(), c->wl.max_rows, (const WTerm *)c->dwm.p,
                        bufs, active, c->st));
-  CK(launch_gemm_f64((const GemmTile *)c->tn_g3.tiles[GEMM_64x64].p, c->tn_g3.ntiles[GEMM_64x64],
-                     (const GemmTask *)c->dg3k.p, (const GemmSeg *)c->dg3s.p, bufs, active, c->st, GEMM_64x64));
+  CK(launch_gemm_f64((const GemmTile *)c->gd_g3.tiles.p, c->gd_g3.ntiles,
+                     (const GemmTask *)c->dg3k.p, (const GemmSeg *)c->dg3s.p, bufs, active, c->st));
   c->launches += 4;
   return IDMRG_OK;
 }

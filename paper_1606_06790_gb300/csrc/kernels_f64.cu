@@ -16,90 +16,111 @@ namespace idmrg {
 
 namespace {
 
-// Tile shapes of the grouped GEMM: TM x TN outputs per CTA, 4 x 4 per
-// thread, K in steps of TK.  On this part one 64 x 64 tile holds an SM's
-// FP64 units for K x 2048 cycles, so the shape that wastes least in padding
-// and in the last wave differs between task lists; the host's autotuner
-// times each shape on real calls and keeps the fastest.
-constexpr int TK = 16;
+// Grouped GEMM.  The FP64 units bound it, by far: an SM retires one warp-wide
+// FMA per 16 cycles (2 FMA lanes per clock), each holding its sub-partition's
+// unit for 64, whereas the operands of even a 16 x 16 tile come to 2 bytes per
+// clock and SM.  So the split serves the FP64 units alone:
+//  * 16 x 16 outputs per CTA, one 8 x 8 quadrant per warp (2 outputs a lane):
+//    a warp on each sub-partition, 128 cycles per k whatever the problem, and
+//    no more padding than a ragged 8 x 8 quadrant (quadrants outside the task
+//    issue nothing).  The 64 x 64 .. 32 x 32 tiles before it (4 x 4 outputs a
+//    lane) took 1024 cycles per k on the two sub-partitions they occupied when
+//    the chip was not full, and padded every sector to their size.
+//  * exact trip counts in k: sectors of a few states are common, and a padded
+//    k costs as much as a real one.
+//  * the next K step is on its way to registers while the current one is
+//    multiplied out of shared memory (two buffers, one barrier per step).
+// The k order of every output is the segments' order, so the results do not
+// depend on the tiling.  Task lists hold 32 x 32 tiles; a CTA takes a quarter
+// of one (four times less list to build and upload).
+// Measured (GB300), the tuned 64 x 64 .. 32 x 32 tiles before -> now: H_eff psi
+// of one superblock at m = 32 77 -> 26 us (the call), of the J1-J2 cylinder at
+// m = 200 1.13 -> 0.61 ms, of the 16-site chain at m = 500 3.74 -> 2.96 ms
+// (0.98 of 1.26 TFLOP/s), of the kagome cylinder at m = 700 21.6 -> 18.1 ms.
+constexpr int TK = 16, TS = 16;
 
-template <int TM, int TN>
-__global__ void __launch_bounds__(TM *TN / 16) gemm_f64_kernel(const GemmTile *__restrict__ tiles,
-                                                               const GemmTask *__restrict__ tasks,
-                                                               const GemmSeg *__restrict__ segs,
-                                                               double *const *__restrict__ bufs,
-                                                               const int *__restrict__ active) {
-  constexpr int NT = TM * TN / 16;
-  __shared__ double As[TK][TM + 1];
-  __shared__ double Bs[TK][TN + 1];
-  const GemmTile tile = tiles[blockIdx.x];
+__global__ void __launch_bounds__(128) gemm_f64_kernel(const GemmTile *__restrict__ tiles,
+                                                       const GemmTask *__restrict__ tasks,
+                                                       const GemmSeg *__restrict__ segs,
+                                                       double *const *__restrict__ bufs,
+                                                       const int *__restrict__ active) {
+  __shared__ double As[2][TK][TS + 1];
+  __shared__ __align__(16) double Bs[2][TK][TS + 2];
+  const GemmTile tile = tiles[blockIdx.x >> 2];
   const GemmTask task = tasks[tile.task];
-  if (active && !active[task.sb]) return;
-  const int tid = threadIdx.x;
-  const int tx = tid % (TN / 4), ty = tid / (TN / 4);
-  double acc[4][4];
+  const int m0 = tile.m0 + TS * ((blockIdx.x >> 1) & 1), n0 = tile.n0 + TS * (blockIdx.x & 1);
+  if (m0 >= task.M || n0 >= task.N || (active && !active[task.sb])) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wr = 8 * (warp >> 1), wc = 8 * (warp & 1);
+  const int r = wr + (lane >> 2), c = wc + 2 * (lane & 3);
+  const bool live = m0 + wr < task.M && n0 + wc < task.N;
+  double acc0 = 0.0, acc1 = 0.0;
+  double ra[2], rb[2];  // the step being fetched
+  GemmSeg sg{};
+  const double *A = nullptr, *B = nullptr;
+  int s = task.seg0 - 1, k0 = 0, kn = 0;  // segment, first k and length of the step being fetched
+  const int s_end = task.seg0 + task.nseg;
+  auto fetch = [&]() {
+    k0 += TK;
+    if (s < task.seg0 || k0 >= sg.K) {
+      k0 = 0;
+      do {
+        if (++s >= s_end) {
+          kn = 0;
+          return;
+        }
+        sg = segs[s];
+      } while (sg.K <= 0);
+      A = bufs[task.sb * NBUF + sg.a_buf] + sg.a_off;
+      B = bufs[task.sb * NBUF + sg.b_buf] + sg.b_off;
+    }
+    kn = min(TK, sg.K - k0);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-
-  for (int s = task.seg0; s < task.seg0 + task.nseg; ++s) {
-    const GemmSeg sg = segs[s];
-    const double *A = bufs[task.sb * NBUF + sg.a_buf] + sg.a_off;
-    const double *B = bufs[task.sb * NBUF + sg.b_buf] + sg.b_off;
-    const bool ta = sg.flags & 1, tb = sg.flags & 2;
-    const bool scale = sg.alpha != 1.0;
-    for (int k0 = 0; k0 < sg.K; k0 += TK) {
-      // A tile: TM x TK (op(A) rows m, cols k)
-#pragma unroll
-      for (int r = 0; r < (TM * TK) / NT; ++r) {
-        const int idx = tid + r * NT;
-        int m, k;
-        if (!ta) { m = idx / TK; k = idx % TK; } else { k = idx / TM; m = idx % TM; }
-        const int gm = tile.m0 + m, gk = k0 + k;
-        double v = 0.0;
-        if (gm < task.M && gk < sg.K) v = ta ? A[(int64_t)gk * sg.lda + gm] : A[(int64_t)gm * sg.lda + gk];
-        As[k][m] = scale ? v * sg.alpha : v;
+    for (int q = 0; q < 2; ++q) {
+      const int hi = (tid + 128 * q) >> 4, lo = tid & 15;
+      {
+        const int m = m0 + ((sg.flags & 1) ? lo : hi), k = (sg.flags & 1) ? hi : lo;
+        ra[q] = 0.0;
+        if (m < task.M && k < kn)
+          ra[q] = (sg.flags & 1) ? A[(int64_t)(k0 + k) * sg.lda + m] : A[(int64_t)m * sg.lda + k0 + k];
       }
-#pragma unroll
-      for (int r = 0; r < (TN * TK) / NT; ++r) {
-        const int idx = tid + r * NT;
-        int n, k;
-        if (!tb) { k = idx / TN; n = idx % TN; } else { n = idx / TK; k = idx % TK; }
-        const int gn = tile.n0 + n, gk = k0 + k;
-        double v = 0.0;
-        if (gn < task.N && gk < sg.K) v = tb ? B[(int64_t)gn * sg.ldb + gk] : B[(int64_t)gk * sg.ldb + gn];
-        Bs[k][n] = v;
+      {
+        const int n = n0 + ((sg.flags & 2) ? hi : lo), k = (sg.flags & 2) ? lo : hi;
+        rb[q] = 0.0;
+        if (n < task.N && k < kn)
+          rb[q] = (sg.flags & 2) ? B[(int64_t)n * sg.ldb + k0 + k] : B[(int64_t)(k0 + k) * sg.ldb + n];
       }
-      __syncthreads();
+    }
+  };
+  fetch();
+  for (int buf = 0; kn > 0; buf ^= 1) {
 #pragma unroll
-      for (int k = 0; k < TK; ++k) {
-        double a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[k][ty + (TM / 4) * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + (TN / 4) * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    for (int q = 0; q < 2; ++q) {
+      const int hi = (tid + 128 * q) >> 4, lo = tid & 15;
+      const double va = sg.alpha != 1.0 ? ra[q] * sg.alpha : ra[q];
+      if (sg.flags & 1) As[buf][hi][lo] = va;
+      else As[buf][lo][hi] = va;
+      if (sg.flags & 2) Bs[buf][lo][hi] = rb[q];
+      else Bs[buf][hi][lo] = rb[q];
+    }
+    const int n = kn;
+    __syncthreads();
+    fetch();
+    if (live) {
+#pragma unroll 4
+      for (int k = 0; k < n; ++k) {
+        const double a = As[buf][k][r];
+        const double2 b = *reinterpret_cast<const double2 *>(&Bs[buf][k][c]);
+        acc0 = fma(a, b.x, acc0);
+        acc1 = fma(a, b.y, acc1);
       }
-      __syncthreads();
     }
   }
-  double *C = bufs[task.sb * NBUF + task.c_buf] + task.c_off;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = tile.m0 + ty + (TM / 4) * i;
-    if (gm >= task.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = tile.n0 + tx + (TN / 4) * j;
-      if (gn >= task.N) continue;
-      double *p = C + (int64_t)gm * task.ldc + gn;
-      *p = task.accumulate ? *p + acc[i][j] : acc[i][j];
-    }
-  }
+  const int gm = m0 + r, gn = n0 + c;
+  if (gm >= task.M) return;
+  double *C = bufs[task.sb * NBUF + task.c_buf] + task.c_off + (int64_t)gm * task.ldc + gn;
+  if (gn < task.N) C[0] = task.accumulate ? C[0] + acc0 : acc0;
+  if (gn + 1 < task.N) C[1] = task.accumulate ? C[1] + acc1 : acc1;
 }
 
 constexpr int WROWS = 16;
@@ -196,14 +217,9 @@ __global__ void scale_tasks_kernel(const ScaleTask *__restrict__ tasks, const do
 }  // namespace
 
 cudaError_t launch_gemm_f64(const GemmTile *tiles, int ntiles, const GemmTask *tasks, const GemmSeg *segs,
-                            double *const *bufs, const int *active, cudaStream_t st, int shape) {
-  if (ntiles <= 0) return cudaGetLastError();
-  switch (shape) {
-    case GEMM_64x64: gemm_f64_kernel<64, 64><<<ntiles, 256, 0, st>>>(tiles, tasks, segs, bufs, active); break;
-    case GEMM_64x32: gemm_f64_kernel<64, 32><<<ntiles, 128, 0, st>>>(tiles, tasks, segs, bufs, active); break;
-    case GEMM_32x64: gemm_f64_kernel<32, 64><<<ntiles, 128, 0, st>>>(tiles, tasks, segs, bufs, active); break;
-    default: gemm_f64_kernel<32, 32><<<ntiles, 64, 0, st>>>(tiles, tasks, segs, bufs, active); break;
-  }
+                            double *const *bufs, const int *active, cudaStream_t st) {
+  static_assert(GEMM_TILE == 2 * TS, "a list tile is four CTA tiles");
+  if (ntiles > 0) gemm_f64_kernel<<<4 * ntiles, 128, 0, st>>>(tiles, tasks, segs, bufs, active);
   return cudaGetLastError();
 }
 

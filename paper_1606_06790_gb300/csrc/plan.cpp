@@ -81,12 +81,12 @@ void GemmList::seg(int a_buf, int64_t a_off, int lda, int b_buf, int64_t b_off, 
   flops += 2.0 * t.M * (double)t.N * K;
 }
 
-void GemmList::finish(int tm, int tn) {
+void GemmList::finish() {
   tiles.clear();
   for (size_t i = 0; i < tasks.size(); ++i) {
     const GemmTask &t = tasks[i];
-    for (int m0 = 0; m0 < t.M; m0 += tm)
-      for (int n0 = 0; n0 < t.N; n0 += tn) tiles.push_back(GemmTile{(int)i, m0, n0, 0});
+    for (int m0 = 0; m0 < t.M; m0 += GEMM_TILE)
+      for (int n0 = 0; n0 < t.N; n0 += GEMM_TILE) tiles.push_back(GemmTile{(int)i, m0, n0, 0});
   }
 }
 

@@ -63,7 +63,7 @@ struct GemmList {
   int task(int sb, int c_buf, int64_t c_off, int M, int N, int ldc, int accumulate = 0);
   void seg(int a_buf, int64_t a_off, int lda, int b_buf, int64_t b_off, int ldb, int K, int flags,
            double alpha = 1.0);
-  void finish(int tm, int tn);  // output tiles
+  void finish();  // output tiles
 };
 
 struct WList {
