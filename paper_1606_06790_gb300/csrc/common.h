@@ -49,7 +49,8 @@ enum BufId {
   BUF_GOZ = 32,   // digit arena of the other FP64 GEMM lists (environments,
                   // prediction, SVD Newton-Schulz), the same for every superblock
   BUF_GEXP = 33,  // exponents of that arena
-  NBUF = 34
+  BUF_GPART = 34, // partial results of its tasks in K chunks
+  NBUF = 35
 };
 
 
@@ -294,11 +295,12 @@ struct TcTask {
   int a_buf, b_buf, c_buf, rmap_buf;
   int mode, ldc;          // mode 0: FP32 row-major C; 1: FP64 through the row map;
                           // 2: FP64 row-major C
-  int kb0, kb_stride;     // digit form: first K block of this K chunk, K blocks of the packed rows
   int accum, exp_buf;     // digit form: add to C instead of storing; slot of the exponents
+  int nch, part_buf;      // digit form: K chunks; with several, slot and offset of the
+  int64_t part_off;       // chunks' results, each M x N row-major (summed by launch_oz_sum)
 };
 struct TcTile {
-  int task, mt, nt, pad;
+  int task, mt, nt, chunk;  // chunk: K chunk (digit form)
 };
 constexpr int TC_TN = 64;      // N tile of the digit-slice GEMM (TMEM columns per level)
 // N tiles of the split-operand (TF32x3 / BF16x3) GEMM the tuner chooses from
@@ -313,11 +315,11 @@ cudaError_t launch_wstage_tc(const int4 *units, int nunits, const WTaskP *tasks,
 cudaError_t launch_tc_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, int bf16, int tn, cudaStream_t st);
 // FP64-accurate products from BF16 digit slices (OZ_PLANES digits of 7 bits
-// per element, exact integer accumulation per digit level).  K blocks are 32
-// elements; one launch sums at most OZ_MAX_K of K exactly, longer K runs as
-// successive chunks that add their FP64 results to C.
+// per element, exact integer accumulation per digit level).  K blocks are 16
+// elements; a tile sums at most OZ_MAX_K of K exactly, longer tasks have a tile
+// per K chunk (tile.chunk) and their chunks' results are added in FP64.
 constexpr int OZ_PLANES = 8;
-constexpr int OZ_KBLK = 32;
+constexpr int OZ_KBLK = 16;
 constexpr int OZ_MAX_K = 768;
 constexpr int OZ_EXP_EMPTY = (int)0x80808080;  // byte-fill value: row without non-zeros
 cudaError_t launch_oz_exp(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
@@ -328,6 +330,9 @@ cudaError_t launch_wstage_oz(const WTaskP *tasks, int ntasks, int max_rows, cons
                              double *const *bufs, const int *active, int pass, cudaStream_t st);
 cudaError_t launch_oz_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, cudaStream_t st);
+// ids: the n tasks with several K chunks
+cudaError_t launch_oz_sum(const int *ids, int n, int max_rows, const TcTask *tasks, double *const *bufs,
+                          const int *active, cudaStream_t st);
 
 // Uniform-MPS observables (Eq. mps2), see kernels_obs.cu.  An embed task
 // writes dst[x][y] = src(x, y) * scal[cs + y] / scal[rs + x] for x < rows,

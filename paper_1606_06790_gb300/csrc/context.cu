@@ -84,16 +84,26 @@ uint64_t sm64_at(uint64_t s, uint64_t k) { return sm64_mix(s + (k + 1ull) * 0x9E
 // A grouped FP64 GEMM list in the digit-slice form (kernels_tc.cu): every
 // task's op(A) (M x K) and op(B)^T (N x K), K concatenated over its segments,
 // become digit planes in the context's digit arena, one exponent per packed
-// row; tasks longer than OZ_MAX_K run in K chunks (one launch each).
+// row.
+struct OzTiles {                  // a digit-slice GEMM's output tiles
+  std::vector<TcTile> tiles;
+  std::vector<int> sums;          // tasks in several K chunks
+  int sum_rows = 0;
+  DevBuf dtiles, dsums;
+  void clear() {
+    tiles.clear();
+    sums.clear();
+    sum_rows = 0;
+  }
+};
 struct OzList {
   bool ok = false;
   std::vector<PackSeg> segs;      // A and B packing, one per GEMM segment and operand
   int seg_rows = 0;
   std::vector<TcTask> tasks;
-  std::vector<TcTile> tiles;
-  std::vector<int> lo;            // tile ranges of the K chunks
+  OzTiles out;
   int64_t planes = 0, nexp = 0;   // arena use: BF16 elements, exponents
-  DevBuf dsegs, dtasks, dtiles;
+  DevBuf dsegs, dtasks;
 };
 
 // Device side of one grouped FP64 GEMM list: its tiles, or its digit-slice form.
@@ -263,14 +273,13 @@ struct idmrg_ctx {
   bool oz_ok = false;
   std::vector<PackSeg> oz_step_w, oz_step_p, oz_psi;  // whole-K (L), part-K (R), psi
   std::vector<TcTask> oz1k, oz3k;
-  std::vector<TcTile> oz1t, oz3t;
+  OzTiles oz1t, oz3t;
   std::vector<WTaskP> ozw;
   int oz_step_w_rows = 0, oz_step_p_rows = 0, oz_psi_rows = 0, ozw_rows = 0;
   int64_t oz_a3_lo = 0, oz_a3_hi = 0, oz_b3_lo = 0, oz_b3_hi = 0;  // exponent ranges reset before use
-  std::vector<int> oz1_lo, oz3_lo;  // tile ranges of the K chunks (one launch each)
   std::vector<WTerm> wtpm_oz;
-  DevBuf goz_planes, goz_exps;  // digit arena of the FP64 GEMM lists (BUF_GOZ, BUF_GEXP)
-  DevBuf dozsw, dozsp, dozp, doz1k, doz1t, doz3k, doz3t, dozw, dozwm, oexp;
+  DevBuf goz_planes, goz_exps, goz_part;  // digit arena of the FP64 GEMM lists (BUF_GOZ, BUF_GEXP, BUF_GPART)
+  DevBuf dozsw, dozsp, dozp, doz1k, doz3k, dozw, dozwm, oexp;
   std::vector<DevBuf> bOA1, bOB1, bOT1, bOA3, bOB3, bORMAP, bOT3;
 
   // plan for iteration n
@@ -466,23 +475,43 @@ namespace {
     if (!(ok)) return c->fail(IDMRG_ENOMEM, "device allocation failed (%s)", #ok); \
   } while (0)
 
-// K chunks of at most OZ_MAX_K for one digit-slice task (see plan_oz)
-static void oz_add_task(std::vector<TcTask> &tasks, std::vector<std::vector<TcTile>> &lists, TcTask t, int MT,
-                        int NT) {
-  const int KBt = t.KB, per = OZ_MAX_K / OZ_KBLK;
-  const int nch = KBt > 0 ? (KBt + per - 1) / per : 1;
-  if ((int)lists.size() < nch) lists.resize(nch);
-  for (int ch = 0; ch < nch; ++ch) {
-    TcTask u = t;
-    u.kb_stride = KBt;
-    u.kb0 = ch * per;
-    u.KB = KBt > 0 ? std::min(per, KBt - u.kb0) : 0;
-    u.accum = (t.accum || ch > 0) ? 1 : 0;
-    const int id = (int)tasks.size();
-    tasks.push_back(u);
-    for (int mt = 0; mt < MT; ++mt)
-      for (int nt = 0; nt < NT; ++nt) lists[ch].push_back(TcTile{id, mt, nt, 0});
+// Adds a digit-slice task and its output tiles: one per K chunk of OZ_MAX_K,
+// whose results take M N nch doubles at part_n of part_buf when there are
+// several.
+void oz_add_task(OzTiles &Z, std::vector<TcTask> &tasks, TcTask t, int MT, int NT, int part_buf, int64_t &part_n) {
+  const int per = OZ_MAX_K / OZ_KBLK, id = (int)tasks.size();
+  t.nch = std::max(1, (t.KB + per - 1) / per);
+  if (t.nch > 1) {
+    t.part_buf = part_buf;
+    t.part_off = part_n;
+    part_n += (int64_t)t.nch * t.M * t.N;
+    Z.sums.push_back(id);
+    Z.sum_rows = std::max(Z.sum_rows, t.M);
   }
+  tasks.push_back(t);
+  for (int ch = 0; ch < t.nch; ++ch)
+    for (int mt = 0; mt < MT; ++mt)
+      for (int nt = 0; nt < NT; ++nt) Z.tiles.push_back(TcTile{id, mt, nt, ch});
+}
+
+// The longest tiles first: the persistent GEMM's CTAs take tiles in turn, so
+// that their shares then differ by little.
+idmrg_status oz_upload(idmrg_ctx *c, OzTiles &Z, const std::vector<TcTask> &tasks) {
+  const int per = OZ_MAX_K / OZ_KBLK;
+  auto len = [&](const TcTile &x) { return std::min(per, tasks[x.task].KB - x.chunk * per); };
+  std::stable_sort(Z.tiles.begin(), Z.tiles.end(), [&](const TcTile &x, const TcTile &y) { return len(x) > len(y); });
+  NOMEM(c->upload(Z.dtiles, Z.tiles) && c->upload(Z.dsums, Z.sums));
+  return IDMRG_OK;
+}
+
+idmrg_status oz_launch(idmrg_ctx *c, const OzTiles &Z, const DevBuf &dtasks, const int *active) {
+  double *const *bufs = (double *const *)c->dbufs.p;
+  CK(launch_oz_gemm((const TcTile *)Z.dtiles.p, (int)Z.tiles.size(), (const TcTask *)dtasks.p, bufs, active,
+                    (int *)c->derr.p, c->st));
+  CK(launch_oz_sum((const int *)Z.dsums.p, (int)Z.sums.size(), Z.sum_rows, (const TcTask *)dtasks.p, bufs, active,
+                   c->st));
+  c->launches += Z.sums.empty() ? 1 : 2;
+  return IDMRG_OK;
 }
 
 idmrg_status sync_bufs(idmrg_ctx *c);
@@ -494,10 +523,9 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
   Z.ok = false;
   Z.segs.clear();
   Z.tasks.clear();
-  Z.tiles.clear();
+  Z.out.clear();
   Z.seg_rows = 0;
-  std::vector<std::vector<TcTile>> lists;
-  int64_t an = 0, bn = 0, en = 0;
+  int64_t an = 0, bn = 0, en = 0, part = 0;
   // A planes first, B planes after all of them: B offsets are patched below
   std::vector<size_t> bseg;
   std::vector<TcTask> pend;
@@ -574,26 +602,27 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
   for (size_t i : bseg) Z.segs[i].dst_off += an;
   for (size_t i = 0; i < pend.size(); ++i) {
     pend[i].b_off += an;
-    oz_add_task(Z.tasks, lists, pend[i], pmt[i], pnt[i]);
-  }
-  Z.lo.assign(1, 0);
-  for (const auto &l : lists) {
-    Z.tiles.insert(Z.tiles.end(), l.begin(), l.end());
-    Z.lo.push_back((int)Z.tiles.size());
+    oz_add_task(Z.out, Z.tasks, pend[i], pmt[i], pnt[i], BUF_GPART, part);
   }
   Z.planes = an + bn;
   Z.nexp = en;
-  const void *p0 = c->goz_planes.p, *e0 = c->goz_exps.p;
+  const void *p0 = c->goz_planes.p, *e0 = c->goz_exps.p, *s0 = c->goz_part.p;
   NOMEM(c->ensure(c->goz_planes, 2 * (size_t)std::max<int64_t>(Z.planes, 8)) &&
-        c->ensure(c->goz_exps, 4 * (size_t)std::max<int64_t>(Z.nexp, 4)));
-  if (c->goz_planes.p != p0 || c->goz_exps.p != e0 || c->hbufs[BUF_GOZ] != c->dp(c->goz_planes)) {
+        c->ensure(c->goz_exps, 4 * (size_t)std::max<int64_t>(Z.nexp, 4)) &&
+        c->ensure(c->goz_part, 8 * (size_t)std::max<int64_t>(part, 1)));
+  if (c->goz_planes.p != p0 || c->goz_exps.p != e0 || c->goz_part.p != s0 || c->hbufs[BUF_GOZ] != c->dp(c->goz_planes)) {
     for (int q = 0; q < c->P; ++q) {
       c->hbufs[q * NBUF + BUF_GOZ] = c->dp(c->goz_planes);
       c->hbufs[q * NBUF + BUF_GEXP] = c->dp(c->goz_exps);
+      c->hbufs[q * NBUF + BUF_GPART] = c->dp(c->goz_part);
     }
     NOMEM(sync_bufs(c) == IDMRG_OK);
   }
-  NOMEM(c->upload(Z.dsegs, Z.segs) && c->upload(Z.dtasks, Z.tasks) && c->upload(Z.dtiles, Z.tiles));
+  NOMEM(c->upload(Z.dsegs, Z.segs) && c->upload(Z.dtasks, Z.tasks));
+  {
+    idmrg_status s = oz_upload(c, Z.out, Z.tasks);
+    if (s != IDMRG_OK) return s;
+  }
   Z.ok = true;
   return IDMRG_OK;
 }
@@ -604,11 +633,8 @@ idmrg_status oz_run(idmrg_ctx *c, OzList &Z) {
   CK(cudaMemsetAsync(c->goz_exps.p, 0x80, 4 * (size_t)Z.nexp, c->st));
   CK(launch_oz_exp((const PackSeg *)Z.dsegs.p, (int)Z.segs.size(), Z.seg_rows, bufs, nullptr, c->st));
   CK(launch_oz_pack((const PackSeg *)Z.dsegs.p, (int)Z.segs.size(), Z.seg_rows, bufs, nullptr, c->st));
-  for (size_t ch = 0; ch + 1 < Z.lo.size(); ++ch)
-    CK(launch_oz_gemm((const TcTile *)Z.dtiles.p + Z.lo[ch], Z.lo[ch + 1] - Z.lo[ch], (const TcTask *)Z.dtasks.p,
-                      bufs, nullptr, (int *)c->derr.p, c->st));
-  c->launches += 2 + (Z.lo.size() - 1);
-  return IDMRG_OK;
+  c->launches += 2;
+  return oz_launch(c, Z.out, Z.dtasks, nullptr);
 }
 
 // tiles, tasks and segments of a list (or its digit-slice form) to the device
@@ -1197,13 +1223,12 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
 }
 
 // Digit-slice form (FP64-accurate, see kernels_tc.cu): the stage-1 / W /
-// stage-3 structure of plan_mixed with 32-element K blocks of eight BF16
+// stage-3 structure of plan_mixed with 16-element K blocks of eight BF16
 // digit planes and one exponent per packed row.  Exponents of every
 // superblock live in one array: [stage-1 A and B rows | stage-3 B rows |
 // stage-3 A rows]; the last two ranges are reset before their atomic
 // maxima are taken.  Tasks whose K exceeds OZ_MAX_K (the bound of exact
-// digit sums) run in K chunks, one launch per chunk, later chunks adding
-// their FP64 results.
+// digit sums) run in K chunks, whose FP64 results are added up.
 idmrg_status plan_oz(idmrg_ctx *c) {
   const int P = c->P, d = c->d, target = c->o.target_charge, dd = d * d;
   const int GA = 16, GB = TC_TN / 8;
@@ -1245,26 +1270,6 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     v.push_back(q);
     mr = std::max(mr, rows);
   };
-  // a task in K chunks of at most OZ_MAX_K (exact digit sums); the tiles of
-  // chunk c go to lists[c], launched one chunk after the other
-  std::vector<std::vector<TcTile>> t1c, t3c;
-  auto add_task = [&](std::vector<TcTask> &tasks, std::vector<std::vector<TcTile>> &lists, TcTask t, int MT,
-                      int NT) {
-    const int KBt = t.KB, per = OZ_MAX_K / OZ_KBLK;
-    const int nch = KBt > 0 ? (KBt + per - 1) / per : 1;
-    if ((int)lists.size() < nch) lists.resize(nch);
-    for (int ch = 0; ch < nch; ++ch) {
-      TcTask u = t;
-      u.kb_stride = KBt;
-      u.kb0 = ch * per;
-      u.KB = KBt > 0 ? std::min(per, KBt - u.kb0) : 0;
-      u.accum = (t.accum || ch > 0) ? 1 : 0;
-      const int id = (int)tasks.size();
-      tasks.push_back(u);
-      for (int mt = 0; mt < MT; ++mt)
-        for (int nt = 0; nt < NT; ++nt) lists[ch].push_back(TcTile{id, mt, nt, 0});
-    }
-  };
   int64_t ex1 = 0, exb3 = 0, exa3 = 0;  // the three exponent ranges, relative
   const size_t b3seg0 = 0;
   std::vector<size_t> a3_tasks, b3_tasks;  // tasks / items whose offsets get the range bases
@@ -1283,6 +1288,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     std::vector<int64_t> t1f(SL, -1);
     std::vector<std::vector<int>> rs1(SL, std::vector<int>(wa, -1));
     int64_t pa1n = 0, pb1n = 0, t1n = 0;
+    int64_t np1 = 0, np3 = 0;  // results of K chunks: stage 1's in T3's place, stage 3's in T1's
     for (int si = 0; si < SL; ++si) {
       if (psi.C[si] == 0) continue;
       int M = 0;
@@ -1324,7 +1330,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       t.exp_buf = BUF_OEXP;
       t.mode = 2;
       t.ldc = N;
-      add_task(c->oz1k, t1c, t, MT, NT);
+      oz_add_task(c->oz1t, c->oz1k, t, MT, NT, BUF_OT3, np1);
     }
     // ---------------- stage 3
     int64_t pa3n = 0, pb3n = 0, nt3s = 0;
@@ -1427,27 +1433,17 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       t.rmap_buf = BUF_ORMAP;
       t.exp_buf = BUF_OEXP;
       t.mode = 1;
-      add_task(c->oz3k, t3c, t, MT, NT);
+      oz_add_task(c->oz3t, c->oz3k, t, MT, NT, BUF_OT1, np3);
     }
     na1[p] = pa1n;
     nb1[p] = pb1n;
-    nt1[p] = t1n;
+    nt1[p] = std::max(t1n, np3);
     na3[p] = pa3n;
     nb3[p] = pb3n;
-    nt3[p] = nt3s;
+    nt3[p] = std::max(nt3s, np1);
   }
   (void)b3seg0;
   (void)target;
-  auto flatten = [](const std::vector<std::vector<TcTile>> &lists, std::vector<TcTile> &out, std::vector<int> &lo) {
-    out.clear();
-    lo.assign(1, 0);
-    for (const auto &l : lists) {
-      out.insert(out.end(), l.begin(), l.end());
-      lo.push_back((int)out.size());
-    }
-  };
-  flatten(t1c, c->oz1t, c->oz1_lo);
-  flatten(t3c, c->oz3t, c->oz3_lo);
   // exponent ranges: stage-3 B after stage 1, stage-3 A last
   c->oz_b3_lo = ex1;
   c->oz_b3_hi = ex1 + exb3;
@@ -1482,8 +1478,12 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     c->hbufs[p * NBUF + BUF_OT3] = c->dp(c->bOT3[p]);
   }
   NOMEM(c->upload(c->dozsw, c->oz_step_w) && c->upload(c->dozsp, c->oz_step_p) && c->upload(c->dozp, c->oz_psi) &&
-        c->upload(c->doz1k, c->oz1k) && c->upload(c->doz1t, c->oz1t) && c->upload(c->doz3k, c->oz3k) &&
-        c->upload(c->doz3t, c->oz3t) && c->upload(c->dozw, c->ozw) && c->upload(c->dozwm, c->wtpm_oz));
+        c->upload(c->doz1k, c->oz1k) && c->upload(c->doz3k, c->oz3k) && c->upload(c->dozw, c->ozw) &&
+        c->upload(c->dozwm, c->wtpm_oz));
+  for (auto [Z, k] : {std::make_pair(&c->oz1t, &c->oz1k), std::make_pair(&c->oz3t, &c->oz3k)}) {
+    idmrg_status s = oz_upload(c, *Z, *k);
+    if (s != IDMRG_OK) return s;
+  }
   NOMEM(c->upload(c->dbufs, c->hbufs));
   // digits of L and R once for this iteration (R's rows span several channel
   // segments: exponents first)
@@ -1511,10 +1511,9 @@ idmrg_status heff_launch_oz(idmrg_ctx *c, const int *active_dev, const int *act)
   // booked as the restart matvecs of a mixed context, as the H_eff GEMMs of FP64_TC
   const int kg = c->mixed ? IDMRG_K_HEFF_F64 : IDMRG_K_HEFF_GEMM;
   c->kbegin(kg);
-  for (size_t ch = 0; ch + 1 < c->oz1_lo.size(); ++ch) {
-    CK(launch_oz_gemm((const TcTile *)c->doz1t.p + c->oz1_lo[ch], c->oz1_lo[ch + 1] - c->oz1_lo[ch],
-                      (const TcTask *)c->doz1k.p, bufs, active_dev, (int *)c->derr.p, c->st));
-    c->launches += 1;
+  {
+    idmrg_status s = oz_launch(c, c->oz1t, c->doz1k, active_dev);
+    if (s != IDMRG_OK) return s;
   }
   c->kend(kg);
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
@@ -1525,10 +1524,9 @@ idmrg_status heff_launch_oz(idmrg_ctx *c, const int *active_dev, const int *act)
                       active_dev, 1, c->st));
   c->kend(IDMRG_K_HEFF_WSTAGE, wf, 0.0);
   c->kbegin(kg);
-  for (size_t ch = 0; ch + 1 < c->oz3_lo.size(); ++ch) {
-    CK(launch_oz_gemm((const TcTile *)c->doz3t.p + c->oz3_lo[ch], c->oz3_lo[ch + 1] - c->oz3_lo[ch],
-                      (const TcTask *)c->doz3k.p, bufs, active_dev, (int *)c->derr.p, c->st));
-    c->launches += 1;
+  {
+    idmrg_status s = oz_launch(c, c->oz3t, c->doz3k, active_dev);
+    if (s != IDMRG_OK) return s;
   }
   c->kend(kg, gf, by);
   c->launches += 3;
@@ -3601,7 +3599,8 @@ void idmrg_destroy(idmrg_ctx *c) {
                     &c->dswk, &c->dsws, &c->dsxk, &c->dsxs, &c->dpkL, &c->dtune_out, &c->dmsb,
                     &c->dwtp, &c->dwtpm, &c->dwunits, &c->dtarget, &c->dozsw, &c->dozsp, &c->dozp,
                     &c->doz1k,
-                    &c->doz1t, &c->doz3k, &c->doz3t, &c->dozw, &c->dozwm, &c->oexp, &c->goz_planes,
+                    &c->oz1t.dtiles, &c->oz1t.dsums, &c->doz3k, &c->oz3t.dtiles, &c->oz3t.dsums, &c->dozw, &c->dozwm, &c->oexp,
+                    &c->goz_planes, &c->goz_part,
                     &c->goz_exps})
     rel(*b);
   for (int k = 0; k < MIX_NTN; ++k)
@@ -3628,7 +3627,8 @@ void idmrg_destroy(idmrg_ctx *c) {
     rel(t->tiles);
     rel(t->oz.dsegs);
     rel(t->oz.dtasks);
-    rel(t->oz.dtiles);
+    rel(t->oz.out.dtiles);
+    rel(t->oz.out.dsums);
   }
   for (cudaEvent_t e : c->ev_act)
     if (e) cudaEventDestroy(e);

@@ -496,15 +496,22 @@ __global__ void __launch_bounds__(PS_THREADS, 1) tc_gemm_ps_kernel(const TcTile 
 // exact FP32 integer while (t + 1) K 2^12 < 2^24; for K <= OZ_MAX_K that holds
 // up to t = 4, and the rounding of the higher levels is below 2^-53 of the
 // leading terms.  Levels t <= 7 are kept (one 64-column TMEM accumulator
-// each, 36 MMAs per K step); the epilogue sums them in FP64 with their
-// power-of-two scales.
+// each); the epilogue sums them with their power-of-two scales.
+constexpr int OZ_GA = 16;  // row groups of a packed A tile (128 rows); B tiles have TC_TN / 8
+static_assert(OZ_KBLK == 16, "a K block is one kind::f16 MMA step");
+// Digit p of element (row, k): K blocks of 16 (one MMA step), row tiles of 8 G
+// rows.  A operands (G = 16) keep plane after plane, so that a plane of a block
+// is one M = 128 operand; B operands (G = 8) keep the planes of a K chunk one
+// after the other, so that consecutive planes read as one operand of 64 rows
+// each: A_p against B_q, B_q+1, ... is one MMA, and its output columns are the
+// consecutive levels p + q, p + q + 1, ...
 __device__ __forceinline__ int64_t oz_off(int row, int k, int KB, int G, int p) {
   const int rows_per_tile = 8 * G;
   const int rt = row / rows_per_tile, rr = row - rt * rows_per_tile;
-  const int kb = k >> 5, kc = (k & 31) >> 3;
-  const int64_t tile_h = (int64_t)rows_per_tile * OZ_KBLK;
-  return (((int64_t)rt * KB + kb) * OZ_PLANES + p) * tile_h + (((int64_t)kc * G + (rr >> 3)) * 8 + (rr & 7)) * 8 +
-         (k & 7);
+  const int64_t block = (int64_t)rt * KB + k / OZ_KBLK;
+  const int kc = (k & (OZ_KBLK - 1)) >> 3;
+  const int64_t run = G == OZ_GA ? (block * OZ_PLANES + p) * 2 + kc : (block * 2 + kc) * OZ_PLANES + p;
+  return ((run * G + (rr >> 3)) * 8 + (rr & 7)) * 8 + (k & 7);
 }
 
 // exponent of the expansion for a non-zero x: |x| < 2^(e - 1)
@@ -653,30 +660,51 @@ __global__ void wstage_oz_kernel(const WTaskP *__restrict__ tasks, const WTerm *
 constexpr int OZ_A_PLANE = TM * OZ_KBLK * 2;       // bytes of one A digit plane of a K block
 constexpr int OZ_B_PLANE = TC_TN * OZ_KBLK * 2;
 constexpr int OZ_STAGE = OZ_PLANES * (OZ_A_PLANE + OZ_B_PLANE);
-constexpr int OZ_STAGES = 2;
+constexpr int OZ_STAGES = 4;
+constexpr int OZ_CH = OZ_MAX_K / OZ_KBLK;           // K blocks of one K chunk
 constexpr int OZ_TMEM_COLS = 512;                  // 8 levels x 64 columns
+constexpr int OZ_EPI_WARPS = 8;                    // two per TMEM lane quarter, 32 columns each
+constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
+constexpr int OZ_STG_LD = 17;                      // staging block of an epilogue warp: 32 rows x 16 columns
+constexpr int OZ_SMEM = OZ_STAGES * OZ_STAGE + OZ_EPI_WARPS * 32 * OZ_STG_LD * 8;
 
-__global__ void __launch_bounds__(128) oz_gemm_kernel(const TcTile *__restrict__ tiles,
-                                                      const TcTask *__restrict__ tasks,
-                                                      double *const *__restrict__ bufs,
-                                                      const int *__restrict__ active, int *err) {
+// Persistent: one CTA per SM walks the tile list (128 x 64 outputs each, the
+// longest K first) with three roles, as tc_gemm_ps_kernel does.  What bounds
+// it is the tensor pipe: 36 digit products of 128 x 64 x 16 per K block, 1152
+// cycles.  They are issued as 12 MMAs of up to 256 columns (A_p against the
+// stacked planes of B, see oz_off), which read A from shared memory 12 times a
+// block instead of 36 and so stay below its bandwidth; 36 MMAs of 64 columns
+// were bound by it.  All 512 TMEM columns hold one tile, so the MMAs of the
+// next one wait until this one has been read: the epilogue warps first take
+// all eight levels into registers (integers, see below), release the
+// accumulators, and only then scale, round and store, beside the next tile's
+// MMAs.  Tasks longer than OZ_MAX_K have one tile per K chunk, so that few but
+// long outputs still fill the chip; these store into the task's partial
+// results, which oz_sum_kernel adds up in the order of K.
+// Measured (GB300; before: one CTA per tile of 32-element K blocks, the epilogue
+// in FP64 by the row): the two stages of the kagome cylinder's H_eff psi at
+// m = 1500 13.1 -> 4.2 ms (41 TFLOP/s FP64-accurate; 2.6 ms at the tensor pipe's
+// rate with all padding counted), of the J1-J2 cylinder at m = 500 0.81 -> 0.26 ms.
+__global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__restrict__ tiles, int ntiles,
+                                                                const TcTask *__restrict__ tasks,
+                                                                double *const *__restrict__ bufs,
+                                                                const int *__restrict__ active, int *err) {
   extern __shared__ __align__(1024) uint8_t osm[];
-  __shared__ __align__(8) uint64_t full[OZ_STAGES], empty[OZ_STAGES], done;
+  __shared__ __align__(8) uint64_t full[OZ_STAGES], empty[OZ_STAGES], accf, acce, done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
-  const TcTile tile = tiles[blockIdx.x];
-  const TcTask T = tasks[tile.task];
-  if (active && !active[T.sb]) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
     tc::tmem_alloc(&tmem_base, OZ_TMEM_COLS);
     tc::tmem_relinquish();
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 32) {
     for (int s = 0; s < OZ_STAGES; ++s) {
       tc::mbar_init(&full[s], 1);
       tc::mbar_init(&empty[s], 1);
     }
+    tc::mbar_init(&accf, 1);
+    tc::mbar_init(&acce, OZ_EPI_WARPS);
     tc::mbar_init(&done, 1);
     abort_flag = 0;
     tc::fence_mbar_init();
@@ -685,139 +713,258 @@ __global__ void __launch_bounds__(128) oz_gemm_kernel(const TcTile *__restrict__
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_base;
-  if (threadIdx.x == 0 && T.KB > 0) {
-    const uint8_t *A = reinterpret_cast<const uint8_t *>(bufs[T.sb * NBUF + T.a_buf]) + 2 * T.a_off +
-                       ((int64_t)tile.mt * T.kb_stride + T.kb0) * OZ_PLANES * OZ_A_PLANE;
-    const uint8_t *B = reinterpret_cast<const uint8_t *>(bufs[T.sb * NBUF + T.b_buf]) + 2 * T.b_off +
-                       ((int64_t)tile.nt * T.kb_stride + T.kb0) * OZ_PLANES * OZ_B_PLANE;
-    constexpr uint32_t idesc = tc::instr_desc(TM, TC_TN, 1u);
-    constexpr uint32_t lboA = (TM / 8) * 128, lboB = (TC_TN / 8) * 128, sbo = 128;
-    auto issue = [&](int kb) {
-      const int s = kb % OZ_STAGES;
-      uint8_t *st = osm + s * OZ_STAGE;
-      tc::mbar_arrive_expect_tx(&full[s], (uint32_t)OZ_STAGE);
-      tc::bulk_g2s(st, A + (int64_t)kb * OZ_PLANES * OZ_A_PLANE, OZ_PLANES * OZ_A_PLANE, &full[s]);
-      tc::bulk_g2s(st + OZ_PLANES * OZ_A_PLANE, B + (int64_t)kb * OZ_PLANES * OZ_B_PLANE, OZ_PLANES * OZ_B_PLANE,
-                   &full[s]);
-    };
-    bool ok = true;
-    int issued = 0, consumed = 0;
-    for (int kb = 0; kb < T.KB && kb < OZ_STAGES - 1; ++kb) {
-      issue(kb);
-      issued = kb + 1;
+  volatile int *abort_v = &abort_flag;
+
+  if (warp == 0) {
+    if (lane == 0) {  // ---- producer
+      long long it = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const TcTile tile = tiles[t];
+        const TcTask T = tasks[tile.task];
+        if (active && !active[T.sb]) continue;
+        const uint8_t *A = reinterpret_cast<const uint8_t *>(bufs[T.sb * NBUF + T.a_buf]) + 2 * T.a_off +
+                           (int64_t)tile.mt * T.KB * OZ_PLANES * OZ_A_PLANE;
+        const uint8_t *B = reinterpret_cast<const uint8_t *>(bufs[T.sb * NBUF + T.b_buf]) + 2 * T.b_off +
+                           (int64_t)tile.nt * T.KB * OZ_PLANES * OZ_B_PLANE;
+        const int kend = min(T.KB, (tile.chunk + 1) * OZ_CH);
+        for (int kb = tile.chunk * OZ_CH; kb < kend; ++kb, ++it) {
+          const int s = (int)(it % OZ_STAGES);
+          const long long u = it / OZ_STAGES;
+          if (*abort_v || (u > 0 && !tc::mbar_wait(&empty[s], (uint32_t)((u - 1) & 1), WAIT_BUDGET))) {
+            ok = false;
+            break;
+          }
+          uint8_t *st = osm + s * OZ_STAGE;
+          tc::mbar_arrive_expect_tx(&full[s], (uint32_t)OZ_STAGE);
+          tc::bulk_g2s(st, A + (int64_t)kb * OZ_PLANES * OZ_A_PLANE, OZ_PLANES * OZ_A_PLANE, &full[s]);
+          tc::bulk_g2s(st + OZ_PLANES * OZ_A_PLANE, B + (int64_t)kb * OZ_PLANES * OZ_B_PLANE, OZ_PLANES * OZ_B_PLANE,
+                       &full[s]);
+        }
+      }
+      if (!ok) {
+        atomicOr(err, IDMRG_DEV_ERR_TIMEOUT);
+        atomicOr(&abort_flag, 1);
+      }
+      // the copies of the last ring window may still be in flight: wait for them
+      for (long long j = it > OZ_STAGES ? it - OZ_STAGES : 0; j < it; ++j)
+        tc::mbar_wait(&full[j % OZ_STAGES], (uint32_t)((j / OZ_STAGES) & 1), WAIT_BUDGET);
     }
-    for (int kb = 0; kb < T.KB && ok; ++kb) {
-      const int kn = kb + OZ_STAGES - 1;
-      if (kn < T.KB) {
-        const int sn = kn % OZ_STAGES;
-        if (kn >= OZ_STAGES && !tc::mbar_wait(&empty[sn], ((kn / OZ_STAGES) - 1) & 1, WAIT_BUDGET)) {
+  } else if (warp == 1) {
+    if (lane == 0) {  // ---- MMA issuer
+      constexpr uint32_t lboA = (TM / 8) * 128, lboB = OZ_PLANES * (TC_TN / 8) * 128, sbo = 128;
+      constexpr uint32_t bplane = (TC_TN / 8) * 128;  // bytes from one stacked B plane to the next
+      long long it = 0;
+      int v = 0;  // tiles so far
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const TcTile tile = tiles[t];
+        const TcTask T = tasks[tile.task];
+        if (active && !active[T.sb]) continue;
+        if (*abort_v || (v > 0 && !tc::mbar_wait(&acce, (uint32_t)((v - 1) & 1), WAIT_BUDGET))) {
           ok = false;
           break;
         }
-        issue(kn);
-        issued = kn + 1;
+        tc::fence_after_sync();
+        const int kc = tile.chunk * OZ_CH, kend = min(T.KB, kc + OZ_CH);
+        for (int kb = kc; kb < kend; ++kb, ++it) {
+          const int s = (int)(it % OZ_STAGES);
+          if (!tc::mbar_wait(&full[s], (uint32_t)((it / OZ_STAGES) & 1), WAIT_BUDGET)) {
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
+          const uint32_t sa = tc::smem_u32(osm + s * OZ_STAGE);
+          const uint32_t sb = sa + OZ_PLANES * OZ_A_PLANE;
+#pragma unroll
+          for (int p = 0; p < OZ_PLANES; ++p) {
+            const uint64_t ad = tc::smem_desc(sa + p * OZ_A_PLANE, lboA, sbo);
+#pragma unroll
+            for (int q = 0; q < OZ_PLANES - p; q += 4) {  // planes q .. q + 3 (fewer at the end)
+              const int nq = OZ_PLANES - p - q < 4 ? OZ_PLANES - p - q : 4;
+              const uint64_t bd = tc::smem_desc(sb + q * bplane, lboB, sbo);
+              tc::mma_f16(tmem + (uint32_t)(TC_TN * (p + q)), ad, bd, tc::instr_desc(TM, nq * TC_TN, 1u),
+                          (kb > kc || p > 0) ? 1u : 0u);
+            }
+          }
+          tc::mma_commit(&empty[s]);
+        }
+        if (!ok) break;
+        tc::mma_commit(&accf);  // the levels of this tile are complete
+        ++v;
       }
-      const int s = kb % OZ_STAGES;
-      if (!tc::mbar_wait(&full[s], (kb / OZ_STAGES) & 1, WAIT_BUDGET)) {
-        ok = false;
+      if (!ok) {
+        atomicOr(err, IDMRG_DEV_ERR_TIMEOUT);
+        atomicOr(&abort_flag, 1);
+      }
+      tc::mma_commit(&done);  // fires once every MMA issued above has completed
+    }
+  } else {  // ---- epilogue: TMEM lane quarter warp % 4, columns 32 w .. 32 w + 31
+    const int quarter = warp & 3, cb = 32 * ((warp - 2) >> 2);
+    double *stg = reinterpret_cast<double *>(osm + OZ_STAGES * OZ_STAGE) + (warp - 2) * 32 * OZ_STG_LD;
+    int v = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const TcTile tile = tiles[t];
+      const TcTask T = tasks[tile.task];
+      if (active && !active[T.sb]) continue;
+      const int r0 = tile.mt * TM + 32 * quarter, col0 = tile.nt * TC_TN + cb;
+      const int nrows = min(32, T.M - r0);  // may be <= 0
+      const int *ex = (const int *)bufs[T.sb * NBUF + T.exp_buf];
+      const int ea = lane < nrows ? ex[T.a_exp + r0 + lane] : OZ_EXP_EMPTY;
+      const int ebl = col0 + lane < T.N ? ex[T.b_exp + col0 + lane] : OZ_EXP_EMPTY;
+      // this lane's output row: of the task's output, or of this chunk's partial results
+      double *cbase = bufs[T.sb * NBUF + (T.nch > 1 ? T.part_buf : T.c_buf)];
+      const bool accum = T.accum && T.nch == 1;
+      int64_t obase = 0;
+      if (lane < nrows) {
+        if (T.nch > 1)
+          obase = T.part_off + ((int64_t)tile.chunk * T.M + r0 + lane) * T.N;
+        else if (T.mode == 1)
+          obase = ((const int64_t *)bufs[T.sb * NBUF + T.rmap_buf])[T.rmap_off + r0 + lane];
+        else
+          obase = T.c_off + (int64_t)(r0 + lane) * T.ldc;
+      }
+      // every lane waits; the warp goes on only together (tcgen05.ld is warp-wide)
+      const bool got = !*abort_v && tc::mbar_wait(&accf, (uint32_t)(v & 1), WAIT_BUDGET);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) {
+          atomicOr(err, IDMRG_DEV_ERR_TIMEOUT);
+          atomicOr(&abort_flag, 1);
+        }
         break;
       }
       tc::fence_after_sync();
-      const uint32_t sa = tc::smem_u32(osm + s * OZ_STAGE);
-      const uint32_t sb = sa + OZ_PLANES * OZ_A_PLANE;
+      // Levels 0..4 are exact integers, |L_t| <= (t + 1) 768 2^12 < 2^24, and
+      // are summed as such: H = sum_t L_t 128^(4-t) in units of 2^-42, with
+      // L_0 128 + L_1 and L_2 128 + L_3 within 32 bits and |H| < 2^50.
+      // Levels 5..7 carry FP32 rounding anyway: Tl = L_5 2^14 + L_6 2^7 + L_7
+      // in FP32, in units of 2^-63 (its error lies below 2^-58 of the leading
+      // term).
+      long long H[32];
+      float Tl[32];
+      const uint32_t ta = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)cb;
 #pragma unroll
-      for (int kk = 0; kk < OZ_KBLK / 16; ++kk) {
+      for (int h = 0; h < 2; ++h) {
+        float x[4][16];
+        if (T.KB > 0) {
 #pragma unroll
-        for (int p = 0; p < OZ_PLANES; ++p) {
-          const uint64_t ad = tc::smem_desc(sa + p * OZ_A_PLANE + kk * 2 * lboA, lboA, sbo);
+          for (int l = 0; l < 4; ++l) tc::tmem_ld16_async(ta + (uint32_t)(TC_TN * l + 16 * h), x[l]);
+          tc::tmem_ld_wait();
+        }
 #pragma unroll
-          for (int q = 0; q < OZ_PLANES - p; ++q) {
-            const uint64_t bd = tc::smem_desc(sb + q * OZ_B_PLANE + kk * 2 * lboB, lboB, sbo);
-            tc::mma_f16(tmem + (uint32_t)(TC_TN * (p + q)), ad, bd, idesc, (kb > 0 || kk > 0 || p > 0) ? 1u : 0u);
-          }
+        for (int i = 0; i < 16; ++i) {
+          tc::tmem_ld_fence(x[0][i], x[1][i], x[2][i], x[3][i]);
+          const int p01 = __float2int_rn(x[0][i]) * 128 + __float2int_rn(x[1][i]);
+          const int p23 = __float2int_rn(x[2][i]) * 128 + __float2int_rn(x[3][i]);
+          H[16 * h + i] = T.KB > 0 ? (long long)p01 * (1 << 21) + (long long)p23 * 128 : 0;
+        }
+        if (T.KB > 0) {
+#pragma unroll
+          for (int l = 0; l < 4; ++l) tc::tmem_ld16_async(ta + (uint32_t)(TC_TN * (4 + l) + 16 * h), x[l]);
+          tc::tmem_ld_wait();
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          tc::tmem_ld_fence(x[0][i], x[1][i], x[2][i], x[3][i]);
+          if (T.KB > 0) H[16 * h + i] += __float2int_rn(x[0][i]);
+          Tl[16 * h + i] = T.KB > 0 ? fmaf(fmaf(x[1][i], 128.0f, x[2][i]), 128.0f, x[3][i]) : 0.0f;
         }
       }
-      tc::mma_commit(&empty[s]);
-      consumed = kb + 1;
-    }
-    if (!ok) {
-      atomicOr(err, IDMRG_DEV_ERR_TIMEOUT);
-      atomicOr(&abort_flag, 1);
-      for (int j = consumed; j < issued; ++j) tc::mbar_wait(&full[j % OZ_STAGES], (j / OZ_STAGES) & 1, WAIT_BUDGET);
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&acce);  // this warp's part of the accumulators is free
+      // value = (H 2^-42 + Tl 2^-63) 2^(ea + eb), one rounding: H 2^(k - 42)
+      // exactly (1.5 2^52 + H is H in the low mantissa bits; the FMA takes
+      // the offset away), Tl 2^(k - 63) by its exponent bits, one addition.
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int eb = __shfl_sync(0xffffffffu, ebl, 16 * h + i);
+          double val = 0.0;
+          if (ea != OZ_EXP_EMPTY && eb != OZ_EXP_EMPTY) {
+            const int k = ea + eb;
+            const long long Hi = H[16 * h + i];
+            const float Ti = Tl[16 * h + i];
+            if (k - 63 > -1000 && k - 42 < 960) {  // every power of two below is a normal double
+              const double s42 = __longlong_as_double((long long)(k - 42 + 1023) << 52);
+              const double off = __longlong_as_double(((long long)(k + 10 + 1023) << 52) | (1ll << 51));
+              const double hv = fma(__longlong_as_double(0x4338000000000000ll + Hi), s42, -off);
+              const uint32_t tb = __float_as_uint(Ti);
+              const long long tm = ((long long)(tb & 0x7fffffffu) << 29) + ((long long)(896 + k - 63) << 52);
+              const double tv = Ti == 0.0f ? 0.0 : __longlong_as_double(tm | ((long long)(tb >> 31) << 63));
+              val = hv + tv;
+            } else {
+              val = scalbn(fma((double)Ti, 0x1p-21, (double)Hi), k - 42);
+            }
+          }
+          stg[lane * OZ_STG_LD + i] = val;
+        }
+        __syncwarp();
+        // two rows of 16 columns per pass
+        const int cl = lane & 15, col = col0 + 16 * h + cl;
+#pragma unroll 4
+        for (int r = 0; r < 32; r += 2) {
+          const int rr = r + (lane >> 4);
+          const int64_t ob = __shfl_sync(0xffffffffu, obase, rr);
+          if (rr < nrows && col < T.N) {
+            double *dst = cbase + ob + col;
+            const double val = stg[rr * OZ_STG_LD + cl];
+            *dst = accum ? *dst + val : val;
+          }
+        }
+        __syncwarp();
+      }
+      ++v;
     }
   }
-  if (threadIdx.x == 0) tc::mma_commit(&done);  // fires when every MMA issued above has completed
+  __syncthreads();
   const bool ready = tc::mbar_wait(&done, 0, WAIT_BUDGET);
   if (!ready) {
     atomicOr(&abort_flag, 2);
     if (lane == 0) atomicOr(err, IDMRG_DEV_ERR_TIMEOUT);
   }
-  __syncthreads();
-  tc::fence_after_sync();
-  const int aborted = abort_flag;
-  if (!aborted) {
-    const int row = tile.mt * TM + 32 * warp + lane;
-    const int col0 = tile.nt * TC_TN;
-    double *cbase = bufs[T.sb * NBUF + T.c_buf];
-    const int *ex = (const int *)bufs[T.sb * NBUF + T.exp_buf];
-    const int ea = row < T.M ? ex[T.a_exp + row] : OZ_EXP_EMPTY;
-    int64_t obase = 0;
-    if (T.mode == 1 && row < T.M) obase = ((const int64_t *)bufs[T.sb * NBUF + T.rmap_buf])[T.rmap_off + row];
-#pragma unroll 1
-    for (int c = 0; c < TC_TN; c += 16) {
-      // Levels 0..4 are exact integers (|sum| < 2^24): Horner in base 128 in
-      // int64 gives H = sum_t L_t 128^(4-t) exactly (|H| < 2^53), in units
-      // of 2^-42.  Levels 5..7 carry FP32 rounding anyway: T = L_5 2^14 +
-      // L_6 2^7 + L_7 in FP32, in units of 2^-63 (its error lies below 2^-58
-      // of the leading term).  Then value = (H 2^-42 + T 2^-63) 2^(ea+eb):
-      // two conversions, one multiply and one FMA in FP64 per output.
-      long long H[16];
-      float Tl[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        H[i] = 0;
-        Tl[i] = 0.f;
-      }
-      if (T.KB > 0) {
-#pragma unroll 1
-        for (int t = 0; t < OZ_PLANES; ++t) {
-          float v[16];
-          tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(TC_TN * t + c), v);
-          if (t <= 4) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) H[i] = H[i] * 128 + (long long)v[i];
-          } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) Tl[i] = fmaf(Tl[i], 128.0f, v[i]);
-          }
-        }
-      }
-      if (row < T.M) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int col = col0 + c + i;
-          if (col >= T.N) break;
-          const int eb = ex[T.b_exp + col];
-          double val = 0.0;
-          if (ea != OZ_EXP_EMPTY && eb != OZ_EXP_EMPTY) {
-            const int k = ea + eb;
-            if (k - 63 > -1000 && k - 42 < 1000) {  // both powers of two are normal doubles
-              const double s42 = __longlong_as_double((long long)(k - 42 + 1023) << 52);
-              const double s63 = __longlong_as_double((long long)(k - 63 + 1023) << 52);
-              val = fma((double)Tl[i], s63, (double)H[i] * s42);
-            } else {
-              val = scalbn(fma((double)Tl[i], 0x1p-21, (double)H[i]), k - 42);
-            }
-          }
-          double &dst = T.mode == 1 ? cbase[obase + col] : cbase[T.c_off + (int64_t)row * T.ldc + col];
-          dst = T.accum ? dst + val : val;
-        }
-      }
-    }
-  }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0 && !(aborted & 2)) tc::tmem_dealloc(tmem, OZ_TMEM_COLS);
+  const int aborted = abort_flag;
+  if (warp == 0 && !(aborted & 2)) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc(tmem, OZ_TMEM_COLS);
+  }
+}
+
+// Sums the partial results of the tasks in K chunks, in the order of K; a warp
+// per output row, memory bound (8 bytes read per output and chunk).
+constexpr int OZ_SUM_ROWS = 8;
+__global__ void __launch_bounds__(32 * OZ_SUM_ROWS) oz_sum_kernel(const int *__restrict__ ids,
+                                                                  const TcTask *__restrict__ tasks,
+                                                                  double *const *__restrict__ bufs,
+                                                                  const int *__restrict__ active) {
+  const TcTask T = tasks[ids[blockIdx.x]];
+  const int row = blockIdx.y * OZ_SUM_ROWS + (threadIdx.x >> 5);
+  if (row >= T.M || (active && !active[T.sb])) return;
+  const double *part = bufs[T.sb * NBUF + T.part_buf] + T.part_off + (int64_t)row * T.N;
+  double *out = bufs[T.sb * NBUF + T.c_buf] +
+                (T.mode == 1 ? ((const int64_t *)bufs[T.sb * NBUF + T.rmap_buf])[T.rmap_off + row]
+                             : T.c_off + (int64_t)row * T.ldc);
+  for (int col = threadIdx.x & 31; col < T.N; col += 32) {
+    double x = T.accum ? out[col] + part[col] : part[col];
+    for (int c = 1; c < T.nch; ++c) x += part[(int64_t)c * T.M * T.N + col];
+    out[col] = x;
+  }
+}
+
+// streaming multiprocessors of the current device (0: query failed)
+int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 0;
+    sms = n;
+  }
+  return sms;
 }
 
 }  // namespace
@@ -851,10 +998,21 @@ cudaError_t launch_wstage_oz(const WTaskP *tasks, int ntasks, int max_rows, cons
 
 cudaError_t launch_oz_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, cudaStream_t st) {
-  const int smem = OZ_STAGES * OZ_STAGE;
-  cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (ntiles <= 0) return cudaGetLastError();
+  const int sms = sm_count();
+  if (sms <= 0) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
   if (e != cudaSuccess) return e;
-  if (ntiles > 0) oz_gemm_kernel<<<ntiles, 128, smem, st>>>(tiles, tasks, bufs, active, err);
+  oz_gemm_kernel<<<ntiles < sms ? ntiles : sms, OZ_THREADS, OZ_SMEM, st>>>(tiles, ntiles, tasks, bufs, active, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_oz_sum(const int *ids, int n, int max_rows, const TcTask *tasks, double *const *bufs,
+                          const int *active, cudaStream_t st) {
+  if (n > 0 && max_rows > 0) {
+    dim3 grid(n, (max_rows + OZ_SUM_ROWS - 1) / OZ_SUM_ROWS);
+    oz_sum_kernel<<<grid, 32 * OZ_SUM_ROWS, 0, st>>>(ids, tasks, bufs, active);
+  }
   return cudaGetLastError();
 }
 
@@ -888,13 +1046,8 @@ static cudaError_t launch_tc_gemm_tn(const TcTile *tiles, int ntiles, const TcTa
 cudaError_t launch_tc_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, int bf16, int tn, cudaStream_t st) {
   if (ntiles <= 0) return cudaGetLastError();
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess || sms <= 0) return e != cudaSuccess ? e : cudaErrorInvalidValue;
-  }
+  const int sms = sm_count();
+  if (sms <= 0) return cudaErrorInvalidValue;
   switch (tn) {
     case 64: return launch_tc_gemm_tn<64>(tiles, ntiles, tasks, bufs, active, err, bf16, sms, st);
     case 128: return launch_tc_gemm_tn<128>(tiles, ntiles, tasks, bufs, active, err, bf16, sms, st);
