@@ -45,7 +45,7 @@ enum BufId {
   BUF_OB3 = 28,   // stage 3 B digits
   BUF_ORMAP = 29, // stage 3 output row -> psi offset (int64)
   BUF_OEXP = 30,  // per packed row: exponent of the digit expansion (int32)
-  BUF_OT3 = 31,   // stage 3 A in FP64 (row-major per task) before its digits
+  BUF_OPART = 31, // stage 1: results of its K chunks
   BUF_GOZ = 32,   // digit arena of the other FP64 GEMM lists (environments,
                   // prediction, SVD Newton-Schulz), the same for every superblock
   BUF_GEXP = 33,  // exponents of that arena
@@ -80,6 +80,7 @@ struct GemmTile {
 struct WTerm {
   int64_t in_off;
   int in_ld;
+  int k0, cols;  // tensor-core W stage: packed K columns [k0, k0 + cols) it adds to
   int pad;
   double coef;
 };
@@ -277,17 +278,23 @@ struct PackSeg {
   int sb, src_buf, dst_buf, src_fp32;
   int whole;              // digit form: the segment holds the whole K range of its rows
   int exp_buf;            // digit form: slot of the exponent array
+  int kpad;               // digit form: zero columns to write after the segment
   double alpha;           // digit form: source values scaled by alpha
 };
-struct WTaskP {           // T3 rectangle written into a packed stage-3 A matrix
+struct WTaskP {           // rows of a packed stage-3 A matrix: one (left sector, s, t)
   int64_t dst_off;
-  int64_t exp_off;        // digit form: exponents of the task's packed rows
-  int row0, k0, KB, G;
-  int sb, rows, cols, term0, nterm;
-  int in_buf, dst_buf;    // stage-1 output read, packed A written
-  int t3_ld;              // digit form: T3 stored at t3_off, rows of t3_ld (the task's K)
-  int64_t t3_off;
+  int64_t exp_off;        // digit form: exponents of the matrix's packed rows
+  int row0, rows, KB, G;
+  int sb, in_buf, dst_buf;  // stage-1 output read, packed A written
+  int pad;                  // (48 bytes: copied in 16-byte pieces)
 };
+struct WUnit {            // W stage work unit: W_ROWS rows x W_K packed K columns
+  int task, r0;           // rows r0 .. of the task
+  int k0;                 // first packed K column (a multiple of W_K)
+  int term0, nterm;       // the terms that reach into the window, in order
+  int slot;               // digit form: where pass 0 keeps the window's sums for pass 1 (-1: formed again)
+};
+constexpr int W_ROWS = 32, W_K = 64;
 struct TcTask {
   int64_t a_off, b_off, c_off, rmap_off;
   int64_t a_exp, b_exp;   // digit form: exponent arrays of the A rows and B rows
@@ -308,9 +315,7 @@ constexpr int MIX_NTN = 3;
 constexpr int MIX_TNS[MIX_NTN] = {64, 128, 256};
 cudaError_t launch_pack(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
                         int bf16, cudaStream_t st);
-// W stage work units: units[k] = (task, first row, K window): 32 rows of the
-// task's rectangle and the packed K columns [64 w, 64 w + 64) it overlaps
-cudaError_t launch_wstage_tc(const int4 *units, int nunits, const WTaskP *tasks, const WTerm *terms,
+cudaError_t launch_wstage_tc(const WUnit *units, int nunits, const WTaskP *tasks, const WTerm *terms,
                              double *const *bufs, const int *active, int bf16, cudaStream_t st);
 cudaError_t launch_tc_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, int bf16, int tn, cudaStream_t st);
@@ -322,12 +327,15 @@ constexpr int OZ_PLANES = 8;
 constexpr int OZ_KBLK = 16;
 constexpr int OZ_MAX_K = 768;
 constexpr int OZ_EXP_EMPTY = (int)0x80808080;  // byte-fill value: row without non-zeros
-cudaError_t launch_oz_exp(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+// units[k] = (segment, first row): PACK_ROWS rows of a segment
+constexpr int PACK_ROWS = 32;
+cudaError_t launch_oz_exp(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                           cudaStream_t st);
-cudaError_t launch_oz_pack(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+cudaError_t launch_oz_pack(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                            cudaStream_t st);
-cudaError_t launch_wstage_oz(const WTaskP *tasks, int ntasks, int max_rows, const WTerm *terms,
-                             double *const *bufs, const int *active, int pass, cudaStream_t st);
+// pass 0: exponents, pass 1: digits
+cudaError_t launch_wstage_oz(const WUnit *units, int nunits, const WTaskP *tasks, const WTerm *terms,
+                             double *const *bufs, double *keep, const int *active, int pass, cudaStream_t st);
 cudaError_t launch_oz_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks, double *const *bufs,
                            const int *active, int *err, cudaStream_t st);
 // ids: the n tasks with several K chunks

@@ -85,6 +85,19 @@ uint64_t sm64_at(uint64_t s, uint64_t k) { return sm64_mix(s + (k + 1ull) * 0x9E
 // task's op(A) (M x K) and op(B)^T (N x K), K concatenated over its segments,
 // become digit planes in the context's digit arena, one exponent per packed
 // row.
+struct OzPacks {                  // segments to pack and their work units
+  std::vector<PackSeg> segs;
+  std::vector<int2> units;        // (segment, first row)
+  DevBuf dsegs, dunits;
+  void clear() {
+    segs.clear();
+    units.clear();
+  }
+  void add(const PackSeg &s) {
+    for (int r = 0; r < s.rows; r += PACK_ROWS) units.push_back(make_int2((int)segs.size(), r));
+    segs.push_back(s);
+  }
+};
 struct OzTiles {                  // a digit-slice GEMM's output tiles
   std::vector<TcTile> tiles;
   std::vector<int> sums;          // tasks in several K chunks
@@ -98,12 +111,11 @@ struct OzTiles {                  // a digit-slice GEMM's output tiles
 };
 struct OzList {
   bool ok = false;
-  std::vector<PackSeg> segs;      // A and B packing, one per GEMM segment and operand
-  int seg_rows = 0;
+  OzPacks pack;                   // A and B packing, one per GEMM segment and operand
   std::vector<TcTask> tasks;
   OzTiles out;
   int64_t planes = 0, nexp = 0;   // arena use: BF16 elements, exponents
-  DevBuf dsegs, dtasks;
+  DevBuf dtasks;
 };
 
 // Device side of one grouped FP64 GEMM list: its tiles, or its digit-slice form.
@@ -245,7 +257,7 @@ struct idmrg_ctx {
   std::vector<TcTile> tc1t[MIX_NTN], tc3t[MIX_NTN];
   std::vector<WTaskP> wtp;
   std::vector<WTerm> wtpm;
-  std::vector<int4> wunits;  // W stage work units (task, first row, rows)
+  std::vector<WUnit> wunits;
   DevBuf dwunits;
   struct TcTune {
     int choice = -1;
@@ -263,7 +275,7 @@ struct idmrg_ctx {
   double inner_factor = 1e-3;
   int inner_cap = 80;
 
-  int pk_L_rows = 0, pk_psi_rows = 0, pk_R_rows = 0, wtp_rows = 0;
+  int pk_L_rows = 0, pk_psi_rows = 0, pk_R_rows = 0;
   DevBuf dpkL, dpkp[MIX_NTN], dpkR[MIX_NTN], dtc1k[MIX_NTN], dtc1t[MIX_NTN], dtc3k[MIX_NTN], dtc3t[MIX_NTN];
   DevBuf dwtp, dwtpm, dtarget, dtune_out;
   std::vector<DevBuf> bPA1, bPB1, bT1F, bPA3, bPB3, bRMAP;
@@ -271,16 +283,17 @@ struct idmrg_ctx {
   // FP64 matvecs that start every mixed-precision Lanczos restart); usable
   // while every task's K fits the exactness bound
   bool oz_ok = false;
-  std::vector<PackSeg> oz_step_w, oz_step_p, oz_psi;  // whole-K (L), part-K (R), psi
+  OzPacks oz_step_w, oz_step_p, oz_psi;  // whole-K (L), part-K (R), psi
   std::vector<TcTask> oz1k, oz3k;
   OzTiles oz1t, oz3t;
   std::vector<WTaskP> ozw;
-  int oz_step_w_rows = 0, oz_step_p_rows = 0, oz_psi_rows = 0, ozw_rows = 0;
+  std::vector<WUnit> ozwu;
+  int ozw_keep = 0;  // windows whose sums pass 0 of the W stage keeps
   int64_t oz_a3_lo = 0, oz_a3_hi = 0, oz_b3_lo = 0, oz_b3_hi = 0;  // exponent ranges reset before use
   std::vector<WTerm> wtpm_oz;
   DevBuf goz_planes, goz_exps, goz_part;  // digit arena of the FP64 GEMM lists (BUF_GOZ, BUF_GEXP, BUF_GPART)
-  DevBuf dozsw, dozsp, dozp, doz1k, doz3k, dozw, dozwm, oexp;
-  std::vector<DevBuf> bOA1, bOB1, bOT1, bOA3, bOB3, bORMAP, bOT3;
+  DevBuf doz1k, doz3k, dozw, dozwu, dozwm, dozkeep, oexp;
+  std::vector<DevBuf> bOA1, bOB1, bOT1, bOA3, bOB3, bORMAP, bOPART;
 
   // plan for iteration n
   std::vector<SBPlan> plan;
@@ -475,6 +488,29 @@ namespace {
     if (!(ok)) return c->fail(IDMRG_ENOMEM, "device allocation failed (%s)", #ok); \
   } while (0)
 
+// Rectangles of one row block of a packed stage-3 A matrix, in K order: packed
+// columns [k0, k0 + cols) and the terms of each (consecutive in the term list).
+struct WRect {
+  int k0, cols, term0, nterm;
+};
+// W stage units of row block `task`: a window of W_ROWS rows x W_K columns
+// wherever a rectangle has terms.  keep (digit form): counts the windows whose
+// sums pass 0 keeps, those that hold a rectangle of more than one term.
+void w_units(std::vector<WUnit> &units, int task, int rows, const std::vector<WRect> &rects, int *keep = nullptr) {
+  for (int r0 = 0; r0 < rows; r0 += W_ROWS) {
+    size_t lo = 0;
+    for (int k0 = 0; lo < rects.size(); k0 += W_K) {
+      while (lo < rects.size() && rects[lo].k0 + rects[lo].cols <= k0) ++lo;
+      size_t hi = lo;
+      while (hi < rects.size() && rects[hi].k0 < k0 + W_K) ++hi;
+      if (hi == lo) continue;
+      const int t0 = rects[lo].term0;
+      const int nterm = rects[hi - 1].term0 + rects[hi - 1].nterm - t0;
+      units.push_back(WUnit{task, r0, k0, t0, nterm, keep && nterm > (int)(hi - lo) ? (*keep)++ : -1});
+    }
+  }
+}
+
 // Adds a digit-slice task and its output tiles: one per K chunk of OZ_MAX_K,
 // whose results take M N nch doubles at part_n of part_buf when there are
 // several.
@@ -521,10 +557,9 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
   auto cdiv = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
   const int64_t TA = (int64_t)128 * OZ_KBLK * OZ_PLANES, TB = (int64_t)TC_TN * OZ_KBLK * OZ_PLANES;
   Z.ok = false;
-  Z.segs.clear();
+  Z.pack.clear();
   Z.tasks.clear();
   Z.out.clear();
-  Z.seg_rows = 0;
   int64_t an = 0, bn = 0, en = 0, part = 0;
   // A planes first, B planes after all of them: B offsets are patched below
   std::vector<size_t> bseg;
@@ -540,7 +575,7 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
     bn += (int64_t)NT * KB * TB;
     en += t.M + t.N;
     const int whole = t.nseg == 1 ? 1 : 0;
-    int k0 = 0;
+    int k0 = 0;  // the last segment of a row also writes the zeros up to the end of its K block
     for (int q = t.seg0; q < t.seg0 + t.nseg; ++q) {
       const GemmSeg &g = L.segs[q];
       if (g.K <= 0) continue;
@@ -561,6 +596,7 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
       a.dst_buf = BUF_GOZ;
       a.whole = whole;
       a.exp_buf = BUF_GEXP;
+      a.kpad = k0 + g.K == K ? KB * OZ_KBLK - (int)K : 0;
       a.alpha = g.alpha;
       PackSeg b = a;
       b.dst_off = pb;
@@ -572,10 +608,9 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
       b.G = TC_TN / 8;
       b.src_buf = g.b_buf;
       b.alpha = 1.0;
-      Z.segs.push_back(a);
-      bseg.push_back(Z.segs.size());
-      Z.segs.push_back(b);
-      Z.seg_rows = std::max(Z.seg_rows, std::max(t.M, t.N));
+      Z.pack.add(a);
+      bseg.push_back(Z.pack.segs.size());
+      Z.pack.add(b);
       k0 += g.K;
     }
     TcTask u{};
@@ -599,7 +634,7 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
     pmt.push_back(MT);
     pnt.push_back(NT);
   }
-  for (size_t i : bseg) Z.segs[i].dst_off += an;
+  for (size_t i : bseg) Z.pack.segs[i].dst_off += an;
   for (size_t i = 0; i < pend.size(); ++i) {
     pend[i].b_off += an;
     oz_add_task(Z.out, Z.tasks, pend[i], pmt[i], pnt[i], BUF_GPART, part);
@@ -618,7 +653,7 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
     }
     NOMEM(sync_bufs(c) == IDMRG_OK);
   }
-  NOMEM(c->upload(Z.dsegs, Z.segs) && c->upload(Z.dtasks, Z.tasks));
+  NOMEM(c->upload(Z.pack.dsegs, Z.pack.segs) && c->upload(Z.pack.dunits, Z.pack.units) && c->upload(Z.dtasks, Z.tasks));
   {
     idmrg_status s = oz_upload(c, Z.out, Z.tasks);
     if (s != IDMRG_OK) return s;
@@ -629,10 +664,12 @@ idmrg_status oz_build(idmrg_ctx *c, const GemmList &L, OzList &Z) {
 
 idmrg_status oz_run(idmrg_ctx *c, OzList &Z) {
   double *const *bufs = (double *const *)c->dbufs.p;
-  CK(cudaMemsetAsync(c->goz_planes.p, 0, 2 * (size_t)Z.planes, c->st));
+  // rows past a task's M or N stay as they are: they only reach outputs that
+  // are not stored
   CK(cudaMemsetAsync(c->goz_exps.p, 0x80, 4 * (size_t)Z.nexp, c->st));
-  CK(launch_oz_exp((const PackSeg *)Z.dsegs.p, (int)Z.segs.size(), Z.seg_rows, bufs, nullptr, c->st));
-  CK(launch_oz_pack((const PackSeg *)Z.dsegs.p, (int)Z.segs.size(), Z.seg_rows, bufs, nullptr, c->st));
+  const int2 *units = (const int2 *)Z.pack.dunits.p;
+  CK(launch_oz_exp(units, (int)Z.pack.units.size(), (const PackSeg *)Z.pack.dsegs.p, bufs, nullptr, c->st));
+  CK(launch_oz_pack(units, (int)Z.pack.units.size(), (const PackSeg *)Z.pack.dsegs.p, bufs, nullptr, c->st));
   c->launches += 2;
   return oz_launch(c, Z.out, Z.dtasks, nullptr);
 }
@@ -970,7 +1007,8 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
   }
   c->wtp.clear();
   c->wtpm.clear();
-  c->pk_L_rows = c->pk_psi_rows = c->pk_R_rows = c->wtp_rows = 0;
+  c->wunits.clear();
+  c->pk_L_rows = c->pk_psi_rows = c->pk_R_rows = 0;
   double work1 = 0.0, work3 = 0.0;
   int64_t max_psi = 1;
   auto seg = [&](std::vector<PackSeg> &v, int &mr, int sb, int dst_buf, int64_t dst_off, int src_buf,
@@ -1107,21 +1145,20 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
           for (int t = 0; t < d; ++t) {
             const int k = psi.sub(i, s, t);
             if (rows_of[k] < 0) continue;
+            WTaskP w{};
+            w.dst_off = pa3[jo];
+            w.row0 = rows_of[k];
+            w.rows = BL.dim[i];
+            w.KB = KB;
+            w.G = GA;
+            w.sb = p;
+            w.in_buf = BUF_T1F;
+            w.dst_buf = BUF_PA3;
+            std::vector<WRect> rects;
             for (int cc = 0; cc < wc; ++cc) {
               if (ks[cc] < 0) continue;
               const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
-              WTaskP w{};
-              w.dst_off = pa3[jo];
-              w.row0 = rows_of[k];
-              w.k0 = ks[cc];
-              w.KB = KB;
-              w.G = GA;
-              w.sb = p;
-              w.rows = BL.dim[i];
-              w.cols = BR.dim[jin];
-              w.in_buf = BUF_T1F;
-              w.dst_buf = BUF_PA3;
-              w.term0 = (int)c->wtpm.size();
+              const int term0 = (int)c->wtpm.size();
               for (int a = 0; a < wa; ++a) {
                 const int si = BL.find(BL.q[i] - L.lay.chq[a]);
                 if (si < 0 || L.lay.so[a * SL + si] != i || rs1[si][a] < 0) continue;
@@ -1134,15 +1171,18 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
                     WTerm term{};
                     term.in_off = t1f[si] + (int64_t)rs1[si][a] * psi.C[si] + psi.scol[k2];
                     term.in_ld = psi.C[si];
+                    term.k0 = ks[cc];
+                    term.cols = BR.dim[jin];
                     term.coef = cf;
                     c->wtpm.push_back(term);
                   }
               }
-              w.nterm = (int)c->wtpm.size() - w.term0;
-              if (w.nterm == 0) continue;  // the packed rectangle stays zero
-              c->wtp.push_back(w);
-              c->wtp_rows = std::max(c->wtp_rows, w.rows);
+              const int nterm = (int)c->wtpm.size() - term0;  // without terms the packed rectangle stays zero
+              if (nterm > 0) rects.push_back(WRect{ks[cc], BR.dim[jin], term0, nterm});
             }
+            if (rects.empty()) continue;
+            w_units(c->wunits, (int)c->wtp.size(), w.rows, rects);
+            c->wtp.push_back(w);
           }
       for (int k = 0; k < MIX_NTN; ++k) {
         const int NT = (int)cdiv(N, MIX_TNS[k]);
@@ -1185,13 +1225,6 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
     c->hbufs[p * NBUF + BUF_PA3] = c->dp(c->bPA3[p]);
     c->hbufs[p * NBUF + BUF_PB3] = c->dp(c->bPB3[p]);
     c->hbufs[p * NBUF + BUF_RMAP] = c->dp(c->bRMAP[p]);
-  }
-  // W stage units: windows of 32 rows x 64 packed K columns of each rectangle
-  c->wunits.clear();
-  for (size_t k = 0; k < c->wtp.size(); ++k) {
-    const WTaskP &w = c->wtp[k];
-    for (int r0 = 0; r0 < w.rows; r0 += 32)
-      for (int kw = w.k0 / 64; kw <= (w.k0 + w.cols - 1) / 64; ++kw) c->wunits.push_back(make_int4((int)k, r0, kw, 0));
   }
   NOMEM(c->upload(c->dwunits, c->wunits));
   NOMEM(c->upload(c->dpkL, c->pk_L) && c->upload(c->dwtp, c->wtp) && c->upload(c->dwtpm, c->wtpm));
@@ -1244,10 +1277,10 @@ idmrg_status plan_oz(idmrg_ctx *c) {
   c->oz3t.clear();
   c->ozw.clear();
   c->wtpm_oz.clear();
-  c->oz_step_w_rows = c->oz_step_p_rows = c->oz_psi_rows = c->ozw_rows = 0;
-  auto seg = [&](std::vector<PackSeg> &v, int &mr, int sb, int dst_buf, int64_t dst_off, int src_buf,
-                 int64_t src_off, int64_t exp_off, int row0, int k0, int rows, int ks, int ld, int trans, int KB,
-                 int G, int whole) {
+  c->ozwu.clear();
+  c->ozw_keep = 0;
+  auto seg = [&](OzPacks &v, int sb, int dst_buf, int64_t dst_off, int src_buf, int64_t src_off, int64_t exp_off,
+                 int row0, int k0, int rows, int ks, int ld, int trans, int KB, int G, int whole, int kpad) {
     if (rows <= 0 || ks <= 0) return;
     PackSeg q{};
     q.dst_off = dst_off;
@@ -1266,15 +1299,15 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     q.dst_buf = dst_buf;
     q.whole = whole;
     q.exp_buf = BUF_OEXP;
+    q.kpad = kpad;
     q.alpha = 1.0;
-    v.push_back(q);
-    mr = std::max(mr, rows);
+    v.add(q);
   };
   int64_t ex1 = 0, exb3 = 0, exa3 = 0;  // the three exponent ranges, relative
   const size_t b3seg0 = 0;
   std::vector<size_t> a3_tasks, b3_tasks;  // tasks / items whose offsets get the range bases
   std::vector<std::vector<int64_t>> rmaps(P);
-  std::vector<int64_t> na1(P), nb1(P), nt1(P), na3(P), nb3(P), nt3(P);
+  std::vector<int64_t> na1(P), nb1(P), nt1(P), na3(P), nb3(P), npart(P);
   for (int p = 0; p < P; ++p) {
     if (!c->owns(p)) continue;
     SBPlan &S = c->plan[p];
@@ -1288,7 +1321,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     std::vector<int64_t> t1f(SL, -1);
     std::vector<std::vector<int>> rs1(SL, std::vector<int>(wa, -1));
     int64_t pa1n = 0, pb1n = 0, t1n = 0;
-    int64_t np1 = 0, np3 = 0;  // results of K chunks: stage 1's in T3's place, stage 3's in T1's
+    int64_t np1 = 0, np3 = 0;  // results of K chunks: stage 3's take T1's place
     for (int si = 0; si < SL; ++si) {
       if (psi.C[si] == 0) continue;
       int M = 0;
@@ -1310,10 +1343,10 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       for (int a = 0; a < wa; ++a) {
         if (rs1[si][a] < 0) continue;
         const int so = L.lay.so[a * SL + si];
-        seg(c->oz_step_w, c->oz_step_w_rows, p, BUF_OA1, pa, BUF_L, L.lay.off[a * SL + si], ea, rs1[si][a], 0,
-            BL.dim[so], K, K, 0, KB, GA, 1);
+        seg(c->oz_step_w, p, BUF_OA1, pa, BUF_L, L.lay.off[a * SL + si], ea, rs1[si][a], 0, BL.dim[so], K, K, 0, KB,
+            GA, 1, KB * OZ_KBLK - K);
       }
-      seg(c->oz_psi, c->oz_psi_rows, p, BUF_OB1, pb, BUF_IN, psi.roff[si], eb, 0, 0, N, K, N, 1, KB, GB, 1);
+      seg(c->oz_psi, p, BUF_OB1, pb, BUF_IN, psi.roff[si], eb, 0, 0, N, K, N, 1, KB, GB, 1, KB * OZ_KBLK - K);
       TcTask t{};
       t.a_off = pa;
       t.b_off = pb;
@@ -1330,10 +1363,10 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       t.exp_buf = BUF_OEXP;
       t.mode = 2;
       t.ldc = N;
-      oz_add_task(c->oz1t, c->oz1k, t, MT, NT, BUF_OT3, np1);
+      oz_add_task(c->oz1t, c->oz1k, t, MT, NT, BUF_OPART, np1);
     }
     // ---------------- stage 3
-    int64_t pa3n = 0, pb3n = 0, nt3s = 0;
+    int64_t pa3n = 0, pb3n = 0;
     std::vector<int64_t> &rmap = rmaps[p];
     for (int jo = 0; jo < SR; ++jo) {
       std::vector<int> ks(wc, -1);
@@ -1360,8 +1393,6 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       const int N = BR.dim[jo];
       const int KB = (int)cdiv(std::max(K, 1), OZ_KBLK), MT = (int)cdiv(M, 128), NT = (int)cdiv(N, TC_TN);
       const int64_t pa = pa3n, pb = pb3n, ea = exa3, eb = exb3;
-      const int64_t t3n = nt3s;
-      nt3s += (int64_t)M * K;
       pa3n += (int64_t)MT * KB * TA;
       pb3n += (int64_t)NT * KB * TB;
       exa3 += M;
@@ -1369,32 +1400,30 @@ idmrg_status plan_oz(idmrg_ctx *c) {
       for (int cc = 0; cc < wc; ++cc) {
         if (ks[cc] < 0) continue;
         const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
-        seg(c->oz_step_p, c->oz_step_p_rows, p, BUF_OB3, pb, BUF_R, R.lay.off[cc * SR + jin], eb, 0, ks[cc], N,
-            BR.dim[jin], BR.dim[jin], 0, KB, GB, 0);
+        const int kp = ks[cc] + BR.dim[jin] == K ? KB * OZ_KBLK - K : 0;  // after the last channel: zeros
+        seg(c->oz_step_p, p, BUF_OB3, pb, BUF_R, R.lay.off[cc * SR + jin], eb, 0, ks[cc], N, BR.dim[jin], BR.dim[jin],
+            0, KB, GB, 0, kp);
       }
       for (int i = 0; i < SL; ++i)
         for (int s = 0; s < d; ++s)
           for (int t = 0; t < d; ++t) {
             const int k = psi.sub(i, s, t);
             if (rows_of[k] < 0) continue;
+            WTaskP w{};
+            w.dst_off = pa;
+            w.exp_off = ea;
+            w.row0 = rows_of[k];
+            w.rows = BL.dim[i];
+            w.KB = KB;
+            w.G = GA;
+            w.sb = p;
+            w.in_buf = BUF_OT1;
+            w.dst_buf = BUF_OA3;
+            std::vector<WRect> rects;
             for (int cc = 0; cc < wc; ++cc) {
               if (ks[cc] < 0) continue;
               const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
-              WTaskP w{};
-              w.dst_off = pa;
-              w.exp_off = ea;
-              w.row0 = rows_of[k];
-              w.k0 = ks[cc];
-              w.KB = KB;
-              w.G = GA;
-              w.sb = p;
-              w.rows = BL.dim[i];
-              w.cols = BR.dim[jin];
-              w.in_buf = BUF_OT1;
-              w.dst_buf = BUF_OA3;
-              w.t3_off = t3n;
-              w.t3_ld = K;
-              w.term0 = (int)c->wtpm_oz.size();
+              const int term0 = (int)c->wtpm_oz.size();
               for (int a = 0; a < wa; ++a) {
                 const int si = BL.find(BL.q[i] - L.lay.chq[a]);
                 if (si < 0 || L.lay.so[a * SL + si] != i || rs1[si][a] < 0) continue;
@@ -1407,15 +1436,18 @@ idmrg_status plan_oz(idmrg_ctx *c) {
                     WTerm term{};
                     term.in_off = t1f[si] + (int64_t)rs1[si][a] * psi.C[si] + psi.scol[k2];
                     term.in_ld = psi.C[si];
+                    term.k0 = ks[cc];
+                    term.cols = BR.dim[jin];
                     term.coef = cf;
                     c->wtpm_oz.push_back(term);
                   }
               }
-              w.nterm = (int)c->wtpm_oz.size() - w.term0;
-              if (w.nterm == 0) continue;
-              c->ozw.push_back(w);
-              c->ozw_rows = std::max(c->ozw_rows, w.rows);
+              const int nterm = (int)c->wtpm_oz.size() - term0;  // without terms the packed rectangle stays zero
+              if (nterm > 0) rects.push_back(WRect{ks[cc], BR.dim[jin], term0, nterm});
             }
+            if (rects.empty()) continue;
+            w_units(c->ozwu, (int)c->ozw.size(), w.rows, rects, &c->ozw_keep);
+            c->ozw.push_back(w);
           }
       TcTask t{};
       t.a_off = pa;
@@ -1440,7 +1472,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     nt1[p] = std::max(t1n, np3);
     na3[p] = pa3n;
     nb3[p] = pb3n;
-    nt3[p] = std::max(nt3s, np1);
+    npart[p] = np1;
   }
   (void)b3seg0;
   (void)target;
@@ -1449,7 +1481,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
   c->oz_b3_hi = ex1 + exb3;
   c->oz_a3_lo = c->oz_b3_hi;
   c->oz_a3_hi = c->oz_a3_lo + exa3;
-  for (PackSeg &q : c->oz_step_p) q.exp_off += c->oz_b3_lo;
+  for (PackSeg &q : c->oz_step_p.segs) q.exp_off += c->oz_b3_lo;
   for (WTaskP &w : c->ozw) w.exp_off += c->oz_a3_lo;
   for (TcTask &t : c->oz3k) {
     t.a_exp += c->oz_a3_lo;
@@ -1462,12 +1494,12 @@ idmrg_status plan_oz(idmrg_ctx *c) {
           c->ensure(c->bOT1[p], 8 * std::max<int64_t>(nt1[p], 1)) &&
           c->ensure(c->bOA3[p], 2 * std::max<int64_t>(na3[p], 8)) &&
           c->ensure(c->bOB3[p], 2 * std::max<int64_t>(nb3[p], 8)) &&
-          c->ensure(c->bOT3[p], 8 * std::max<int64_t>(nt3[p], 1)) && c->upload(c->bORMAP[p], rmaps[p]));
-    // zero digits in the padding (only real elements are rewritten later)
-    CK(cudaMemsetAsync(c->bOA1[p].p, 0, 2 * na1[p], c->st));
-    CK(cudaMemsetAsync(c->bOB1[p].p, 0, 2 * nb1[p], c->st));
+          c->ensure(c->bOPART[p], 8 * std::max<int64_t>(npart[p], 1)) && c->upload(c->bORMAP[p], rmaps[p]));
+    // zero digits where the W stage has no term, and in the K padding (only
+    // real elements are rewritten later); the other operands' K padding is
+    // written with their last segment, and rows past M or N only reach outputs
+    // that are not stored
     CK(cudaMemsetAsync(c->bOA3[p].p, 0, 2 * na3[p], c->st));
-    CK(cudaMemsetAsync(c->bOB3[p].p, 0, 2 * nb3[p], c->st));
     c->hbufs[p * NBUF + BUF_OA1] = c->dp(c->bOA1[p]);
     c->hbufs[p * NBUF + BUF_OB1] = c->dp(c->bOB1[p]);
     c->hbufs[p * NBUF + BUF_OT1] = c->dp(c->bOT1[p]);
@@ -1475,9 +1507,11 @@ idmrg_status plan_oz(idmrg_ctx *c) {
     c->hbufs[p * NBUF + BUF_OB3] = c->dp(c->bOB3[p]);
     c->hbufs[p * NBUF + BUF_ORMAP] = c->dp(c->bORMAP[p]);
     c->hbufs[p * NBUF + BUF_OEXP] = c->dp(c->oexp);
-    c->hbufs[p * NBUF + BUF_OT3] = c->dp(c->bOT3[p]);
+    c->hbufs[p * NBUF + BUF_OPART] = c->dp(c->bOPART[p]);
   }
-  NOMEM(c->upload(c->dozsw, c->oz_step_w) && c->upload(c->dozsp, c->oz_step_p) && c->upload(c->dozp, c->oz_psi) &&
+  for (OzPacks *k : {&c->oz_step_w, &c->oz_step_p, &c->oz_psi})
+    NOMEM(c->upload(k->dsegs, k->segs) && c->upload(k->dunits, k->units));
+  NOMEM(c->upload(c->dozwu, c->ozwu) && c->ensure(c->dozkeep, 8 * (size_t)(W_ROWS * W_K) * std::max(c->ozw_keep, 1)) &&
         c->upload(c->doz1k, c->oz1k) && c->upload(c->doz3k, c->oz3k) && c->upload(c->dozw, c->ozw) &&
         c->upload(c->dozwm, c->wtpm_oz));
   for (auto [Z, k] : {std::make_pair(&c->oz1t, &c->oz1k), std::make_pair(&c->oz3t, &c->oz3k)}) {
@@ -1490,9 +1524,13 @@ idmrg_status plan_oz(idmrg_ctx *c) {
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
   CK(cudaMemsetAsync((int *)c->oexp.p + c->oz_b3_lo, 0x80, 4 * (c->oz_b3_hi - c->oz_b3_lo), c->st));
   double *const *bufs = (double *const *)c->dbufs.p;
-  CK(launch_oz_exp((const PackSeg *)c->dozsp.p, (int)c->oz_step_p.size(), c->oz_step_p_rows, bufs, nullptr, c->st));
-  CK(launch_oz_pack((const PackSeg *)c->dozsp.p, (int)c->oz_step_p.size(), c->oz_step_p_rows, bufs, nullptr, c->st));
-  CK(launch_oz_pack((const PackSeg *)c->dozsw.p, (int)c->oz_step_w.size(), c->oz_step_w_rows, bufs, nullptr, c->st));
+  auto pack = [&](const OzPacks &k, bool exps) {
+    return (exps ? launch_oz_exp : launch_oz_pack)((const int2 *)k.dunits.p, (int)k.units.size(),
+                                                   (const PackSeg *)k.dsegs.p, bufs, nullptr, c->st);
+  };
+  CK(pack(c->oz_step_p, true));
+  CK(pack(c->oz_step_p, false));
+  CK(pack(c->oz_step_w, false));
   c->kend(IDMRG_K_HEFF_WSTAGE);
   c->launches += 3;
   c->oz_ok = true;
@@ -1506,7 +1544,8 @@ idmrg_status heff_launch_oz(idmrg_ctx *c, const int *active_dev, const int *act)
   for (int q = 0; q < c->P; ++q)
     if (!act || act[q]) { gf += c->plan[q].gemm_flops; wf += c->plan[q].w_flops; by += c->plan[q].heff_bytes; }
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
-  CK(launch_oz_pack((const PackSeg *)c->dozp.p, (int)c->oz_psi.size(), c->oz_psi_rows, bufs, active_dev, c->st));
+  CK(launch_oz_pack((const int2 *)c->oz_psi.dunits.p, (int)c->oz_psi.units.size(),
+                    (const PackSeg *)c->oz_psi.dsegs.p, bufs, active_dev, c->st));
   c->kend(IDMRG_K_HEFF_WSTAGE);
   // booked as the restart matvecs of a mixed context, as the H_eff GEMMs of FP64_TC
   const int kg = c->mixed ? IDMRG_K_HEFF_F64 : IDMRG_K_HEFF_GEMM;
@@ -1518,10 +1557,9 @@ idmrg_status heff_launch_oz(idmrg_ctx *c, const int *active_dev, const int *act)
   c->kend(kg);
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
   CK(cudaMemsetAsync((int *)c->oexp.p + c->oz_a3_lo, 0x80, 4 * (c->oz_a3_hi - c->oz_a3_lo), c->st));
-  CK(launch_wstage_oz((const WTaskP *)c->dozw.p, (int)c->ozw.size(), c->ozw_rows, (const WTerm *)c->dozwm.p, bufs,
-                      active_dev, 0, c->st));
-  CK(launch_wstage_oz((const WTaskP *)c->dozw.p, (int)c->ozw.size(), c->ozw_rows, (const WTerm *)c->dozwm.p, bufs,
-                      active_dev, 1, c->st));
+  for (int pass = 0; pass < 2; ++pass)
+    CK(launch_wstage_oz((const WUnit *)c->dozwu.p, (int)c->ozwu.size(), (const WTaskP *)c->dozw.p,
+                        (const WTerm *)c->dozwm.p, bufs, c->dp(c->dozkeep), active_dev, pass, c->st));
   c->kend(IDMRG_K_HEFF_WSTAGE, wf, 0.0);
   c->kbegin(kg);
   {
@@ -1560,7 +1598,7 @@ idmrg_status heff_launch_mixed(idmrg_ctx *c, const int *active_dev, const int *a
                     active_dev, (int *)c->derr.p, c->bf16, MIX_TNS[k1], c->st));
   c->kend(IDMRG_K_HEFF_GEMM);
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
-  CK(launch_wstage_tc((const int4 *)c->dwunits.p, (int)c->wunits.size(), (const WTaskP *)c->dwtp.p,
+  CK(launch_wstage_tc((const WUnit *)c->dwunits.p, (int)c->wunits.size(), (const WTaskP *)c->dwtp.p,
                       (const WTerm *)c->dwtpm.p, bufs, active_dev, c->bf16, c->st));
   c->kend(IDMRG_K_HEFF_WSTAGE, wf, wb);
   c->kbegin(IDMRG_K_HEFF_GEMM);
@@ -3536,7 +3574,7 @@ idmrg_status idmrg_create_batch(const idmrg_mpo *mpos, int nmpo, const int *m_pe
   c->bVT.resize(P);
   c->bStart.resize(P);
   for (auto *v : {&c->bPA1, &c->bPB1, &c->bT1F, &c->bPA3, &c->bPB3, &c->bRMAP, &c->bOA1, &c->bOB1, &c->bOT1,
-                  &c->bOA3, &c->bOB3, &c->bORMAP, &c->bOT3})
+                  &c->bOA3, &c->bOB3, &c->bORMAP, &c->bOPART})
     v->resize(P);
   c->hbufs.assign((size_t)P * NBUF, nullptr);
   if (!c->ensure(c->derr, 256)) return bail(IDMRG_ENOMEM);
@@ -3587,7 +3625,7 @@ void idmrg_destroy(idmrg_ctx *c) {
     for (auto &t : *v) { rel(t.U); rel(t.V); }
   for (auto *v : {&c->bT1, &c->bT3, &c->bX, &c->bY, &c->bV, &c->bW, &c->bPsi, &c->bUT, &c->bVT, &c->bStart, &c->bPA1,
                   &c->bPB1, &c->bT1F, &c->bPA3, &c->bPB3, &c->bRMAP, &c->bOA1, &c->bOB1, &c->bOT1, &c->bOA3,
-                  &c->bOB3, &c->bORMAP, &c->bOT3})
+                  &c->bOB3, &c->bORMAP, &c->bOPART})
     for (auto &b : *v) rel(b);
   for (DevBuf *b : {&c->dbufs, &c->dg1k, &c->dg1s, &c->dg3k, &c->dg3s, &c->dwt, &c->dwm, &c->ddt,
                     &c->ddp, &c->drb, &c->dgpk, &c->dgps, &c->dst, &c->dstab, &c->dge1k,
@@ -3597,7 +3635,8 @@ void idmrg_destroy(idmrg_ctx *c) {
                     &c->ssv, &c->sjob0, &c->snjob, &c->skpj, &c->sperm, &c->slam, &c->seps, &c->sepsb, &c->skept,
                     &c->scj, &c->slamk, &c->siw, &c->sorder, &c->sorderq, &c->dsgk, &c->dsgs,
                     &c->dswk, &c->dsws, &c->dsxk, &c->dsxs, &c->dpkL, &c->dtune_out, &c->dmsb,
-                    &c->dwtp, &c->dwtpm, &c->dwunits, &c->dtarget, &c->dozsw, &c->dozsp, &c->dozp,
+                    &c->dwtp, &c->dwtpm, &c->dwunits, &c->dtarget, &c->oz_step_w.dsegs, &c->oz_step_w.dunits, &c->oz_step_p.dsegs,
+                    &c->oz_step_p.dunits, &c->oz_psi.dsegs, &c->oz_psi.dunits, &c->dozwu, &c->dozkeep,
                     &c->doz1k,
                     &c->oz1t.dtiles, &c->oz1t.dsums, &c->doz3k, &c->oz3t.dtiles, &c->oz3t.dsums, &c->dozw, &c->dozwm, &c->oexp,
                     &c->goz_planes, &c->goz_part,
@@ -3625,7 +3664,8 @@ void idmrg_destroy(idmrg_ctx *c) {
   if (c->pin_act) cudaFreeHost(c->pin_act);
   for (GemmDev *t : {&c->gd_g1, &c->gd_g3, &c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX}) {
     rel(t->tiles);
-    rel(t->oz.dsegs);
+    rel(t->oz.pack.dsegs);
+    rel(t->oz.pack.dunits);
     rel(t->oz.dtasks);
     rel(t->oz.out.dtiles);
     rel(t->oz.out.dsums);

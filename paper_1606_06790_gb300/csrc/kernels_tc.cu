@@ -38,6 +38,19 @@ namespace idmrg {
 
 namespace {
 
+// streaming multiprocessors of the current device (0: query failed)
+int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 0;
+    sms = n;
+  }
+  return sms;
+}
+
 __device__ __forceinline__ float tf32_round(float x) {
   return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
@@ -99,146 +112,193 @@ __global__ void pack_kernel(const PackSeg *__restrict__ segs, double *const *__r
 }
 
 // T3 = sum W12 T1 into the packed stage-3 A operand.  The two-site MPO is
-// mostly pass-through (a T3 rectangle copies one T1 rectangle, or sums a
-// few), so the stage streams T1 in and T3 out.  A CTA takes a window of 32
-// rows and 64 packed K columns (aligned to 64) of one rectangle.  Phase 1:
+// mostly pass-through (T3 copies one T1 rectangle per channel; the completed
+// channel sums many), so the stage streams T1 in and T3 out.  A unit is 32 rows
+// and 64 packed K columns, across however many channels' rectangles these fall
+// into: the many small rectangles of the outer charge sectors share a window,
+// and the terms that reach into it are one run of the term list.  Phase 1:
 // warps read T1 rows with the lanes along K (coalesced) and accumulate the
-// terms.  Phase 2: through a shared-memory tile, each thread takes one row
-// and one 16-byte group of the packed layout (8 BF16 or 4 TF32 elements),
-// the lanes along the rows, so that a warp's hi (and lo) stores fill 512
-// contiguous bytes of a K block.  Groups cut by the rectangle's K edges
-// belong partly to the neighbouring rectangle and are written element by
-// element.
+// terms.  Phase 2: through a shared-memory tile, each thread takes one row and
+// one 16-byte group of the packed layout, the lanes along the rows, so that a
+// warp's stores fill 512 contiguous bytes; columns that no rectangle covers,
+// and the K padding inside the window, are zeros.
+// A window is a microsecond of work behind a chain of dependent loads (unit,
+// its terms, T1), which is what bounded one CTA per window; the CTAs are
+// persistent instead, and while one window is worked on the next one's terms
+// are on their way to shared memory and the one after that's unit to registers.
+// Measured (GB300, kagome cylinder at m = 1000, all superblocks, under a
+// profiler; before: a CTA per window of a single rectangle): 180 -> 171 us, two
+// thirds of the issue slots taken; the FP64 form's two passes 419 + 608 -> 338 +
+// 407 us.
+constexpr int W_BATCH = 64;  // terms in shared memory at a time
+
+struct __align__(16) WStage {  // the shared-memory part of one unit
+  WTaskP task;
+  WTerm term[W_BATCH];
+};
+static_assert(sizeof(WTerm) == 32 && sizeof(WTaskP) == 48, "copied in 16-byte pieces");
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Walks the units of this CTA (blockIdx.x, + gridDim.x, ...): body(u, S) for
+// each, S holding its task and first W_BATCH terms; every thread of the block
+// takes part, and body is free to use barriers.
+template <class Body>
+__device__ __forceinline__ void w_walk(const WUnit *__restrict__ units, int nunits, const WTaskP *__restrict__ tasks,
+                                       const WTerm *__restrict__ terms, WStage (&S)[2], Body body) {
+  auto fetch = [&](const WUnit &u, WStage &to) {
+    const int n = 2 * min(u.nterm, W_BATCH);
+    const char *t = reinterpret_cast<const char *>(terms + u.term0), *k = reinterpret_cast<const char *>(tasks + u.task);
+    if (threadIdx.x < n) cp_async16(reinterpret_cast<char *>(to.term) + 16 * threadIdx.x, t + 16 * threadIdx.x);
+    if (threadIdx.x >= 128 && threadIdx.x < 131)
+      cp_async16(reinterpret_cast<char *>(&to.task) + 16 * (threadIdx.x - 128), k + 16 * (threadIdx.x - 128));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int i = blockIdx.x, buf = 0;
+  if (i >= nunits) return;
+  WUnit u = units[i], next{};
+  if (i + gridDim.x < nunits) next = units[i + gridDim.x];
+  fetch(u, S[0]);
+  for (; i < nunits; i += gridDim.x, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this unit's terms are there; the other buffer is free
+    WUnit after{};
+    if (i + gridDim.x < nunits) fetch(next, S[buf ^ 1]);
+    if (i + 2 * gridDim.x < nunits) after = units[i + 2 * gridDim.x];
+    body(u, S[buf]);
+    u = next;
+    next = after;
+  }
+}
+
+// The window's sums: warp w holds rows w, w + 8, w + 16, w + 24, lane l the
+// columns l and l + 32.  Most elements have one term of coefficient 1, which is
+// copied (an FMA in FP64 holds its unit for 64 cycles); halves of the window
+// that a narrow rectangle does not reach issue nothing.
+template <class T>
+__device__ __forceinline__ void w_accumulate(const WUnit &u, const WTerm *__restrict__ terms, const T *in, int nr,
+                                             WTerm *st, T (&acc)[4][2]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = T(0);
+  const int nrow = (nr - warp + 7) >> 3;  // rows of this warp (may be <= 0)
+  int last = -1;  // first column of the last term's rectangle: terms of one rectangle are consecutive
+  for (int b = 0; b < u.nterm; b += W_BATCH) {
+    const int n = min(W_BATCH, u.nterm - b);
+    if (b > 0) {
+      __syncthreads();
+      const double *from = reinterpret_cast<const double *>(terms + u.term0 + b);
+      for (int j = threadIdx.x; j < 4 * n; j += blockDim.x) reinterpret_cast<double *>(st)[j] = from[j];
+      __syncthreads();
+    }
+    for (int q = 0; q < n; ++q) {
+      const WTerm w = st[q];
+      const int k = u.k0 - w.k0;  // the window's first column in the rectangle
+      const bool copy = w.k0 != last && w.coef == 1.0;
+      last = w.k0;
+      const bool on[2] = {(unsigned)(k + lane) < (unsigned)w.cols, (unsigned)(k + lane + 32) < (unsigned)w.cols};
+      const bool half[2] = {k + 31 >= 0 && k < w.cols, k + 32 < w.cols};  // (every term reaches the window)
+      const T *src = in + (w.in_off + (int64_t)(u.r0 + warp) * w.in_ld + (k + lane));
+      const int64_t step = 8 * (int64_t)w.in_ld;
+      T x[4][2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (half[h]) {
+          const T *row = src + 32 * h;
+#pragma unroll
+          for (int i = 0; i < 4; ++i, row += step) {
+            x[i][h] = T(0);
+            if (on[h] && i < nrow) x[i][h] = *row;
+          }
+        }
+      }
+      if (copy) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (half[h]) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (on[h]) acc[i][h] = x[i][h];
+          }
+      } else {
+        const T cf = (T)w.coef;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (half[h]) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i][h] = fma(cf, x[i][h], acc[i][h]);
+          }
+      }
+    }
+  }
+}
 
 __device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 a, __nv_bfloat16 b) {
   return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
 }
 
-constexpr int WT_ROWS = 32, WT_K = 64, WT_LD = WT_K + 4;  // window and tile row stride (floats)
+constexpr int WT_LD = W_K + 4;  // row stride of the tile (floats)
 
-// group of GW packed elements [kg, kg + GW) of packed row `row` from the tile
-// row v[0..GW); elements outside [ka, kb) are left to their owners
-template <int GW>
-__device__ __forceinline__ void wt_store(float *dst, const WTaskP &t, int row, int kg, int ka, int kb,
-                                         const float *v) {
-  const int rpt = 8 * t.G;
-  const int rt = row / rpt, rr = row - rt * rpt;
-  const bool full = kg >= ka && kg + GW <= kb;
-  if (GW == 8) {  // BF16 pairs, 64 elements per K block
-    const int kbk = kg >> 6, kc = (kg & 63) >> 3;
-    const int64_t tile_h = (int64_t)rpt * 64;
-    const int64_t o = ((int64_t)rt * t.KB + kbk) * 2 * tile_h + (((int64_t)kc * t.G + (rr >> 3)) * 8 + (rr & 7)) * 8;
+// hi/lo split of one 16-byte group (8 BF16 or 4 TF32 elements from packed K kg
+// on) of packed row `row`
+__device__ __forceinline__ void put_group(float *dst, int row, int kg, int KB, int G, int bf16, const float *v) {
+  if (bf16) {
     __nv_bfloat16 hi[8], lo[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       hi[j] = __float2bfloat16_rn(v[j]);
       lo[j] = __float2bfloat16_rn(v[j] - __bfloat162float(hi[j]));
     }
-    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst) + o;
-    if (full) {
-      uint4 hv, lv;
-      hv.x = pack_bf16x2(hi[0], hi[1]);
-      hv.y = pack_bf16x2(hi[2], hi[3]);
-      hv.z = pack_bf16x2(hi[4], hi[5]);
-      hv.w = pack_bf16x2(hi[6], hi[7]);
-      lv.x = pack_bf16x2(lo[0], lo[1]);
-      lv.y = pack_bf16x2(lo[2], lo[3]);
-      lv.z = pack_bf16x2(lo[4], lo[5]);
-      lv.w = pack_bf16x2(lo[6], lo[7]);
-      *reinterpret_cast<uint4 *>(h) = hv;
-      *reinterpret_cast<uint4 *>(h + tile_h) = lv;
-    } else {
+    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst) + packed_off_h(row, kg, KB, G);
+    *reinterpret_cast<uint4 *>(h) = make_uint4(pack_bf16x2(hi[0], hi[1]), pack_bf16x2(hi[2], hi[3]),
+                                               pack_bf16x2(hi[4], hi[5]), pack_bf16x2(hi[6], hi[7]));
+    *reinterpret_cast<uint4 *>(h + (int64_t)8 * G * 64) =
+        make_uint4(pack_bf16x2(lo[0], lo[1]), pack_bf16x2(lo[2], lo[3]), pack_bf16x2(lo[4], lo[5]),
+                   pack_bf16x2(lo[6], lo[7]));
+  } else {
+    float hi[4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (kg + j >= ka && kg + j < kb) {
-          h[j] = hi[j];
-          h[tile_h + j] = lo[j];
-        }
-    }
-  } else {  // TF32 pairs, 32 elements per K block
-    const int kbk = kg >> 5, kc = (kg & 31) >> 2;
-    const int64_t tile_f = (int64_t)rpt * 32;
-    const int64_t o = ((int64_t)rt * t.KB + kbk) * 2 * tile_f + (((int64_t)kc * t.G + (rr >> 3)) * 8 + (rr & 7)) * 4;
-    float hi[4], lo[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      hi[j] = tf32_round(v[j]);
-      lo[j] = v[j] - hi[j];
-    }
-    float *f = dst + o;
-    if (full) {
-      *reinterpret_cast<float4 *>(f) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      *reinterpret_cast<float4 *>(f + tile_f) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (kg + j >= ka && kg + j < kb) {
-          f[j] = hi[j];
-          f[tile_f + j] = lo[j];
-        }
-    }
+    for (int j = 0; j < 4; ++j) hi[j] = tf32_round(v[j]);
+    float *f = dst + packed_off(row, kg, KB, G);
+    *reinterpret_cast<float4 *>(f) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<float4 *>(f + (int64_t)8 * G * 32) =
+        make_float4(v[0] - hi[0], v[1] - hi[1], v[2] - hi[2], v[3] - hi[3]);
   }
 }
 
-__global__ void __launch_bounds__(256) wstage_tc_kernel(const int4 *__restrict__ units,
-                                                        const WTaskP *__restrict__ tasks,
-                                                        const WTerm *__restrict__ terms,
-                                                        double *const *__restrict__ bufs,
-                                                        const int *__restrict__ active, int bf16) {
-  __shared__ __align__(16) float tile[WT_ROWS * WT_LD];
-  const int4 u = units[blockIdx.x];  // (task, first row, K window)
-  const WTaskP t = tasks[u.x];
-  if (active && !active[t.sb]) return;
-  const int r0 = u.y, kw = u.z * WT_K;
-  const int nr = min(WT_ROWS, t.rows - r0);
-  const int ka = max(kw, t.k0), kb = min(kw + WT_K, t.k0 + t.cols);  // packed K of the rectangle in the window
-  const float *in = (const float *)bufs[t.sb * NBUF + t.in_buf];
-  float *dst = (float *)bufs[t.sb * NBUF + t.dst_buf] + t.dst_off;
+constexpr int W_TC_CTAS = 6;  // resident per SM
+__global__ void __launch_bounds__(256, W_TC_CTAS) wstage_tc_kernel(const WUnit *__restrict__ units, int nunits,
+                                                                   const WTaskP *__restrict__ tasks,
+                                                                   const WTerm *__restrict__ terms,
+                                                                   double *const *__restrict__ bufs,
+                                                                   const int *__restrict__ active, int bf16) {
+  __shared__ __align__(16) float tile[W_ROWS * WT_LD];
+  __shared__ WStage S[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // phase 1: warp w holds rows w, w + 8, w + 16, w + 24; lane l columns kw + l, kw + l + 32
-  float acc[4][2];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
-  for (int q = 0; q < t.nterm; ++q) {
-    const WTerm w = terms[t.term0 + q];
-    const float cf = (float)w.coef;
+  w_walk(units, nunits, tasks, terms, S, [&](const WUnit &u, WStage &st) {
+    const WTaskP &t = st.task;
+    if (active && !active[t.sb]) return;
+    const int nr = min(W_ROWS, t.rows - u.r0);
+    float *dst = (float *)bufs[t.sb * NBUF + t.dst_buf] + t.dst_off;
+    float acc[4][2];
+    w_accumulate<float>(u, terms, (const float *)bufs[t.sb * NBUF + t.in_buf], nr, st.term, acc);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = warp + 8 * i;
-      if (r < nr) {
-        const float *src = in + w.in_off + (int64_t)(r0 + r) * w.in_ld;  // packed k at src[k - k0]
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = kw + lane + 32 * h;
-          if (k >= ka && k < kb) acc[i][h] = fmaf(cf, src[k - t.k0], acc[i][h]);
-        }
-      }
+      tile[(warp + 8 * i) * WT_LD + lane] = acc[i][0];
+      tile[(warp + 8 * i) * WT_LD + lane + 32] = acc[i][1];
     }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    tile[(warp + 8 * i) * WT_LD + lane] = acc[i][0];
-    tile[(warp + 8 * i) * WT_LD + lane + 32] = acc[i][1];
-  }
-  __syncthreads();
-  // phase 2: item (group g, row r), r fastest, so a warp covers 32 rows of one group
-  const int gw = bf16 ? 8 : 4, ngr = WT_K / gw;
-  for (int it = threadIdx.x; it < ngr * WT_ROWS; it += blockDim.x) {
-    const int g = it >> 5, r = it & 31;
-    const int kg = kw + g * gw;
-    if (r >= nr || kg + gw <= ka || kg >= kb) continue;
-    const float *v = tile + r * WT_LD + g * gw;
-    if (bf16) {
-      float x[8];
-      *reinterpret_cast<float4 *>(x) = *reinterpret_cast<const float4 *>(v);
-      *reinterpret_cast<float4 *>(x + 4) = *reinterpret_cast<const float4 *>(v + 4);
-      wt_store<8>(dst, t, t.row0 + r0 + r, kg, ka, kb, x);
-    } else {
-      float x[4];
-      *reinterpret_cast<float4 *>(x) = *reinterpret_cast<const float4 *>(v);
-      wt_store<4>(dst, t, t.row0 + r0 + r, kg, ka, kb, x);
+    __syncthreads();  // (the walk's barrier keeps the next window off the tile)
+    if (lane >= nr) return;
+    const int gw = bf16 ? 8 : 4, kend = min(W_K, (bf16 ? 64 : 32) * t.KB - u.k0);
+    for (int k = gw * warp; k < kend; k += 8 * gw) {
+      float v[8];
+      *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(tile + lane * WT_LD + k);
+      if (bf16) *reinterpret_cast<float4 *>(v + 4) = *reinterpret_cast<const float4 *>(tile + lane * WT_LD + k + 4);
+      put_group(dst, t.row0 + u.r0 + lane, u.k0 + k, t.KB, t.G, bf16, v);
     }
-  }
+  });
 }
 
 constexpr int TM = 128;
@@ -520,141 +580,252 @@ __device__ __forceinline__ int oz_exp_of(double x) {
   return be ? be - 1023 + 2 : ilogb(x) + 2;
 }
 
-// The digits from the bits of x, in integer arithmetic (FP64 instructions are
-// scarce here): Y = round(x 2^(56 - e)), |Y| <= 2^55, then balanced base-128
-// digits (-64..63) from the least significant one up, the leading digit
-// taking what is left (|d_0| <= 64): Y = sum_p d_p 128^(7 - p).
-__device__ __forceinline__ void oz_put(__nv_bfloat16 *dst, int row, int k, int KB, int G, int e, double x) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  long long Y = 0;
-  if (e != OZ_EXP_EMPTY && (bits << 1) != 0) {
-    const int be = (int)((bits >> 52) & 0x7FF);
-    unsigned long long mant = bits & ((1ull << 52) - 1);
-    int ex = -1074;  // x = mant 2^ex
-    if (be) {
-      mant |= 1ull << 52;
-      ex = be - 1075;
-    }
-    const int sh = ex + 56 - e;
+// Digits of eight consecutive K elements, from the bits of x in integer
+// arithmetic (FP64 instructions are scarce here): Y = round(x 2^(56 - e)),
+// |Y| <= 2^55, then balanced base-128 digits (-64 .. 63; the leading one takes
+// what is left, |d_0| <= 64): Y = sum_p d_p 128^(7 - p).  Adding 64 to every
+// digit but the leading one makes them plain 7-bit fields u_p = d_p + 64 of
+// Y + 64 sum_{j<7} 128^j.  BF16 128 + u is 0x4300 + u, and subtracting 192 leaves
+// d, exactly.  out[p]: plane p, the eight elements in order.
+__device__ __forceinline__ uint32_t oz_sub192(uint32_t w) {
+  const __nv_bfloat162 r =
+      __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&w), __floats2bfloat162_rn(192.0f, 192.0f));
+  return *reinterpret_cast<const uint32_t *>(&r);
+}
+__device__ __forceinline__ void oz_digits8(const double *v, int e, uint4 (&out)[OZ_PLANES]) {
+  constexpr long long bias = 64ll * ((1ll << 49) - 1) / 127;
+  uint32_t w[OZ_PLANES][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v[i]);
     unsigned long long u = 0;
-    if (sh >= 0)
-      u = mant << sh;  // sh <= 2 since |x| < 2^(e - 1)
-    else if (sh > -62)
-      u = (mant + (1ull << (-sh - 1))) >> (-sh);
-    Y = (bits >> 63) ? -(long long)u : (long long)u;
+    if (e != OZ_EXP_EMPTY && (bits << 1) != 0) {
+      const int be = (int)((bits >> 52) & 0x7FF);
+      unsigned long long mant = bits & ((1ull << 52) - 1);
+      int ex = -1074;  // x = mant 2^ex
+      if (be) {
+        mant |= 1ull << 52;
+        ex = be - 1075;
+      }
+      const int sh = ex + 56 - e;
+      if (sh >= 0)
+        u = mant << sh;  // sh <= 2 since |x| < 2^(e - 1)
+      else if (sh > -62)
+        u = (mant + (1ull << (-sh - 1))) >> (-sh);
+    }
+    const long long Y = ((bits >> 63) ? -(long long)u : (long long)u) + bias;
+    const uint32_t lo = (uint32_t)Y, mid = (uint32_t)(Y >> 28), top = (uint32_t)((int)(Y >> 49) + 64);
+    const uint32_t d[OZ_PLANES] = {top,               (mid >> 14) & 127u, (mid >> 7) & 127u, mid & 127u,
+                                   (lo >> 21) & 127u, (lo >> 14) & 127u,  (lo >> 7) & 127u,  lo & 127u};
+#pragma unroll
+    for (int p = 0; p < OZ_PLANES; ++p)
+      w[p][i >> 1] = (i & 1) ? w[p][i >> 1] + (d[p] << 16) : 0x43004300u + d[p];
   }
 #pragma unroll
-  for (int p = OZ_PLANES - 1; p > 0; --p) {
-    int r = (int)(Y & 127);
-    if (r >= 64) r -= 128;
-    Y = (Y - r) >> 7;
-    dst[oz_off(row, k, KB, G, p)] = __float2bfloat16_rn((float)r);
-  }
-  dst[oz_off(row, k, KB, G, 0)] = __float2bfloat16_rn((float)Y);  // what is left: |Y| <= 64
+  for (int p = 0; p < OZ_PLANES; ++p)
+    out[p] = make_uint4(oz_sub192(w[p][0]), oz_sub192(w[p][1]), oz_sub192(w[p][2]), oz_sub192(w[p][3]));
 }
 
-__device__ __forceinline__ double oz_src(const PackSeg &s, double *const *bufs, int r, int k) {
-  const int64_t si = s.trans ? (int64_t)k * s.src_ld + r : (int64_t)r * s.src_ld + k;
-  const double x = s.src_fp32 ? (double)((const float *)bufs[s.sb * NBUF + s.src_buf])[s.src_off + si]
-                              : bufs[s.sb * NBUF + s.src_buf][s.src_off + si];
+// Packing runs through windows of 32 rows and 64 packed K columns (aligned to
+// 64) held in shared memory: read with the lanes along whatever is contiguous
+// in the source, written with a row and eight K elements per thread, so that a
+// warp fills 512 contiguous bytes of every plane (128 of a B plane).  It is
+// memory bound: 8 bytes in, 16 out per element.  (Before, a thread per element
+// stored 16 bits per plane; environments and prediction of the kagome cylinder
+// at m = 1000 11.6 -> 8.2 ms a step with it.)
+static_assert(W_ROWS == PACK_ROWS && W_K == 64, "windows of oz_store_window");
+constexpr int OP_ROWS = PACK_ROWS, OP_K = 64, OP_LD = OP_K + 2;
+
+// The thread's share of a window: packed row row0 + lane (lane < nr), K group
+// kw + 8 warp; elements outside [ka, kb) belong to a neighbour.
+__device__ __forceinline__ void oz_store_window(__nv_bfloat16 *dst, const double *tile, int e, int row0, int nr, int kw,
+                                                int ka, int kb, int KB, int G) {
+  const int g = threadIdx.x >> 5, r = threadIdx.x & 31;
+  const int kg = kw + 8 * g;
+  if (r >= nr || kg + 8 <= ka || kg >= kb) return;
+  double v[8];
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    const double2 x = *reinterpret_cast<const double2 *>(tile + r * OP_LD + 8 * g + j);
+    v[j] = x.x;
+    v[j + 1] = x.y;
+  }
+  uint4 d[OZ_PLANES];
+  oz_digits8(v, e, d);
+  const int64_t step = oz_off(0, 0, KB, G, 1);  // from plane to plane
+  __nv_bfloat16 *o = dst + oz_off(row0 + r, kg, KB, G, 0);
+  if (kg >= ka && kg + 8 <= kb) {
+#pragma unroll
+    for (int p = 0; p < OZ_PLANES; ++p) *reinterpret_cast<uint4 *>(o + p * step) = d[p];
+  } else {
+#pragma unroll
+    for (int p = 0; p < OZ_PLANES; ++p) {
+      const uint32_t w[4] = {d[p].x, d[p].y, d[p].z, d[p].w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (kg + j >= ka && kg + j < kb)
+          o[p * step + j] = __ushort_as_bfloat16((unsigned short)(w[j >> 1] >> (16 * (j & 1))));
+    }
+  }
+}
+
+__device__ __forceinline__ double oz_src(const PackSeg &s, const double *src, int r, int k) {
+  const double x = src[s.trans ? (int64_t)k * s.src_ld + r : (int64_t)r * s.src_ld + k];
   return s.alpha == 1.0 ? x : s.alpha * x;
 }
 
-// exponents of rows whose K range spans several segments
-__global__ void oz_exp_kernel(const PackSeg *__restrict__ segs, double *const *__restrict__ bufs,
-                              const int *__restrict__ active) {
-  const PackSeg s = segs[blockIdx.x];
-  if (active && !active[s.sb]) return;
-  const int r0 = blockIdx.y * PROWS;
-  if (r0 >= s.rows || s.whole) return;
-  const int r1 = min(s.rows, r0 + PROWS);
-  __shared__ int rexp[PROWS];
-  int *ex = (int *)bufs[s.sb * NBUF + s.exp_buf] + s.exp_off + s.row0;
-  const int n = (r1 - r0) * s.ks;
-  if (threadIdx.x < PROWS) rexp[threadIdx.x] = OZ_EXP_EMPTY;
+// exponents of the rows r0 .. r0 + nr - 1 of a segment into rexp[32] (every
+// thread of the block takes part)
+__device__ __forceinline__ void oz_row_exps(const PackSeg &s, const double *src, int r0, int nr, int *rexp) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < OP_ROWS) rexp[threadIdx.x] = OZ_EXP_EMPTY;
   __syncthreads();
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    const int r = r0 + e / s.ks, k = e % s.ks;
-    const double x = oz_src(s, bufs, r, k);
-    if (x != 0.0) atomicMax(&rexp[r - r0], oz_exp_of(x));
+  // several loads in flight per thread: the source is read at memory latency
+  if (s.trans) {
+    int m = OZ_EXP_EMPTY;
+    if (lane < nr) {
+#pragma unroll 8
+      for (int k = warp; k < s.ks; k += 8) {
+        const double x = oz_src(s, src, r0 + lane, k);
+        if (x != 0.0) m = max(m, oz_exp_of(x));
+      }
+    }
+    if (m != OZ_EXP_EMPTY) atomicMax(&rexp[lane], m);
+  } else {
+    int m[4] = {OZ_EXP_EMPTY, OZ_EXP_EMPTY, OZ_EXP_EMPTY, OZ_EXP_EMPTY};
+#pragma unroll 2
+    for (int k = lane; k < s.ks; k += 32) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const double x = warp + 8 * i < nr ? oz_src(s, src, r0 + warp + 8 * i, k) : 0.0;
+        if (x != 0.0) m[i] = max(m[i], oz_exp_of(x));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+      if (lane == 0) rexp[warp + 8 * i] = m[i];
+    }
   }
   __syncthreads();
-  if (threadIdx.x < r1 - r0 && rexp[threadIdx.x] != OZ_EXP_EMPTY) atomicMax(ex + r0 + threadIdx.x, rexp[threadIdx.x]);
+}
+
+// exponents of rows whose K range spans several segments
+__global__ void __launch_bounds__(256) oz_exp_kernel(const int2 *__restrict__ units, const PackSeg *__restrict__ segs,
+                                                     double *const *__restrict__ bufs,
+                                                     const int *__restrict__ active) {
+  __shared__ int rexp[OP_ROWS];
+  const int2 u = units[blockIdx.x];  // (segment, first row)
+  const PackSeg s = segs[u.x];
+  if (s.whole || (active && !active[s.sb])) return;
+  const int nr = min(OP_ROWS, s.rows - u.y);
+  oz_row_exps(s, bufs[s.sb * NBUF + s.src_buf] + s.src_off, u.y, nr, rexp);
+  int *ex = (int *)bufs[s.sb * NBUF + s.exp_buf] + s.exp_off + s.row0 + u.y;
+  if (threadIdx.x < nr && rexp[threadIdx.x] != OZ_EXP_EMPTY) atomicMax(ex + threadIdx.x, rexp[threadIdx.x]);
 }
 
 // digits; a segment that holds the whole K range of its rows finds their
 // exponents itself (and stores them), the others read them
-__global__ void oz_pack_kernel(const PackSeg *__restrict__ segs, double *const *__restrict__ bufs,
-                               const int *__restrict__ active) {
-  __shared__ int rexp[PROWS];
-  const PackSeg s = segs[blockIdx.x];
+__global__ void __launch_bounds__(256, 3) oz_pack_kernel(const int2 *__restrict__ units,
+                                                      const PackSeg *__restrict__ segs,
+                                                      double *const *__restrict__ bufs,
+                                                      const int *__restrict__ active) {
+  __shared__ __align__(16) double tile[OP_ROWS * OP_LD];
+  __shared__ int rexp[OP_ROWS];
+  const int2 u = units[blockIdx.x];  // (segment, first row)
+  const PackSeg s = segs[u.x];
   if (active && !active[s.sb]) return;
-  const int r0 = blockIdx.y * PROWS;
-  if (r0 >= s.rows) return;
-  const int r1 = min(s.rows, r0 + PROWS);
-  int *ex = (int *)bufs[s.sb * NBUF + s.exp_buf] + s.exp_off + s.row0;
+  const int r0 = u.y, nr = min(OP_ROWS, s.rows - r0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int *ex = (int *)bufs[s.sb * NBUF + s.exp_buf] + s.exp_off + s.row0 + r0;
+  const double *src = bufs[s.sb * NBUF + s.src_buf] + s.src_off;
   __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(bufs[s.sb * NBUF + s.dst_buf]) + s.dst_off;
-  const int n = (r1 - r0) * s.ks;
   if (s.whole) {
-    if (threadIdx.x < PROWS) rexp[threadIdx.x] = OZ_EXP_EMPTY;
+    oz_row_exps(s, src, r0, nr, rexp);
+    if (threadIdx.x < nr) ex[threadIdx.x] = rexp[threadIdx.x];
+  } else {
+    if (threadIdx.x < nr) rexp[threadIdx.x] = ex[threadIdx.x];
+  }
+  const int k1 = s.k0 + s.ks, kend = k1 + s.kpad;  // zeros up to the end of the last K block
+  for (int kw = s.k0 & ~(OP_K - 1); kw < kend; kw += OP_K) {
     __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int r = r0 + e / s.ks, k = e % s.ks;
-      const double x = oz_src(s, bufs, r, k);
-      if (x != 0.0) atomicMax(&rexp[r - r0], oz_exp_of(x));
+    if (s.trans) {
+#pragma unroll
+      for (int i = 0; i < OP_K / 8; ++i) {
+        const int kk = warp + 8 * i, k = kw + kk;
+        if (lane < nr) tile[lane * OP_LD + kk] = k >= s.k0 && k < k1 ? oz_src(s, src, r0 + lane, k - s.k0) : 0.0;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < OP_ROWS / 8; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = warp + 8 * i, kk = lane + 32 * h, k = kw + kk;
+          if (r < nr) tile[r * OP_LD + kk] = k >= s.k0 && k < k1 ? oz_src(s, src, r0 + r, k - s.k0) : 0.0;
+        }
     }
     __syncthreads();
-    if (threadIdx.x < r1 - r0) ex[r0 + threadIdx.x] = rexp[threadIdx.x];
-  } else {
-    if (threadIdx.x < r1 - r0) rexp[threadIdx.x] = ex[r0 + threadIdx.x];
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    const int r = r0 + e / s.ks, k = e % s.ks;
-    oz_put(dst, s.row0 + r, s.k0 + k, s.KB, s.G, rexp[r - r0], oz_src(s, bufs, r, k));
+    oz_store_window(dst, tile, lane < nr ? rexp[lane] : 0, s.row0 + r0, nr, kw, s.k0, kend, s.KB, s.G);
   }
 }
 
-// T3 = sum W12 T1 in FP64 from the FP64 stage-1 output.  Pass 0 stores T3
-// (row-major per stage-3 task, K = the task's full K) and takes the row
-// exponents (a maximum per block in shared memory, then one atomic per row
-// and block); pass 1 turns the stored values into digits.
-__global__ void wstage_oz_kernel(const WTaskP *__restrict__ tasks, const WTerm *__restrict__ terms,
-                                 double *const *__restrict__ bufs, const int *__restrict__ active, int pass) {
-  __shared__ int rexp[PROWS];
-  const WTaskP t = tasks[blockIdx.x];
-  if (active && !active[t.sb]) return;
-  const int r0 = blockIdx.y * PROWS;
-  if (r0 >= t.rows) return;
-  const int r1 = min(t.rows, r0 + PROWS);
-  int *ex = (int *)bufs[t.sb * NBUF + BUF_OEXP] + t.exp_off + t.row0;
-  double *t3 = bufs[t.sb * NBUF + BUF_OT3] + t.t3_off + (int64_t)t.row0 * t.t3_ld + t.k0;
-  const int n = (r1 - r0) * t.cols;
-  if (pass == 0) {
-    const double *in = bufs[t.sb * NBUF + t.in_buf];
-    if (threadIdx.x < PROWS) rexp[threadIdx.x] = OZ_EXP_EMPTY;
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int r = r0 + e / t.cols, c = e % t.cols;
-      double acc = 0.0;
-      for (int q = 0; q < t.nterm; ++q) {
-        const WTerm w = terms[t.term0 + q];
-        acc = fma(w.coef, in[w.in_off + (int64_t)r * w.in_ld + c], acc);
+// T3 = sum W12 T1 in FP64 from the FP64 stage-1 output, in the windows of
+// wstage_tc_kernel.  Pass 0 takes the row exponents of T3, which need all of a
+// row (every channel's rectangle); pass 1 writes the digits.  Where T3 copies
+// T1 pass 1 reads T1 again, which moves less than storing T3 would; windows
+// with sums (the completed channel's, about one in w, of up to 2 w terms, bound
+// by the FP64 units) are kept by pass 0 in `keep`, 16 KB each.
+constexpr int W_OZ_CTAS[2] = {4, 3};  // resident per SM
+template <int PASS>
+__global__ void __launch_bounds__(256, W_OZ_CTAS[PASS]) wstage_oz_kernel(const WUnit *__restrict__ units, int nunits,
+                                                                         const WTaskP *__restrict__ tasks,
+                                                                         const WTerm *__restrict__ terms,
+                                                                         double *const *__restrict__ bufs,
+                                                                         double *__restrict__ keep,
+                                                                         const int *__restrict__ active) {
+  __shared__ __align__(16) double tile[PASS ? W_ROWS * OP_LD : 2];
+  __shared__ WStage S[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  w_walk(units, nunits, tasks, terms, S, [&](const WUnit &u, WStage &st) {
+    const WTaskP &t = st.task;
+    if (active && !active[t.sb]) return;
+    const int nr = min(W_ROWS, t.rows - u.r0);
+    int *ex = (int *)bufs[t.sb * NBUF + BUF_OEXP] + t.exp_off + t.row0 + u.r0;
+    const int e = PASS && lane < nr ? ex[lane] : 0;
+    double *kept = u.slot >= 0 ? keep + (int64_t)u.slot * (W_ROWS * W_K) + warp * W_K + lane : nullptr;
+    double acc[4][2];
+    if (PASS == 0 || !kept) {
+      w_accumulate<double>(u, terms, bufs[t.sb * NBUF + t.in_buf], nr, st.term, acc);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[i][0] = kept[8 * i * W_K];
+        acc[i][1] = kept[8 * i * W_K + 32];
       }
-      t3[(int64_t)r * t.t3_ld + c] = acc;
-      if (acc != 0.0) atomicMax(&rexp[r - r0], oz_exp_of(acc));
     }
-    __syncthreads();
-    if (threadIdx.x < r1 - r0 && rexp[threadIdx.x] != OZ_EXP_EMPTY) atomicMax(ex + r0 + threadIdx.x, rexp[threadIdx.x]);
-  } else {
-    __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(bufs[t.sb * NBUF + t.dst_buf]) + t.dst_off;
-    if (threadIdx.x < r1 - r0) rexp[threadIdx.x] = ex[r0 + threadIdx.x];
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      const int r = r0 + e / t.cols, c = e % t.cols;
-      oz_put(dst, t.row0 + r, t.k0 + c, t.KB, t.G, rexp[r - r0], t3[(int64_t)r * t.t3_ld + c]);
+    if (PASS == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        int m = OZ_EXP_EMPTY;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (acc[i][h] != 0.0) m = max(m, oz_exp_of(acc[i][h]));
+          if (kept) kept[8 * i * W_K + 32 * h] = acc[i][h];
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0 && m != OZ_EXP_EMPTY) atomicMax(ex + warp + 8 * i, m);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        tile[(warp + 8 * i) * OP_LD + lane] = acc[i][0];
+        tile[(warp + 8 * i) * OP_LD + lane + 32] = acc[i][1];
+      }
+      __syncthreads();
+      __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(bufs[t.sb * NBUF + t.dst_buf]) + t.dst_off;
+      oz_store_window(dst, tile, e, t.row0 + u.r0, nr, u.k0, u.k0, min(u.k0 + W_K, OZ_KBLK * t.KB), t.KB, t.G);
     }
-  }
+  });
 }
 
 constexpr int OZ_A_PLANE = TM * OZ_KBLK * 2;       // bytes of one A digit plane of a K block
@@ -954,45 +1125,28 @@ __global__ void __launch_bounds__(32 * OZ_SUM_ROWS) oz_sum_kernel(const int *__r
   }
 }
 
-// streaming multiprocessors of the current device (0: query failed)
-int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return 0;
-    sms = n;
-  }
-  return sms;
-}
-
 }  // namespace
 
-cudaError_t launch_oz_exp(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+cudaError_t launch_oz_exp(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                           cudaStream_t st) {
-  if (nseg > 0 && max_rows > 0) {
-    dim3 grid(nseg, (max_rows + PROWS - 1) / PROWS);
-    oz_exp_kernel<<<grid, 256, 0, st>>>(segs, bufs, active);
-  }
+  if (nunits > 0) oz_exp_kernel<<<nunits, 256, 0, st>>>(units, segs, bufs, active);
   return cudaGetLastError();
 }
 
-cudaError_t launch_oz_pack(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+cudaError_t launch_oz_pack(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                            cudaStream_t st) {
-  if (nseg > 0 && max_rows > 0) {
-    dim3 grid(nseg, (max_rows + PROWS - 1) / PROWS);
-    oz_pack_kernel<<<grid, 256, 0, st>>>(segs, bufs, active);
-  }
+  if (nunits > 0) oz_pack_kernel<<<nunits, 256, 0, st>>>(units, segs, bufs, active);
   return cudaGetLastError();
 }
 
-cudaError_t launch_wstage_oz(const WTaskP *tasks, int ntasks, int max_rows, const WTerm *terms,
-                             double *const *bufs, const int *active, int pass, cudaStream_t st) {
-  if (ntasks > 0 && max_rows > 0) {
-    dim3 grid(ntasks, (max_rows + PROWS - 1) / PROWS);
-    wstage_oz_kernel<<<grid, 256, 0, st>>>(tasks, terms, bufs, active, pass);
-  }
+cudaError_t launch_wstage_oz(const WUnit *units, int nunits, const WTaskP *tasks, const WTerm *terms,
+                             double *const *bufs, double *keep, const int *active, int pass, cudaStream_t st) {
+  if (nunits <= 0) return cudaGetLastError();
+  const int sms = sm_count();
+  if (sms <= 0) return cudaErrorInvalidValue;
+  const int most = W_OZ_CTAS[pass ? 1 : 0] * sms, grid = nunits < most ? nunits : most;
+  (pass ? wstage_oz_kernel<1> : wstage_oz_kernel<0>)<<<grid, 256, 0, st>>>(units, nunits, tasks, terms, bufs, keep,
+                                                                             active);
   return cudaGetLastError();
 }
 
@@ -1025,9 +1179,13 @@ cudaError_t launch_pack(const PackSeg *segs, int nseg, int max_rows, double *con
   return cudaGetLastError();
 }
 
-cudaError_t launch_wstage_tc(const int4 *units, int nunits, const WTaskP *tasks, const WTerm *terms,
+cudaError_t launch_wstage_tc(const WUnit *units, int nunits, const WTaskP *tasks, const WTerm *terms,
                              double *const *bufs, const int *active, int bf16, cudaStream_t st) {
-  if (nunits > 0) wstage_tc_kernel<<<nunits, 256, 0, st>>>(units, tasks, terms, bufs, active, bf16);
+  if (nunits <= 0) return cudaGetLastError();
+  const int sms = sm_count();
+  if (sms <= 0) return cudaErrorInvalidValue;
+  const int most = W_TC_CTAS * sms;
+  wstage_tc_kernel<<<nunits < most ? nunits : most, 256, 0, st>>>(units, nunits, tasks, terms, bufs, active, bf16);
   return cudaGetLastError();
 }
 
