@@ -2383,16 +2383,8 @@ idmrg_status truncate(idmrg_ctx *c, int p) {
   c->kend(PH + 0);
   c->kbegin(PH + 1);
   CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 0, sw, c->st));
-  {
-    // group 0 from g0b on fits the shared-memory FP32 tournament (none in
-    // the forced large-sector mode, which exercises the all-global kernel)
-    const int bmax = c->svd_global ? 0 : svd_jacobi32_big_max_cols();
-    int g0b = 0;
-    while (g0b < g[0] && c->jobs[c->torder[g0b]].cols_a > bmax) ++g0b;
-    const int cols0b = g0b < g[0] ? c->jobs[c->torder[g0b]].cols_a : 0;
-    CK(launch_svd_jacobi32(dj, (const int *)c->sorder.p, nj, g, gcols, cols0, g0b, cols0b, sw, (const int *)c->siw.p,
-                           c->st, c->side, c->sev));
-  }
+  CK(launch_svd_jacobi32(dj, (const int *)c->sorder.p, nj, g, gcols, cols0, sw, (const int *)c->siw.p, c->st,
+                         c->side, c->sev));
   c->kend(PH + 1);
   c->kbegin(PH + 2);
   for (int it = 0; it < 2; ++it) {

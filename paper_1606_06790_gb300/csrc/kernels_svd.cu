@@ -1826,204 +1826,95 @@ __global__ void __launch_bounds__(BJ_THREADS, 2)
   }
 }
 
-// FP32 stage for sectors of up to 32 * J32B_REG rows whose rotations do not
-// fit next to B in shared memory: the block tournament of
-// jacobi32_block_kernel with only B's columns in shared memory (four slots of
-// bw columns) and the rotations in global memory (FP32, n x n, in the job's
-// x_off area), each column of the rotations updated by the CTA that holds
-// its block in that round; the cluster barrier that ends a round also
-// publishes those updates to the CTA that holds the block next.
-constexpr int J32B_REG = 32;  // rows per lane in registers: up to 1024 rows
-__global__ void __launch_bounds__(BJ_THREADS, 1)
-    jacobi32_big_kernel(const SvdJob *__restrict__ jobs, const int *__restrict__ order, double *__restrict__ work,
-                        const int *__restrict__ iwork) {
-  extern __shared__ __align__(16) float bg_sm[];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank();
-  const int C = (int)cluster.num_blocks();
-  const SvdJob Jb = jobs[order[blockIdx.x / C]];
-  const int nr = Jb.cols_a;
-  const int n = iwork[Jb.perm_off + Jb.cols_a];
-  const int P = 2 * C;
-  const int bw = (n + P - 1) / P;
-  const int nreg = (nr + 31) >> 5;
-  const int ldb = 32 * nreg;
-  const int slot = (bw * ldb + 3) & ~3;  // 16-byte aligned blocks
-  __shared__ int flag, local_changed, sweep_rmax, cl_rmax;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const double *Bg = work + Jb.b_off;
-  double *Vg = work + Jb.j_off;
-  float *V32 = reinterpret_cast<float *>(work + Jb.x_off);  // n x n, leading dimension n
-  const int pos[2] = {crank, P - 1 - crank};
-  auto slotp = [&](int buf, int which) { return bg_sm + (buf * 2 + which) * slot; };
-  auto valid = [&](int k) { return max(0, min(bw, n - k * bw)); };
-  if (nreg > J32B_REG || n < 2) return;  // uniform over the cluster
-  for (int w = 0; w < 2; ++w) {
-    const int k = pos[w], nv = valid(k);
-    float *sb = slotp(0, w);
-    for (int e = threadIdx.x; e < bw * ldb; e += blockDim.x) {
-      const int j = e / ldb, i = e - j * ldb;
-      sb[e] = (j < nv && i < nr) ? (float)Bg[(int64_t)(k * bw + j) * nr + i] : 0.0f;
-    }
-    for (int64_t e = threadIdx.x; e < (int64_t)nv * n; e += blockDim.x) {
-      const int64_t j = e / n, i = e - j * n;
-      V32[(k * bw + j) * n + i] = (i == k * bw + j) ? 1.0f : 0.0f;
-    }
-  }
-  const float tol = sqrtf((float)nr) * FLT_EPSILON;
-  int *flag0 = cluster.map_shared_rank(&flag, 0);
-  int *rmax0 = cluster.map_shared_rank(&cl_rmax, 0);
-  int cur = 0;
-  bool converged = false;
-  auto wsumf = [](float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  };
-  // one pair, one warp: columns i of s0 (block b0) and j of s1 (block b1)
-  auto pair = [&](float *s0, int b0, int i, float *s1, int b1, int j, float &rmax) -> bool {
-    float *xp = s0 + i * ldb, *xq = s1 + j * ldb;
-    float x[J32B_REG], y[J32B_REG], a = 0.f, b = 0.f, g = 0.f;
-#pragma unroll
-    for (int r = 0; r < J32B_REG; ++r)
-      if (r < nreg) {
-        x[r] = xp[lane + 32 * r];
-        y[r] = xq[lane + 32 * r];
-        a = fmaf(x[r], x[r], a);
-        b = fmaf(y[r], y[r], b);
-        g = fmaf(x[r], y[r], g);
-      }
-    a = wsumf(a);
-    b = wsumf(b);
-    g = wsumf(g);
-    if (!(a > 0.f) || !(b > 0.f)) return false;
-    const float ratio = fabsf(g) / sqrtf(a) / sqrtf(b);
-    if (!(ratio > tol)) return false;
-    const float z = (b - a) / (2.0f * g);
-    const float t = z == 0.f ? 1.0f : copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
-    if (!(fabsf(t) >= FLT_MIN) || !isfinite(t)) return false;
-    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
-#pragma unroll
-    for (int r = 0; r < J32B_REG; ++r)
-      if (r < nreg) {
-        xp[lane + 32 * r] = c * x[r] - sn * y[r];
-        xq[lane + 32 * r] = fmaf(sn, x[r], c * y[r]);
-      }
-    float *jp = V32 + (int64_t)(b0 * bw + i) * n, *jq = V32 + (int64_t)(b1 * bw + j) * n;
-    for (int e = lane; e < n; e += 32) {
-      const float u = jp[e], v = jq[e];
-      jp[e] = c * u - sn * v;
-      jq[e] = fmaf(sn, u, c * v);
-    }
-    rmax = fmaxf(rmax, ratio);
-    return true;
-  };
-  int sweep = 0;
-  for (; sweep < 15 && !converged; ++sweep) {
-    if (threadIdx.x == 0) {
-      local_changed = 0;
-      sweep_rmax = 0;
-    }
-    if (crank == 0 && threadIdx.x == 0) {
-      flag = 0;
-      cl_rmax = 0;
-    }
-    cluster.sync();
-    bool any = false;
-    float rmax = 0.f;
-    for (int rnd = 0; rnd < P - 1; ++rnd) {
-      float *st0 = slotp(cur, 0), *st1 = slotp(cur, 1);
-      const int b0 = bj_block_at(pos[0], rnd, P), b1 = bj_block_at(pos[1], rnd, P);
-      const int nv0 = valid(b0), nv1 = valid(b1);
-      if (rnd == 0) {
-        const int bp = bw + (bw & 1), half = bp / 2, bm = bp - 1;
-        for (int w = 0; w < 2; ++w) {
-          const int nv = w ? nv1 : nv0, bk = w ? b1 : b0;
-          float *sb = w ? st1 : st0;
-          for (int sr = 0; sr < bm; ++sr) {
-            for (int i = warp; i < half; i += nw) {
-              int p = 0, q;
-              if (i != 0) {
-                p = i - 1 + sr;
-                p = 1 + (p >= bm ? p - bm : p);
-              }
-              q = bp - 2 - i + sr;
-              q = 1 + (q >= bm ? q - bm : q);
-              if (p < nv && q < nv) any |= pair(sb, bk, p, sb, bk, q, rmax);
-            }
-            __syncthreads();
-          }
-        }
-      }
-      for (int sr = 0; sr < bw; ++sr) {
-        for (int i = warp; i < bw; i += nw) {
-          int j = i + sr;
-          if (j >= bw) j -= bw;
-          if (i < nv0 && j < nv1) any |= pair(st0, b0, i, st1, b1, j, rmax);
-        }
-        __syncthreads();
-      }
-      if (C > 1) {
-        for (int w = 0; w < 2; ++w) {
-          const int dpn = pos[w] == 0 ? 0 : (pos[w] == P - 1 ? 1 : pos[w] + 1);
-          const int drank = dpn < C ? dpn : P - 1 - dpn, dw = dpn < C ? 0 : 1;
-          float4 *dst = reinterpret_cast<float4 *>(cluster.map_shared_rank(slotp(cur ^ 1, dw), drank));
-          const float4 *src = reinterpret_cast<const float4 *>(w ? st1 : st0);
-          for (int e = threadIdx.x; e < slot / 4; e += blockDim.x) dst[e] = src[e];
-        }
-        cluster.sync();
-        cur ^= 1;
-      } else {
-        __syncthreads();
-      }
-    }
-    if (any && lane == 0) local_changed = 1;
-    if (lane == 0) atomicMax(&sweep_rmax, __float_as_int(rmax));
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (local_changed) atomicOr(flag0, 1);
-      atomicMax(rmax0, sweep_rmax);
-    }
-    cluster.sync();
-    const float r = __int_as_float(*rmax0);
-    converged = (*flag0 == 0) || ((float)n * r * r < tol) || r < J32_PRECOND_R;
-    cluster.sync();
-  }
-  if (crank == 0 && threadIdx.x == 0) iwork32_sweeps(iwork, Jb, sweep);
-  // rotations to V (FP64, cols_a x cols_a): the columns of this CTA's two
-  // home blocks (every block is back at its starting position after whole sweeps)
-  for (int w = 0; w < 2; ++w) {
-    const int k = pos[w], nv = valid(k);
-    for (int64_t e = threadIdx.x; e < (int64_t)nv * n; e += blockDim.x) {
-      const int64_t j = e / n, i = e - j * n;
-      Vg[(k * bw + j) * nr + i] = (double)V32[(k * bw + j) * n + i];
-    }
-  }
-}
-
-// FP32 stage for sectors too large for jacobi32_big_kernel: the same block
-// tournament, with the blocks kept in global memory (the FP32 copy of B in
-// the job's x_off area) and streamed through shared memory.  The rank-n
-// columns are cut into P = 2 C k blocks of bw columns, bw small enough that
-// one pair of blocks fits in a CTA's shared memory; in every round each CTA
-// visits k of the round's P/2 block pairs in turn: it loads both blocks,
-// rotates every column of one against every column of the other (bw
-// sub-rounds of bw disjoint pairs; in the first round of a sweep also the
-// pairs inside each block), writes them back and applies the visit's
-// rotations, accumulated in a 2bw x 2bw matrix Q, to the same columns of the
-// FP32 rotations V (n x n, after B32) in one pass.  Rounds are separated by
-// the cluster barrier; blocks written in one round are read by other CTAs of
-// the cluster in the next, through L2 (loads bypass L1).  A sweep costs
-// P - 1 cluster barriers instead of n - 1.
-constexpr int JS_THREADS = 512;
+// FP32 stage for sectors beyond the block kernels: a block tournament with the
+// blocks kept in global memory (the FP32 copy of B in the job's x_off area, in
+// L2) and streamed through shared memory.  The rank-n columns are cut into
+// P = 2 C k blocks of bw columns, bw small enough that one pair of blocks fits
+// in a CTA's shared memory; in every round each CTA visits k of the round's P/2
+// block pairs in turn: it loads both blocks, rotates every column of one
+// against every column of the other (bw sub-rounds of bw disjoint pairs; in the
+// first round of a sweep also the pairs inside each block), writes them back
+// and applies the visit's rotations, accumulated in a 2bw x 2bw matrix Q, to the
+// same columns of the FP32 rotations V (n x n, after B32) in one pass.  Rounds
+// are separated by the cluster barrier; blocks written in one round are read by
+// other CTAs of the cluster in the next, through L2 (loads bypass L1).  A sweep
+// costs P - 1 cluster barriers instead of n - 1.
+//
+// A sub-round is bound by the latency of its pairs (dot product, reduction,
+// rotation) and by shared-memory bandwidth.  Hence one warp per pair of the
+// sub-round (bw warps), and for columns of up to 128 R4 rows a warp keeps its
+// column of the first block, and that column of Q, in registers for the whole
+// visit: only the partner is read and written, once each.  R4 = 0: columns of
+// any length, both read from shared memory for the dot product and again for
+// the rotation.
+// Measured (GB300; before: sectors of up to 640 columns on a kernel that held B
+// in shared memory and V's columns in L2, a round trip per pair): FP32 stage of
+// a step of the J1-J2 cylinder at m = 1024 (sectors of up to 566 columns) 49 ->
+// 23 ms, of the kagome cylinder at m = 1000 127 -> 30 ms.  A visit of 17 + 17
+// columns of 537 rows took 30 k cycles in its sub-rounds and 58 k in V Q (a
+// branch between any two loads of Q) before js_apply_q.
 constexpr int JS_BW_MAX = 20;  // columns per block: a row of the two blocks of V fits in registers
+constexpr int JS_THREADS = 32 * JS_BW_MAX;
 
 // shared memory of jacobi32_stream_kernel: two blocks of bw_cap columns of
 // ldb floats, Q (2 bw_cap columns of leading dimension qld), two norm arrays
-__host__ __device__ constexpr int js_qld(int bw_cap) { return (2 * bw_cap + 3) & ~3; }
+__host__ __device__ constexpr int js_qld(int bw_cap) { return (2 * bw_cap + 7) & ~7; }
 __host__ __device__ constexpr int64_t js_smem_floats(int bw_cap, int ldb) {
   return 2 * (int64_t)bw_cap * ldb + (int64_t)js_qld(bw_cap) * 2 * bw_cap + 2 * bw_cap;
 }
 
+// The rotation that makes columns of squared norms a, b and overlap g
+// orthogonal, in FP32: false if their relative overlap is at most tol.
+__device__ __forceinline__ bool js_rotation(float a, float b, float g, float tol, float &ratio, float &t, float &c,
+                                            float &sn) {
+  if (!(a > 0.f) || !(b > 0.f)) return false;
+  ratio = fabsf(g) * rsqrtf(a) * rsqrtf(b);
+  if (!(ratio > tol)) return false;
+  const float z = __fdividef(b - a, 2.0f * g);
+  const float q = fmaf(z, z, 1.0f);
+  t = z == 0.f ? 1.0f : copysignf(__fdividef(1.0f, fabsf(z) + q * rsqrtf(q)), z);
+  if (!(fabsf(t) >= FLT_MIN) || !isfinite(t)) return false;
+  c = rsqrtf(fmaf(t, t, 1.0f));
+  sn = c * t;
+  return true;
+}
+
+// V's columns of blocks b0 (nv0 valid ones) and b1 times Q, whose 2 bw rows are
+// padded with zeros to QD: a row per thread, four outputs at a time, without a
+// branch between the loads of Q.
+template <int QD>
+__device__ __forceinline__ void js_apply_q(float *V32, int n, const float *Q, int bw, int b0, int nv0, int b1,
+                                           int nv1) {
+  static_assert(QD <= 2 * JS_BW_MAX, "a row in registers");
+  float *V0 = V32 + (int64_t)b0 * bw * n, *V1 = V32 + (int64_t)(b1 * bw - bw) * n;
+  const int qd = 2 * bw;
+  auto there = [&](int c) { return c < bw ? c < nv0 : c - bw < nv1; };  // c < qd
+  for (int row = threadIdx.x; row < n; row += blockDim.x) {
+    float x[QD];
+#pragma unroll
+    for (int r = 0; r < QD; ++r)
+      x[r] = r < qd && there(r) ? __ldcg((r < bw ? V0 : V1) + (int64_t)r * n + row) : 0.0f;
+#pragma unroll 1
+    for (int oc = 0; oc < qd; oc += 4) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int r = 0; r < QD; r += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float4 w = *reinterpret_cast<const float4 *>(Q + min(oc + u, qd - 1) * QD + r);
+          acc[u] = fmaf(x[r], w.x, acc[u]);
+          acc[u] = fmaf(x[r + 1], w.y, acc[u]);
+          acc[u] = fmaf(x[r + 2], w.z, acc[u]);
+          acc[u] = fmaf(x[r + 3], w.w, acc[u]);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (oc + u < qd && there(oc + u)) (oc + u < bw ? V0 : V1)[(int64_t)(oc + u) * n + row] = acc[u];
+    }
+  }
+}
+
+template <int R4>
 __global__ void __launch_bounds__(JS_THREADS, 1)
     jacobi32_stream_kernel(const SvdJob *__restrict__ jobs, const int *__restrict__ order, double *__restrict__ work,
                            const int *__restrict__ iwork, int bw_cap, int ldb) {
@@ -2040,10 +1931,11 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
   const int nb = (n + bw - 1) / bw;
   const int P = 2 * C * ((nb + 2 * C - 1) / (2 * C));
   bw = (n + P - 1) / P;
-  const int k = P / (2 * C), qd = 2 * bw, qld = js_qld(bw_cap);
+  const int k = P / (2 * C), qd = 2 * bw, qld = (qd + 7) & ~7;
+  const int ld = (nr + 31) & ~31;                  // this job's column stride in shared memory (<= ldb)
   float *S0 = js_sm, *S1 = js_sm + (size_t)bw_cap * ldb;
   float *Q = S1 + (size_t)bw_cap * ldb;            // column c at Q + c qld, rows 0 .. qd-1 (padding rows zero)
-  float *N0 = Q + (size_t)qld * 2 * bw_cap, *N1 = N0 + bw_cap;  // squared column norms of S0, S1
+  float *N0 = Q + (size_t)js_qld(bw_cap) * 2 * bw_cap, *N1 = N0 + bw_cap;  // squared column norms of S0, S1
   __shared__ int flag, local_changed, sweep_rmax, cl_rmax;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const double *Bg = work + Jb.b_off;
@@ -2062,14 +1954,14 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
   };
-  const int l4 = ldb >> 2;  // float4 per column (ldb is a multiple of 32)
-  // one pair, one warp: column i of sA (squared norm na[i]) and column j of
-  // sB (nb_[j]), Q's columns qi and qj.  One dot product per pair: the
-  // rotation that zeroes the overlap g moves the squared norms to a - t g
-  // and b + t g, exactly in exact arithmetic; they are recomputed from the
-  // data whenever a block is loaded.
+  const int l4 = ld >> 2;  // float4 per column (ld is a multiple of 32)
+  // one pair, one warp, from shared memory: column i of sA (squared norm
+  // na[i]) and column j of sB (nb_[j]), Q's columns qi and qj.  One dot product
+  // per pair: the rotation that zeroes the overlap g moves the squared norms to
+  // a - t g and b + t g, exactly in exact arithmetic; they are recomputed from
+  // the data whenever a block is loaded.
   auto pair = [&](float *sA, float *na, int i, float *sB, float *nb_, int j, int qi, int qj, float &rmax) -> bool {
-    float4 *xp = reinterpret_cast<float4 *>(sA + i * ldb), *xq = reinterpret_cast<float4 *>(sB + j * ldb);
+    float4 *xp = reinterpret_cast<float4 *>(sA + i * ld), *xq = reinterpret_cast<float4 *>(sB + j * ld);
     float g = 0.f;
     for (int r = lane; r < l4; r += 32) {
       const float4 x = xp[r], y = xq[r];
@@ -2080,13 +1972,8 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
     }
     g = wsumf(g);
     const float a = na[i], b = nb_[j];
-    if (!(a > 0.f) || !(b > 0.f)) return false;
-    const float ratio = fabsf(g) / sqrtf(a) / sqrtf(b);
-    if (!(ratio > tol)) return false;
-    const float z = (b - a) / (2.0f * g);
-    const float t = z == 0.f ? 1.0f : copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
-    if (!(fabsf(t) >= FLT_MIN) || !isfinite(t)) return false;
-    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
+    float ratio, t, c, sn;
+    if (!js_rotation(a, b, g, tol, ratio, t, c, sn)) return false;
     for (int r = lane; r < l4; r += 32) {
       const float4 x = xp[r], y = xq[r];
       xp[r] = make_float4(c * x.x - sn * y.x, c * x.y - sn * y.y, c * x.z - sn * y.z, c * x.w - sn * y.w);
@@ -2108,23 +1995,6 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
     rmax = fmaxf(rmax, ratio);
     return true;
   };
-  // the intra-block pairs of one block in shared memory (round robin)
-  auto inner = [&](float *sb, float *nv_, int nv, int q0, bool &any, float &rmax) {
-    const int bp = bw + (bw & 1), half = bp / 2, bm = bp - 1;
-    for (int sr = 0; sr < bm; ++sr) {
-      for (int i = warp; i < half; i += nw) {
-        int p = 0, q;
-        if (i != 0) {
-          p = i - 1 + sr;
-          p = 1 + (p >= bm ? p - bm : p);
-        }
-        q = bp - 2 - i + sr;
-        q = 1 + (q >= bm ? q - bm : q);
-        if (p < nv && q < nv) any |= pair(sb, nv_, p, sb, nv_, q, q0 + p, q0 + q, rmax);
-      }
-      __syncthreads();
-    }
-  };
   bool converged = false;
   int sweep = 0;
   for (; sweep < 15 && !converged; ++sweep) {
@@ -2145,75 +2015,138 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
         const int b0 = bj_block_at(pi, rnd, P), b1 = bj_block_at(P - 1 - pi, rnd, P);
         const int nv0 = valid(b0), nv1 = valid(b1);
         if (nv0 == 0 && nv1 == 0) continue;  // uniform over the CTA
-        // load both blocks (rows >= nr and columns >= nv zero), Q = I
-        for (int e = threadIdx.x; e < bw * ldb; e += blockDim.x) {
-          const int j = e / ldb, r = e - j * ldb;
-          S0[e] = (j < nv0 && r < nr) ? __ldcg(B32 + (int64_t)(b0 * bw + j) * nr + r) : 0.0f;
-          S1[e] = (j < nv1 && r < nr) ? __ldcg(B32 + (int64_t)(b1 * bw + j) * nr + r) : 0.0f;
+        // load both blocks, a warp per column (rows >= nr and columns >= nv
+        // zero), with their squared norms; Q = I
+        for (int j = warp; j < 2 * bw; j += nw) {
+          const int jj = j < bw ? j : j - bw;
+          const bool ok = jj < (j < bw ? nv0 : nv1);
+          float *to = (j < bw ? S0 : S1) + jj * ld;
+          const float *from = B32 + (int64_t)((j < bw ? b0 : b1) * bw + jj) * nr;
+          float a = 0.f;
+#pragma unroll 4
+          for (int r = lane; r < ld; r += 32) {
+            const float u = (ok && r < nr) ? __ldcg(from + r) : 0.0f;
+            to[r] = u;
+            a = fmaf(u, u, a);
+          }
+          a = wsumf(a);
+          if (lane == 0) (j < bw ? N0 : N1)[jj] = a;
         }
         for (int e = threadIdx.x; e < qld * qd; e += blockDim.x) Q[e] = (e / qld == e % qld) ? 1.0f : 0.0f;
         __syncthreads();
-        for (int j = warp; j < 2 * bw; j += nw) {  // squared column norms
-          const float4 *x = reinterpret_cast<const float4 *>((j < bw ? S0 : S1) + (j < bw ? j : j - bw) * ldb);
-          float a = 0.f;
-          for (int r = lane; r < l4; r += 32) {
-            const float4 u = x[r];
-            a = fmaf(u.x, u.x, a);
-            a = fmaf(u.y, u.y, a);
-            a = fmaf(u.z, u.z, a);
-            a = fmaf(u.w, u.w, a);
-          }
-          a = wsumf(a);
-          if (lane == 0) (j < bw ? N0 : N1)[j < bw ? j : j - bw] = a;
-        }
-        __syncthreads();
         if (rnd == 0) {
-          inner(S0, N0, nv0, 0, any, rmax);
-          inner(S1, N1, nv1, bw, any, rmax);
+          // the pairs inside each block (round robin), both blocks at a time
+          const int bp = bw + (bw & 1), half = bp / 2, bm = bp - 1;
+          for (int sr = 0; sr < bm; ++sr) {
+            for (int ii = warp; ii < 2 * half; ii += nw) {
+              const int i = ii < half ? ii : ii - half;
+              int p = 0, q;
+              if (i != 0) {
+                p = i - 1 + sr;
+                p = 1 + (p >= bm ? p - bm : p);
+              }
+              q = bp - 2 - i + sr;
+              q = 1 + (q >= bm ? q - bm : q);
+              if (ii < half) {
+                if (p < nv0 && q < nv0) any |= pair(S0, N0, p, S0, N0, q, p, q, rmax);
+              } else {
+                if (p < nv1 && q < nv1) any |= pair(S1, N1, p, S1, N1, q, bw + p, bw + q, rmax);
+              }
+            }
+            __syncthreads();
+          }
         }
-        for (int sr = 0; sr < bw; ++sr) {
-          for (int i = warp; i < bw; i += nw) {
-            int j = i + sr;
+        if (R4 == 0) {
+          for (int sr = 0; sr < bw; ++sr) {
+            for (int i = warp; i < bw; i += nw) {
+              int j = i + sr;
+              if (j >= bw) j -= bw;
+              if (i < nv0 && j < nv1) any |= pair(S0, N0, i, S1, N1, j, i, bw + j, rmax);
+            }
+            __syncthreads();
+          }
+        } else {
+          constexpr int R = R4 > 0 ? R4 : 1;
+          const bool own = warp < nv0;  // (nw >= bw)
+          float4 *xp = reinterpret_cast<float4 *>(S0 + warp * ld);
+          float *qp = Q + warp * qld;
+          float4 x[R];
+          float a = 0.f, qx[2] = {0.f, 0.f};
+          if (own) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              x[q] = lane + 32 * q < l4 ? xp[lane + 32 * q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            a = N0[warp];
+            if (lane < qd) qx[0] = qp[lane];
+            if (lane + 32 < qd) qx[1] = qp[lane + 32];
+          }
+          for (int sr = 0; sr < bw; ++sr) {
+            int j = warp + sr;
             if (j >= bw) j -= bw;
-            if (i < nv0 && j < nv1) any |= pair(S0, N0, i, S1, N1, j, i, bw + j, rmax);
+            if (own && j < nv1) {
+              float4 *yp = reinterpret_cast<float4 *>(S1 + j * ld);
+              float4 y[R], d = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int q = 0; q < R; ++q)
+                y[q] = lane + 32 * q < l4 ? yp[lane + 32 * q] : make_float4(0.f, 0.f, 0.f, 0.f);
+              const float b = N1[j];
+#pragma unroll
+              for (int q = 0; q < R; ++q) {
+                d.x = fmaf(x[q].x, y[q].x, d.x);
+                d.y = fmaf(x[q].y, y[q].y, d.y);
+                d.z = fmaf(x[q].z, y[q].z, d.z);
+                d.w = fmaf(x[q].w, y[q].w, d.w);
+              }
+              const float g = wsumf((d.x + d.y) + (d.z + d.w));
+              float ratio, t, c, sn;
+              if (js_rotation(a, b, g, tol, ratio, t, c, sn)) {
+                any = true;
+                rmax = fmaxf(rmax, ratio);
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                  const float4 u = x[q], w = y[q];
+                  x[q] = make_float4(c * u.x - sn * w.x, c * u.y - sn * w.y, c * u.z - sn * w.z, c * u.w - sn * w.w);
+                  if (lane + 32 * q < l4)
+                    yp[lane + 32 * q] = make_float4(fmaf(sn, u.x, c * w.x), fmaf(sn, u.y, c * w.y),
+                                                    fmaf(sn, u.z, c * w.z), fmaf(sn, u.w, c * w.w));
+                }
+                float *cq = Q + (bw + j) * qld;
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                  if (lane + 32 * q < qd) {
+                    const float u = qx[q], w = cq[lane + 32 * q];
+                    qx[q] = c * u - sn * w;
+                    cq[lane + 32 * q] = fmaf(sn, u, c * w);
+                  }
+                a = fmaxf(a - t * g, 0.f);
+                if (lane == 0) N1[j] = fmaxf(b + t * g, 0.f);
+              }
+            }
+            __syncthreads();
+          }
+          if (own) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              if (lane + 32 * q < l4) xp[lane + 32 * q] = x[q];
+            if (lane < qd) qp[lane] = qx[0];
+            if (lane + 32 < qd) qp[lane + 32] = qx[1];
           }
           __syncthreads();
         }
-        // blocks back; V's columns of the two blocks times Q, one row per
-        // thread (x[r]: V's entry in the column of Q's row r)
-        for (int e = threadIdx.x; e < bw * ldb; e += blockDim.x) {
-          const int j = e / ldb, r = e - j * ldb;
-          if (r < nr) {
-            if (j < nv0) B32[(int64_t)(b0 * bw + j) * nr + r] = S0[e];
-            if (j < nv1) B32[(int64_t)(b1 * bw + j) * nr + r] = S1[e];
-          }
+        // blocks back, V's columns of the two blocks times Q
+        for (int j = warp; j < 2 * bw; j += nw) {
+          const int jj = j < bw ? j : j - bw;
+          if (jj >= (j < bw ? nv0 : nv1)) continue;
+          const float *from = (j < bw ? S0 : S1) + jj * ld;
+          float *to = B32 + (int64_t)((j < bw ? b0 : b1) * bw + jj) * nr;
+          for (int r = lane; r < nr; r += 32) to[r] = from[r];
         }
-        for (int row = threadIdx.x; row < n; row += blockDim.x) {
-          float x[2 * JS_BW_MAX];
-#pragma unroll
-          for (int r = 0; r < 2 * JS_BW_MAX; ++r) {
-            const bool first = r < bw;
-            const int lc = first ? r : r - bw, nv = first ? nv0 : nv1, bb = first ? b0 : b1;
-            x[r] = (r < qd && lc < nv) ? __ldcg(V32 + (int64_t)(bb * bw + lc) * n + row) : 0.0f;
-          }
-#pragma unroll 1
-          for (int oc = 0; oc < qd; ++oc) {
-            const bool first = oc < bw;
-            const int lo = first ? oc : oc - bw, nv = first ? nv0 : nv1, bb = first ? b0 : b1;
-            if (lo >= nv) continue;
-            const float4 *qc = reinterpret_cast<const float4 *>(Q + oc * qld);
-            float acc = 0.f;
-#pragma unroll
-            for (int r4 = 0; r4 < (2 * JS_BW_MAX) / 4; ++r4)
-              if (4 * r4 < qd) {
-                const float4 w = qc[r4];
-                acc = fmaf(x[4 * r4], w.x, acc);
-                acc = fmaf(x[4 * r4 + 1], w.y, acc);
-                acc = fmaf(x[4 * r4 + 2], w.z, acc);
-                acc = fmaf(x[4 * r4 + 3], w.w, acc);
-              }
-            V32[(int64_t)(bb * bw + lo) * n + row] = acc;
-          }
+        switch ((qd + 7) / 8) {
+          case 1: js_apply_q<8>(V32, n, Q, bw, b0, nv0, b1, nv1); break;
+          case 2: js_apply_q<16>(V32, n, Q, bw, b0, nv0, b1, nv1); break;
+          case 3: js_apply_q<24>(V32, n, Q, bw, b0, nv0, b1, nv1); break;
+          case 4: js_apply_q<32>(V32, n, Q, bw, b0, nv0, b1, nv1); break;
+          default: js_apply_q<40>(V32, n, Q, bw, b0, nv0, b1, nv1);
         }
         __syncthreads();
       }
@@ -2673,24 +2606,41 @@ static cudaError_t launch_block32_clusters(const SvdJob *jobs, const int *order,
   return cudaLaunchKernelEx(&cfg, jacobi32_block_kernel, jobs, order, work, iwork);
 }
 
-// shared memory of jacobi32_big_kernel for sectors of up to `cols` columns,
-// and whether such sectors fit it
-static size_t big32_smem(int cols) {
-  const int64_t bw = (cols + 31) / 32, ld = 32 * (((int64_t)cols + 31) / 32);
-  return (size_t)(4 * ((bw * ld + 3) & ~(int64_t)3) * sizeof(float));
-}
-static bool big32_fits(int cols) {
-  return 32 * (((int64_t)cols + 31) / 32) <= 32 * J32B_REG && big32_smem(cols) <= SVD_BLOCK_SMEM_MAX;
-}
-
-int svd_jacobi32_big_max_cols() {
-  int c = 32 * J32B_REG;
-  while (c > 0 && !big32_fits(c)) --c;
-  return c;
+// jacobi32_stream_kernel on the jobs order[0 .. njobs) of at most `cols` columns
+static cudaError_t launch_jacobi32_stream(const SvdJob *jobs, const int *order, int njobs, int cols, int csize,
+                                          double *work, const int *iwork, cudaStream_t st) {
+  const int ldb = 32 * ((cols + 31) / 32);
+  const int64_t budget = 200 * 1024 / (int)sizeof(float);
+  int bw_cap = std::min(JS_BW_MAX, (cols + 2 * csize - 1) / (2 * csize));
+  while (bw_cap >= 1 && js_smem_floats(bw_cap, ldb) > budget) --bw_cap;
+  if (bw_cap < 1) return cudaErrorInvalidValue;
+  // registers per column: 128 rows each
+  auto kern = ldb <= 384   ? jacobi32_stream_kernel<3>
+              : ldb <= 640 ? jacobi32_stream_kernel<5>
+              : ldb <= 896 ? jacobi32_stream_kernel<7>
+              : ldb <= 1280 ? jacobi32_stream_kernel<10>
+                            : jacobi32_stream_kernel<0>;
+  const size_t smem = (size_t)js_smem_floats(bw_cap, ldb) * sizeof(float);
+  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(njobs * csize, 1, 1);
+  cfg.blockDim = dim3(32 * std::max(bw_cap, 8), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, jobs, order, work, iwork, bw_cap, ldb);
 }
 
 cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs, const int *g, const int *cols,
-                                int cols0, int g0b, int cols0b, double *work, const int *iwork, cudaStream_t st,
+                                int cols0, double *work, const int *iwork, cudaStream_t st,
                                 const cudaStream_t *side, const cudaEvent_t *ev) {
   if (njobs <= 0) return cudaGetLastError();
   cudaFuncSetAttribute(jacobi32_block_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -2710,81 +2660,18 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
     e = cudaEventRecord(ev[k - 1], side[k - 2]);
     if (e != cudaSuccess) return e;
   }
-  // beyond the block kernels (jobs 0 .. g[0], largest first): the jobs from
-  // g0b on (at most cols0b columns) on jacobi32_big_kernel (B's columns in
-  // shared memory, the rotations in global memory) on side stream 3,
-  // concurrently with the larger ones on the all-global kernel; every job
-  // on the all-global kernel if 16-CTA clusters or the shared memory are
-  // not available
-  bool big_on_side = false;
-  int nglob = hi[0];
+  // beyond the block kernels: the block tournament streamed through shared
+  // memory; the all-global pair kernel if asked for, or if that launch is not
+  // possible (no 16-CTA clusters)
   if (hi[0] > lo[0]) {
-    const int split = g0b < 0 ? 0 : (g0b > hi[0] ? hi[0] : g0b);
-    const int bcols = split == 0 ? cols0 : cols0b;
-    if (split < hi[0] && big32_fits(bcols)) {
-      const size_t smem0 = big32_smem(bcols);
-      cudaFuncSetAttribute(jacobi32_big_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      e = cudaFuncSetAttribute(jacobi32_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(side[3], ev[0], 0);
-      if (e == cudaSuccess) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((hi[0] - split) * 16, 1, 1);
-        cfg.blockDim = dim3(BJ_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = smem0;
-        cfg.stream = side[3];
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 16;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, jacobi32_big_kernel, jobs, order + split, work, iwork);
-      }
-      if (e == cudaSuccess) e = cudaEventRecord(ev[4], side[3]);
-      if (e == cudaSuccess) {
-        big_on_side = true;
-        nglob = split;
-      } else {
-        cudaGetLastError();
-      }
-    }
-  }
-  if (nglob > 0) {
-    // the block tournament streamed through shared memory; the all-global
-    // pair kernel if that launch is not possible
-    const int ldb0 = 32 * ((cols0 + 31) / 32);
-    const int64_t budget = 200 * 1024 / (int)sizeof(float);
-    int bw_cap = JS_BW_MAX;
-    while (bw_cap >= 1 && js_smem_floats(bw_cap, ldb0) > budget) --bw_cap;
-    e = cudaErrorInvalidValue;
-    if (bw_cap >= 1) {
-      const size_t smem = (size_t)js_smem_floats(bw_cap, ldb0) * sizeof(float);
-      cudaFuncSetAttribute(jacobi32_stream_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      e = cudaFuncSetAttribute(jacobi32_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(nglob * 16, 1, 1);
-        cfg.blockDim = dim3(JS_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 16;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, jacobi32_stream_kernel, jobs, order, work, iwork, bw_cap, ldb0);
-      }
-    }
+    e = launch_jacobi32_stream(jobs, order, hi[0], cols0, 16, work, iwork, st);
     if (e != cudaSuccess) {
       cudaGetLastError();
       cudaFuncSetAttribute(jacobi32_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      e = launch_jacobi32_clusters(jobs, order, nglob, 16, work, iwork, st);
+      e = launch_jacobi32_clusters(jobs, order, hi[0], 16, work, iwork, st);
       if (e != cudaSuccess) {
         cudaGetLastError();
-        e = launch_jacobi32_clusters(jobs, order, nglob, 8, work, iwork, st);
+        e = launch_jacobi32_clusters(jobs, order, hi[0], 8, work, iwork, st);
       }
     }
     if (e != cudaSuccess) return e;
@@ -2796,10 +2683,6 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
   for (int k = 2; k < 5; ++k) {
     if (hi[k] <= lo[k]) continue;
     e = cudaStreamWaitEvent(st, ev[k - 1], 0);
-    if (e != cudaSuccess) return e;
-  }
-  if (big_on_side) {
-    e = cudaStreamWaitEvent(st, ev[4], 0);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
