@@ -430,8 +430,9 @@ idmrg_status idmrg_set_svd_path(idmrg_ctx *ctx, int global_only);
 idmrg_status idmrg_set_jacobi_arithmetic(idmrg_ctx *ctx, int mode);
 
 /* Shape of the last truncation's SVD work (Step 4): sector matrices, their
- * largest short side, largest numerical rank, and the Jacobi sweeps taken
- * (maximum and mean over the sectors). */
+ * largest short side, largest numerical rank, and the sweeps of the final
+ * Jacobi (maximum and mean over the sectors; 0 in a sector whose columns the
+ * refinement before it left orthogonal to the Jacobi's own threshold). */
 idmrg_status idmrg_svd_stats(const idmrg_ctx *ctx, int *jobs, int *max_cols, int *max_rank, int *max_sweeps,
                              double *mean_sweeps);
 

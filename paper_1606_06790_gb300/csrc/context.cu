@@ -328,9 +328,13 @@ struct idmrg_ctx {
   int tiw = 0, tsv = 0, tentries_max = 1, tmaxcols = 0;
   // FP32-preconditioned Jacobi: G = V^T V, W = V G (Newton-Schulz), X = B V
   GemmList svdG, svdW, svdX;
+  // refinement (sectors of SVD_REFINE_MIN columns on): G = Xs^T Xs, V^T V, As^2, V T, Xs Ts
+  GemmList svdH, svdR, svdK, svdV, svdT;
+  DevBuf dshk, dshs, dsrk, dsrs, dskk, dsks, dsvk, dsvs, dstk, dsts;
   DevBuf dsgk, dsgs, dswk, dsws, dsxk, dsxs;
   // device side of every grouped-GEMM list
-  GemmDev gd_g1, gd_g3, gd_gp, gd_env1, gd_env3, gd_svdG, gd_svdW, gd_svdX;
+  GemmDev gd_g1, gd_g3, gd_gp, gd_env1, gd_env3, gd_svdG, gd_svdW, gd_svdX, gd_svdH, gd_svdR, gd_svdK,
+      gd_svdV, gd_svdT;
   int64_t tmaxel_all = 0;
 
   int svd_jobs = 0, svd_max_cols = 0, svd_max_rank = 0, svd_max_sweeps = 0;
@@ -2153,8 +2157,10 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
       work += J.cols_a;
       J.w_off = work;
       work += (int64_t)J.cols_a * J.cols_a;
+      J.t_off = work;
+      if (J.cols_a >= SVD_REFINE_MIN) work += (int64_t)J.cols_a * J.cols_a;
       J.perm_off = iw;
-      iw += J.cols_a + 3;  // permutation, rank, FP64 and FP32 Jacobi sweeps
+      iw += J.cols_a + 4;  // permutation, rank, FP64 and FP32 Jacobi sweeps, final Jacobi to run
       J.sv_off = sv;
       sv += J.cols_a;
       entries += J.cols_a;
@@ -2195,6 +2201,7 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
   c->svdG.clear();
   c->svdW.clear();
   c->svdX.clear();
+  for (GemmList *l : {&c->svdH, &c->svdR, &c->svdK, &c->svdV, &c->svdT}) l->clear();
   c->tmaxcols = 0;
   for (const SvdJob &J : c->jobs) {
     const int ca = J.cols_a;
@@ -2205,6 +2212,16 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
     c->svdW.seg(BUF_SVD, J.x_off, ca, BUF_SVD, J.j_off, ca, ca, 0);
     c->svdX.task(J.sb, BUF_SVD, J.w_off, ca, ca, ca);
     c->svdX.seg(BUF_SVD, J.j_off, ca, BUF_SVD, J.b_off, ca, ca, 0);
+    if (ca < SVD_REFINE_MIN) continue;
+    auto product = [&](GemmList &l, int64_t out, int64_t a, int64_t b, int flags) {
+      l.task(J.sb, BUF_SVD, out, ca, ca, ca);
+      l.seg(BUF_SVD, a, ca, BUF_SVD, b, ca, ca, flags);
+    };
+    product(c->svdH, J.x_off, J.b_off, J.b_off, 2);
+    product(c->svdR, J.t_off, J.j_off, J.j_off, 2);
+    product(c->svdK, J.t_off, J.w_off, J.w_off, 0);
+    product(c->svdV, J.x_off, J.t_off, J.j_off, 0);
+    product(c->svdT, J.x_off, J.w_off, J.b_off, 0);
   }
   NOMEM(c->ensure(c->siw, 4 * std::max(iw, 1)));
   NOMEM(c->upload(c->sjobs, c->jobs) && c->ensure(c->swork, 8 * std::max<int64_t>(work, 1)) &&
@@ -2215,7 +2232,13 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
         c->ensure(c->slamk, 8 * (size_t)P * std::max(1, c->o.m)));
   for (auto [L, dk, ds, T] : {std::make_tuple(&c->svdG, &c->dsgk, &c->dsgs, &c->gd_svdG),
                                std::make_tuple(&c->svdW, &c->dswk, &c->dsws, &c->gd_svdW),
-                               std::make_tuple(&c->svdX, &c->dsxk, &c->dsxs, &c->gd_svdX)}) {
+                               std::make_tuple(&c->svdX, &c->dsxk, &c->dsxs, &c->gd_svdX),
+                               std::make_tuple(&c->svdH, &c->dshk, &c->dshs, &c->gd_svdH),
+                               std::make_tuple(&c->svdR, &c->dsrk, &c->dsrs, &c->gd_svdR),
+                               std::make_tuple(&c->svdK, &c->dskk, &c->dsks, &c->gd_svdK),
+                               std::make_tuple(&c->svdV, &c->dsvk, &c->dsvs, &c->gd_svdV),
+                               std::make_tuple(&c->svdT, &c->dstk, &c->dsts, &c->gd_svdT)}) {
+    if (L->tasks.empty()) continue;  // (no refined sector)
     idmrg_status sg = gemm_upload(c, *L, *dk, *ds, *T);
     if (sg != IDMRG_OK) return sg;
   }
@@ -2343,6 +2366,45 @@ void svd_stats_reset(idmrg_ctx *c) {
   c->svd_jobs32 = 0;
 }
 
+// Two correction steps for the sectors of SVD_REFINE_MIN columns on, and the
+// check that decides which of them the final Jacobi still has to sweep (see
+// the refinement in kernels_svd.cu).
+idmrg_status svd_refine(idmrg_ctx *c) {
+  if (c->svdH.tasks.empty()) return IDMRG_OK;
+  int nref = 0;  // torder lists the largest sectors first
+  while (nref < (int)c->torder.size() && c->jobs[c->torder[nref]].cols_a >= SVD_REFINE_MIN) ++nref;
+  auto part = [&](SvdRefine what) {
+    c->launches += 1;
+    return launch_svd_refine(what, (const SvdJob *)c->sjobs.p, (const int *)c->sorder.p, nref, c->tmaxcols,
+                             c->dp(c->swork), (int *)c->siw.p, c->dp(c->ssv), c->st);
+  };
+#define REF_GEMM(x, k, s)                                    \
+  do {                                                       \
+    const idmrg_status s_ = gemm_run(c, c->x, c->k, c->s, nullptr); \
+    if (s_ != IDMRG_OK) return s_;                           \
+  } while (0)
+  CK(part(REF_SCALE));
+  for (int step = 0; step < 2; ++step) {
+    REF_GEMM(gd_svdH, dshk, dshs);
+    if (step == 0) {
+      CK(part(REF_BUILD));
+    } else {
+      REF_GEMM(gd_svdR, dsrk, dsrs);
+      CK(part(REF_BUILD_R));
+    }
+    REF_GEMM(gd_svdK, dskk, dsks);
+    CK(part(REF_FINISH));
+    REF_GEMM(gd_svdV, dsvk, dsvs);
+    CK(part(REF_PUT_V));
+    REF_GEMM(gd_svdT, dstk, dsts);
+    CK(part(REF_PUT_X));
+  }
+  REF_GEMM(gd_svdH, dshk, dshs);
+  CK(part(REF_CHECK));
+#undef REF_GEMM
+  return IDMRG_OK;
+}
+
 idmrg_status truncate(idmrg_ctx *c, int p) {
   const int P = c->P;
   for (int q = 0; q < P; ++q)
@@ -2382,7 +2444,7 @@ idmrg_status truncate(idmrg_ctx *c, int p) {
   double *const *svb = (double *const *)c->dbufs.p;
   c->kend(PH + 0);
   c->kbegin(PH + 1);
-  CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 0, sw, c->st));
+  CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 0, sw, (int *)c->siw.p, c->st));
   CK(launch_svd_jacobi32(dj, (const int *)c->sorder.p, nj, g, gcols, cols0, sw, (const int *)c->siw.p, c->st,
                          c->side, c->sev));
   c->kend(PH + 1);
@@ -2396,13 +2458,17 @@ idmrg_status truncate(idmrg_ctx *c, int p) {
     idmrg_status sg_ = gemm_run(c, c->gd_svdW, c->dswk, c->dsws, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
-    CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 1, sw, c->st));
+    CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 1, sw, (int *)c->siw.p, c->st));
   }
   {
     idmrg_status sg_ = gemm_run(c, c->gd_svdX, c->dsxk, c->dsxs, nullptr);
     if (sg_ != IDMRG_OK) return sg_;
   }
-  CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 2, sw, c->st));
+  CK(launch_svd_elementwise(dj, nj, c->tmaxcols, 2, sw, (int *)c->siw.p, c->st));
+  {
+    const idmrg_status s = svd_refine(c);
+    if (s != IDMRG_OK) return s;
+  }
   c->kend(PH + 2);
   c->kbegin(PH + 3);
   CK(launch_svd_jacobi(dj, (const int *)c->sorder.p, nj, g, gcols, sw, (int *)c->siw.p, c->dp(c->ssv),
@@ -3462,7 +3528,9 @@ idmrg_status idmrg_create_batch(const idmrg_mpo *mpos, int nmpo, const int *m_pe
     return bail(IDMRG_EINVAL);
   c->mixed = opts->prec == IDMRG_TF32X3 || opts->prec == IDMRG_BF16X3;
   c->fp64tc = opts->prec == IDMRG_FP64_TC;
-  for (GemmDev *t : {&c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX}) t->oz_use = true;
+  for (GemmDev *t : {&c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX,
+                     &c->gd_svdH, &c->gd_svdR, &c->gd_svdK, &c->gd_svdV, &c->gd_svdT})
+    t->oz_use = true;
   c->bf16 = opts->prec == IDMRG_BF16X3 ? 1 : 0;
   c->inner_factor = c->bf16 ? 1e-2 : 1e-3;
   c->d = d;
@@ -3626,7 +3694,8 @@ void idmrg_destroy(idmrg_ctx *c) {
                     &c->lconv, &c->ltheta, &c->ly, &c->lresid, &c->lpsi, &c->lv0, &c->ldot, &c->sjobs, &c->swork,
                     &c->ssv, &c->sjob0, &c->snjob, &c->skpj, &c->sperm, &c->slam, &c->seps, &c->sepsb, &c->skept,
                     &c->scj, &c->slamk, &c->siw, &c->sorder, &c->sorderq, &c->dsgk, &c->dsgs,
-                    &c->dswk, &c->dsws, &c->dsxk, &c->dsxs, &c->dpkL, &c->dtune_out, &c->dmsb,
+                    &c->dswk, &c->dsws, &c->dsxk, &c->dsxs, &c->dshk, &c->dshs, &c->dsrk, &c->dsrs, &c->dskk, &c->dsks,
+                    &c->dsvk, &c->dsvs, &c->dstk, &c->dsts, &c->dpkL, &c->dtune_out, &c->dmsb,
                     &c->dwtp, &c->dwtpm, &c->dwunits, &c->dtarget, &c->oz_step_w.dsegs, &c->oz_step_w.dunits, &c->oz_step_p.dsegs,
                     &c->oz_step_p.dunits, &c->oz_psi.dsegs, &c->oz_psi.dunits, &c->dozwu, &c->dozkeep,
                     &c->doz1k,
@@ -3654,7 +3723,8 @@ void idmrg_destroy(idmrg_ctx *c) {
   for (cudaStream_t x : c->side)
     if (x) cudaStreamDestroy(x);
   if (c->pin_act) cudaFreeHost(c->pin_act);
-  for (GemmDev *t : {&c->gd_g1, &c->gd_g3, &c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX}) {
+  for (GemmDev *t : {&c->gd_g1, &c->gd_g3, &c->gd_gp, &c->gd_env1, &c->gd_env3, &c->gd_svdG, &c->gd_svdW, &c->gd_svdX,
+                     &c->gd_svdH, &c->gd_svdR, &c->gd_svdK, &c->gd_svdV, &c->gd_svdT}) {
     rel(t->tiles);
     rel(t->oz.pack.dsegs);
     rel(t->oz.pack.dunits);

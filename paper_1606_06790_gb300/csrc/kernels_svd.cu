@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(JAC_THREADS, 2)
   const int np = n + (n & 1);
   int *flag0 = cluster.map_shared_rank(&flag, 0);
   int *rmax0 = cluster.map_shared_rank(&cl_rmax, 0);
-  bool converged = (n < 2);
+  bool converged = n < 2 || iwork[Jb.perm_off + Jb.cols_a + 3] == 0;  // nothing to rotate: see refinement
   int sweep = 0;
   for (; sweep < 40 && !converged; ++sweep) {
     if (threadIdx.x == 0) {
@@ -1071,7 +1071,7 @@ __global__ void __launch_bounds__(BJ_THREADS, 2)
   const Split floor_split = split_f64(4.0 * DBL_EPSILON * DBL_EPSILON * fro);
   int *flag0 = cluster.map_shared_rank(&flag, 0);
   int *lmax0 = cluster.map_shared_rank(&cl_lmax, 0);
-  bool converged = (n < 2);
+  bool converged = n < 2 || iwork[Jb.perm_off + Jb.cols_a + 3] == 0;  // nothing to rotate: see refinement
   // Cyclic Jacobi converges quadratically at the end: after a sweep in which
   // no rotation exceeded |g| / sqrt(a b) = r = 1e-9, every pair is left with
   // an overlap of order n r^2 <= 1e-15 relative, below the threshold
@@ -1392,6 +1392,21 @@ __global__ void __launch_bounds__(JAC_THREADS, 1)
     cluster.sync();
     for (int64_t e = e0; e < nn; e += stride) Jm[e] = tmp[e];
   }
+  if (n >= 2 && iwork[Jb.perm_off + Jb.cols_a + 3] == 0) {  // no overlap left (see refinement): norms only, in FP64
+    for (int j = gw; j < Jb.cols_a; j += gnw) {
+      double *bj = B + (int64_t)j * nr;
+      double s = 0.0;
+      if (j < n)
+        for (int i = lane; i < nr; i += 32) s = fma(bj[i], bj[i], s);
+      s = sqrt(wsum(s));
+      if (lane == 0) sv[Jb.sv_off + j] = s;
+      const double inv = s > 0.0 ? 1.0 / s : 0.0;
+      if (j < n)
+        for (int i = lane; i < nr; i += 32) bj[i] *= inv;
+    }
+    if (crank == 0 && threadIdx.x == 0) iwork[Jb.perm_off + Jb.cols_a + 1] = 0;
+    return;  // (uniform over the cluster)
+  }
   for (int64_t e = e0; e < n; e += stride) dsc[e] = 1.0;
   double fro = 0.0;
   for (int64_t e = e0; e < nb; e += stride) {
@@ -1453,7 +1468,7 @@ __global__ void __launch_bounds__(JAC_THREADS, 1)
     }
     cluster.sync();
   };
-  bool converged = (n < 2);
+  bool converged = n < 2 || iwork[Jb.perm_off + Jb.cols_a + 3] == 0;  // nothing to rotate: see refinement
   int sweep = 0;
   for (; sweep < 40 && !converged; ++sweep) {
     fold();
@@ -2173,9 +2188,11 @@ __global__ void __launch_bounds__(JS_THREADS, 1)
 }
 
 // per job over cols_a x cols_a elements: 0 V = I, 1 V = 1.5 V - 0.5 W, 2 B = X
-__global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *__restrict__ work, int mode) {
+__global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *__restrict__ work,
+                                       int *__restrict__ iwork, int mode) {
   const SvdJob J = jobs[blockIdx.y];
   const int ca = J.cols_a;
+  if (mode == 0 && blockIdx.x == 0 && threadIdx.x == 0) iwork[J.perm_off + ca + 3] = 1;
   const int64_t tot = (int64_t)ca * ca;
   double *V = work + J.j_off, *W = work + J.w_off, *B = work + J.b_off;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
@@ -2186,6 +2203,175 @@ __global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *
     else
       B[e] = W[e];
   }
+}
+
+// ------------------------------------------------------------ refinement
+// After the FP32 stage, Newton-Schulz and X = B V, the columns of X overlap by
+// about 1e-6 of their norms (more where sigma is so small that the rounding of
+// X shows), and the final Jacobi would need two to three sweeps: one that
+// rotates by these overlaps, and one or two that find next to nothing left.
+// A correction takes all overlaps to second order at once, by matrix products
+// (Ogita and Aishima, "Iterative refinement for symmetric eigenvalue
+// decomposition", Japan J. Indust. Appl. Math. 35, 2018, for eigenvectors): with
+// D the column norms, X = Xs D, G = Xs^T Xs, b_i = D_i^2 G_ii, R = V^T V - 1 and
+//   A = K - R / 2,  K_ij = (G_ij D_i D_j - R_ij (b_i + b_j) / 2) / (b_j - b_i),
+// X' = X (1 + A + A^2 / 2) and V' = V (1 + A + A^2 / 2) have overlaps of order
+// K G, and with R = 0 the factor is orthogonal to K^4 / 4.  The first step (R is
+// rounding) takes pairs of |K| <= 2e-2: few sectors have nearer
+// singular values than that.  It leaves overlaps of 1e-8 at most and V
+// orthogonal to 4e-8; the second one, with R and |K| <= 1e-4, takes both to
+// rounding.  What they reach is then checked (REF_CHECK): a sector in which some
+// pair is still above the threshold of the FP64 Jacobi goes through the final
+// Jacobi's sweeps as before, the others only have their norms taken.
+// The spectra are graded over up to 13 decades, and overlaps must shrink
+// relative to their own columns: X is corrected in the scaled form
+// Xs' = Xs (1 + As + As^2 / 2), As = D A D^-1, whose entries are of the size of
+// the overlaps (Ks_ij ~ -G_ij for D_i >> D_j, vanishing for D_i << D_j), so that
+// the products' rounding stays relative to every column; R, whose rounding would
+// not, is used where D_i and D_j are within a factor of 4, or of 64 if it stands
+// out of the rounding.
+// All matrices lie transposed (row j belongs to column j of X): G and the
+// results in x_off, As^T and then (1 + As + As^2/2)^T in w_off, V^T V, (As^2)^T
+// and then (1 + A + A^2/2)^T in t_off, D in the job's singular values.
+// Measured (GB300, ms of a step; before -> now, the ten products included):
+// final Jacobi 39.8 -> 6.1 and Newton-Schulz to check 1.2 -> 4.1 for the J1-J2
+// cylinder at m = 1024, 55.8 -> 6.0 and 1.7 -> 5.6 for kagome at m = 1000, 13.2 ->
+// 0.8 and 0.5 -> 1.6 for J1-J2 at m = 500; sectors below SVD_REFINE_MIN columns
+// (2.7 -> 0.9 against 0.3 -> 1.0 for the chain at m = 256, half of whose sectors
+// are refined) gain less than the launches cost.
+constexpr float REF_KMAX = 2e-2f, REF_KMAX_R = 1e-4f;
+
+// column norms of X and Xs = X / D (rows of the transposed X at b_off, one
+// warp each; columns past the rank become zero)
+__global__ void __launch_bounds__(256) refine_scale_kernel(const SvdJob *__restrict__ jobs,
+                                                           const int *__restrict__ order, double *__restrict__ work,
+                                                           int *__restrict__ iwork, double *__restrict__ sv) {
+  const SvdJob J = jobs[order[blockIdx.y]];
+  const int ca = J.cols_a, n = iwork[J.perm_off + ca], lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) iwork[J.perm_off + ca + 3] = 0;
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= ca) return;
+  double *x = work + J.b_off + (int64_t)j * ca;
+  double s = 0.0;
+  if (j < n)
+    for (int i = lane; i < ca; i += 32) s = fma(x[i], x[i], s);
+  s = sqrt(wsum(s));
+  const double inv = s > 0.0 ? 1.0 / s : 0.0;
+  for (int i = lane; i < ca; i += 32) x[i] = s > 0.0 ? x[i] * inv : 0.0;
+  if (lane == 0) sv[J.sv_off + j] = s;
+}
+
+// The pairs (i, j), i <= j, of one 32 x 32 tile (rows j of the transposed
+// matrices, tile (tj, ti) with ti <= tj) and their mirror images: reads and
+// writes of both tiles coalesced, the mirrored one through shared memory.
+//   REF_BUILD  : G -> As^T (w), R = 0
+//   REF_BUILD_R: G, V^T V (t) -> As^T (w)
+//   REF_FINISH : As^T (w), (As^2)^T (t) -> the two correction factors
+//   REF_CHECK  : G -> is any overlap above the FP64 Jacobi's threshold
+template <int PART>
+__global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restrict__ jobs,
+                                                          const int *__restrict__ order, double *__restrict__ work,
+                                                          int *__restrict__ iwork, const double *__restrict__ sv) {
+  __shared__ double m1[32][33], m2[32][33];
+  const SvdJob J = jobs[order[blockIdx.y]];
+  const int ca = J.cols_a, n = iwork[J.perm_off + ca];
+  // tile (tj, ti), ti <= tj, number tj (tj + 1) / 2 + ti
+  int tj = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+  while ((tj + 1) * (tj + 2) / 2 <= (int)blockIdx.x) ++tj;
+  while (tj * (tj + 1) / 2 > (int)blockIdx.x) --tj;
+  const int ti = (int)blockIdx.x - tj * (tj + 1) / 2;
+  if (32 * tj >= ca) return;
+  const double *G = work + J.x_off;
+  double *w = work + J.w_off, *t = work + J.t_off;
+  const double *D = sv + J.sv_off;
+  const int c = threadIdx.x & 31, r8 = threadIdx.x >> 5;
+  auto at = [&](int row, int col) { return (int64_t)row * ca + col; };
+  if (PART == REF_FINISH) {  // the mirrored tiles
+    for (int r = r8; r < 32; r += 8) {
+      const int row = 32 * ti + r, col = 32 * tj + c;
+      m1[r][c] = row < ca && col < ca ? w[at(row, col)] : 0.0;
+      m2[r][c] = row < ca && col < ca ? t[at(row, col)] : 0.0;
+    }
+    __syncthreads();
+  }
+  bool bad = false;
+  for (int r = r8; r < 32; r += 8) {
+    const int j = 32 * tj + r, i = 32 * ti + c;
+    double a1 = 0.0, a2 = 0.0;  // mirrored values: element (i, j)
+    if (j < ca && i <= j) {
+      const double Di = D[i], Dj = D[j];
+      const double inv_i = Di > 0.0 ? 1.0 / Di : 0.0, inv_j = Dj > 0.0 ? 1.0 / Dj : 0.0;
+      if (PART == REF_FINISH) {
+        // p, q: As at (i, j), (j, i); s, u: its square
+        const double p = w[at(j, i)], q = m1[c][r], s = t[at(j, i)], u = m2[c][r];
+        if (i == j) {
+          w[at(j, j)] = t[at(j, j)] = 1.0 + fma(0.5, s, p);
+        } else {
+          // A^2 from the triangle in which As^2 carries all digits
+          const double h = 0.5 * (Di >= Dj ? s * (Dj * inv_i) : u * (Di * inv_j));
+          w[at(j, i)] = fma(0.5, s, p);
+          a1 = fma(0.5, u, q);
+          t[at(j, i)] = fma(p, Dj * inv_i, h);
+          a2 = fma(q, Di * inv_j, h);
+        }
+      } else if (PART == REF_CHECK) {
+        // bj_rotation's own test: relative overlap above sqrt(rows) 2^-52 (and
+        // g above its floor 4 eps^2 ||X||^2)
+        const double g = G[at(j, i)];
+        if (j < n && i < j)
+          bad |= !(fabsf((float)g) <= 0x1p-52f * sqrtf((float)ca)) &&
+                 fabs(g) * Di * Dj > 4.0 * DBL_EPSILON * DBL_EPSILON * D[0] * D[0];
+      } else {
+        double k = 0.0, h = 0.0;  // K_ij, R_ij / 2
+        if (j < n && Di > 0.0 && Dj > 0.0) {
+          if (PART == REF_BUILD_R) {
+            h = 0.5 * (i == j ? t[at(j, j)] - 1.0 : t[at(j, i)]);
+            const double hi = fmax(Di, Dj), lo = fmin(Di, Dj);
+            if (!(hi < 4.0 * lo) && !(hi < 64.0 * lo && fabs(h) > 0.5e-15)) h = 0.0;
+          }
+          if (i < j) {
+            const double bi = Di * Di * G[at(i, i)], bj = Dj * Dj * G[at(j, j)];
+            const double num = G[at(j, i)] * (Di * Dj) - h * (bi + bj);
+            // FP32 is enough for the angle (a relative error of K leaves that
+            // part of the overlap); both triangles use the same rounded value
+            const float kf = __fdividef((float)num, (float)(bj - bi));
+            if (fabsf(kf) <= (PART == REF_BUILD ? REF_KMAX : REF_KMAX_R)) k = (double)kf;
+          }
+        }
+        w[at(j, i)] = (k - h) * (Di * inv_j);
+        a1 = (-k - h) * (Dj * inv_i);
+      }
+    }
+    if (PART != REF_CHECK) {  // (an element of the mirrored tile is read above by this thread only)
+      m1[c][r] = a1;
+      if (PART == REF_FINISH) m2[c][r] = a2;
+    }
+  }
+  if (PART == REF_CHECK) {
+    if (bad) iwork[J.perm_off + ca + 3] = 1;
+    return;
+  }
+  __syncthreads();
+  for (int r = r8; r < 32; r += 8) {
+    const int row = 32 * ti + r, col = 32 * tj + c;  // element (row, col), row < col
+    if (row < ca && col < ca && row < col) {
+      w[at(row, col)] = m1[r][c];
+      if (PART == REF_FINISH) t[at(row, col)] = m2[r][c];
+    }
+  }
+}
+
+// mode REF_PUT_V: V = X (x_off); REF_PUT_X: Xs = X; REF_CHECK: X = Xs D
+__global__ void __launch_bounds__(256) refine_put_kernel(const SvdJob *__restrict__ jobs,
+                                                         const int *__restrict__ order, double *__restrict__ work,
+                                                         const double *__restrict__ sv, int mode) {
+  const SvdJob J = jobs[order[blockIdx.y]];
+  const int ca = J.cols_a;
+  const int64_t tot = (int64_t)ca * ca;
+  const double *from = work + (mode == REF_CHECK ? J.b_off : J.x_off);
+  double *to = work + (mode == REF_PUT_V ? J.j_off : J.b_off);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
+    to[e] = mode == REF_CHECK ? from[e] * sv[J.sv_off + e / ca] : from[e];
 }
 
 // ---------------------------------------------------------------- select
@@ -2688,12 +2874,44 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
   return cudaGetLastError();
 }
 
-cudaError_t launch_svd_elementwise(const SvdJob *jobs, int njobs, int max_cols, int mode, double *work,
+cudaError_t launch_svd_elementwise(const SvdJob *jobs, int njobs, int max_cols, int mode, double *work, int *iwork,
                                    cudaStream_t st) {
   if (njobs <= 0 || max_cols <= 0) return cudaGetLastError();
   const int64_t tot = (int64_t)max_cols * max_cols;
   dim3 grid((unsigned)std::min<int64_t>((tot + 255) / 256, 64), (unsigned)njobs);
-  svd_elementwise_kernel<<<grid, 256, 0, st>>>(jobs, work, mode);
+  svd_elementwise_kernel<<<grid, 256, 0, st>>>(jobs, work, iwork, mode);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_svd_refine(SvdRefine part, const SvdJob *jobs, const int *order, int njobs, int max_cols,
+                              double *work, int *iwork, double *sv, cudaStream_t st) {
+  if (njobs <= 0 || max_cols <= 0) return cudaGetLastError();
+  const int nt = (max_cols + 31) / 32;
+  const dim3 tiles((unsigned)(nt * (nt + 1) / 2), (unsigned)njobs);
+  const dim3 elems((unsigned)std::min<int64_t>(((int64_t)max_cols * max_cols + 255) / 256, 64), (unsigned)njobs);
+  switch (part) {
+    case REF_SCALE:
+      refine_scale_kernel<<<dim3((unsigned)((max_cols + 7) / 8), (unsigned)njobs), 256, 0, st>>>(jobs, order, work,
+                                                                                                 iwork, sv);
+      break;
+    case REF_BUILD:
+      refine_pair_kernel<REF_BUILD><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+      break;
+    case REF_BUILD_R:
+      refine_pair_kernel<REF_BUILD_R><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+      break;
+    case REF_FINISH:
+      refine_pair_kernel<REF_FINISH><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+      break;
+    case REF_PUT_V:
+    case REF_PUT_X:
+      refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, sv, part);
+      break;
+    case REF_CHECK:
+      refine_pair_kernel<REF_CHECK><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+      refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, sv, part);
+      break;
+  }
   return cudaGetLastError();
 }
 

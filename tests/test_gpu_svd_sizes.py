@@ -7,7 +7,7 @@ weight."""
 import numpy as np
 import pytest
 
-from workloads import build_mpo, yc4_j1j2_bonds
+from workloads import build_mpo, random_chain_bonds, yc4_j1j2_bonds
 
 from gpu_helpers import context, gpu_psi_dense
 
@@ -46,3 +46,25 @@ def test_large_sector_singular_values(bonds, ell, m, steps, rows):
     assert len(lam) == len(s)
     assert np.max(np.abs(lam - s)) < 1e-10
     assert abs((1.0 - eps[0]) - np.sum(s[:kept[0]] ** 2)) < 1e-10
+
+
+@pytest.mark.parametrize("bonds,m,steps,prec", [
+    (yc4_j1j2_bonds(1.0, 0.5), 130, 8, "fp64"),      # sectors around 64 columns: some refined, some not
+    (yc4_j1j2_bonds(1.0, 0.5), 300, 9, "tf32x3"),    # block kernels
+    (yc4_j1j2_bonds(1.0, 0.5), 300, 9, "fp64"),
+    (random_chain_bonds(8, 0.5, 1.5, 5), 300, 9, "fp64tc"),  # ranks below the sector sizes
+    (yc4_j1j2_bonds(1.0, 0.5), 1000, 11, "bf16x3"),  # large-sector kernels
+])
+def test_kept_bases_orthonormal(bonds, m, steps, prec):
+    """The identity channels of the new blocks are U^T U and V V^T: the kept
+    singular vectors are orthonormal to rounding, whichever of the refinement
+    and the final Jacobi's sweeps finished a sector.  (1e-12: a product of up to
+    2 m terms of rounding 2^-53 per step, over a dozen steps.)"""
+    mpo = build_mpo(bonds, 8)
+    ctx = context(mpo, m, prec=prec)
+    for _ in range(steps):
+        ctx.unit_cell_step()
+    for p in range(ctx.P):
+        for side, channel in ((0, -1), (1, 0)):
+            op = ctx.block_to_host(p, side)[channel]
+            assert np.max(np.abs(op - np.eye(len(op)))) < 1e-12, (p, side)
