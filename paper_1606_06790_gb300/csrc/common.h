@@ -81,7 +81,7 @@ struct WTerm {
   int64_t in_off;
   int in_ld;
   int k0, cols;  // tensor-core W stage: packed K columns [k0, k0 + cols) it adds to
-  int pad;
+  float coef32;  // (float)coef: a conversion would go through the FP64 pipe
   double coef;
 };
 struct WTask {
@@ -281,11 +281,11 @@ struct PackSeg {
   int row0, k0, rows, ks;
   int src_ld, trans;      // trans: source element (row, k) at src[k * src_ld + row]
   int KB, G;              // K blocks and row groups of the packed matrix
-  int sb, src_buf, dst_buf, src_fp32;
+  int sb, src_buf, dst_buf;
+  int kpad;               // zero columns to write after the segment
   int whole;              // digit form: the segment holds the whole K range of its rows
   int exp_buf;            // digit form: slot of the exponent array
-  int kpad;               // digit form: zero columns to write after the segment
-  double alpha;           // digit form: source values scaled by alpha
+  double alpha;           // source values scaled by alpha
 };
 struct WTaskP {           // rows of a packed stage-3 A matrix: one (left sector, s, t)
   int64_t dst_off;
@@ -319,7 +319,10 @@ constexpr int TC_TN = 64;      // N tile of the digit-slice GEMM (TMEM columns p
 // N tiles of the split-operand (TF32x3 / BF16x3) GEMM the tuner chooses from
 constexpr int MIX_NTN = 3;
 constexpr int MIX_TNS[MIX_NTN] = {64, 128, 256};
-cudaError_t launch_pack(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+// units[k] = (segment, first row, first packed K column): a window of PACK_ROWS
+// rows and PACK_K columns
+constexpr int PACK_ROWS = 32, PACK_K = 64;
+cudaError_t launch_pack(const int4 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                         int bf16, cudaStream_t st);
 cudaError_t launch_wstage_tc(const WUnit *units, int nunits, const WTaskP *tasks, const WTerm *terms,
                              double *const *bufs, const int *active, int bf16, cudaStream_t st);
@@ -334,7 +337,6 @@ constexpr int OZ_KBLK = 16;
 constexpr int OZ_MAX_K = 768;
 constexpr int OZ_EXP_EMPTY = (int)0x80808080;  // byte-fill value: row without non-zeros
 // units[k] = (segment, first row): PACK_ROWS rows of a segment
-constexpr int PACK_ROWS = 32;
 cudaError_t launch_oz_exp(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                           cudaStream_t st);
 cudaError_t launch_oz_pack(const int2 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,

@@ -98,6 +98,34 @@ struct OzPacks {                  // segments to pack and their work units
     segs.push_back(s);
   }
 };
+// Split operands of the TF32x3 / BF16x3 matvec: the segments of L, and of psi
+// and R in each N-tile layout, with one work unit per window; each operand and
+// layout is a run of the units.
+enum { MP_L = 0, MP_PSI = 1, MP_R = MP_PSI + MIX_NTN, MP_N = MP_R + MIX_NTN };
+struct MixPacks {
+  std::vector<PackSeg> segs;
+  std::vector<int4> units[MP_N], all;
+  int u0[MP_N + 1] = {};
+  DevBuf dsegs, dunits;
+  void clear() {
+    segs.clear();
+    all.clear();
+    for (auto &u : units) u.clear();
+  }
+  void add(int list, const PackSeg &s) {
+    for (int r = 0; r < s.rows; r += PACK_ROWS)
+      for (int k = s.k0 & ~(PACK_K - 1); k < s.k0 + s.ks + s.kpad; k += PACK_K)
+        units[list].push_back(make_int4((int)segs.size(), r, k, 0));
+    segs.push_back(s);
+  }
+  void finish() {
+    for (int i = 0; i < MP_N; ++i) {
+      u0[i] = (int)all.size();
+      all.insert(all.end(), units[i].begin(), units[i].end());
+    }
+    u0[MP_N] = (int)all.size();
+  }
+};
 struct OzTiles {                  // a digit-slice GEMM's output tiles
   std::vector<TcTile> tiles;
   std::vector<int> sums;          // tasks in several K chunks
@@ -252,7 +280,7 @@ struct idmrg_ctx {
   // matvec), the R split (once per iteration, the chosen candidate's only)
   // and the tasks and tiles of both GEMM stages; tt1 / tt3 hold the tuner's
   // choice for stage 1 / stage 3
-  std::vector<PackSeg> pk_L, pk_psi[MIX_NTN], pk_R[MIX_NTN];
+  MixPacks pk;
   std::vector<TcTask> tc1k[MIX_NTN], tc3k[MIX_NTN];
   std::vector<TcTile> tc1t[MIX_NTN], tc3t[MIX_NTN];
   std::vector<WTaskP> wtp;
@@ -275,8 +303,7 @@ struct idmrg_ctx {
   double inner_factor = 1e-3;
   int inner_cap = 80;
 
-  int pk_L_rows = 0, pk_psi_rows = 0, pk_R_rows = 0;
-  DevBuf dpkL, dpkp[MIX_NTN], dpkR[MIX_NTN], dtc1k[MIX_NTN], dtc1t[MIX_NTN], dtc3k[MIX_NTN], dtc3t[MIX_NTN];
+  DevBuf dtc1k[MIX_NTN], dtc1t[MIX_NTN], dtc3k[MIX_NTN], dtc3t[MIX_NTN];
   DevBuf dwtp, dwtpm, dtarget, dtune_out;
   std::vector<DevBuf> bPA1, bPB1, bT1F, bPA3, bPB3, bRMAP;
   // FP64-accurate digit-slice form of H_eff psi on the tensor cores (the
@@ -935,6 +962,11 @@ idmrg_status sync_bufs(idmrg_ctx *c) {
 // a scratch vector put in the output slot meanwhile).  Stage 3 packs R in each
 // candidate's layout before timing it; the caller packs the chosen one.
 idmrg_status check_dev_err(idmrg_ctx *c);
+cudaError_t mix_pack(idmrg_ctx *c, int list, const int *active_dev) {
+  c->launches += 1;
+  return launch_pack((const int4 *)c->pk.dunits.p + c->pk.u0[list], c->pk.u0[list + 1] - c->pk.u0[list],
+                     (const PackSeg *)c->pk.dsegs.p, (double *const *)c->dbufs.p, active_dev, c->bf16, c->st);
+}
 idmrg_status tc_tune(idmrg_ctx *c, idmrg_ctx::TcTune &T, int stage, double work, int64_t max_psi) {
   const int forced = c->force_tn[stage == 1 ? 0 : 1];
   if (forced > 0) {
@@ -964,11 +996,7 @@ idmrg_status tc_tune(idmrg_ctx *c, idmrg_ctx::TcTune &T, int stage, double work,
   for (int k = 0; k < MIX_NTN; ++k) {
     if (!T.e0[k]) CK(cudaEventCreate(&T.e0[k]));
     if (!T.e1[k]) CK(cudaEventCreate(&T.e1[k]));
-    if (stage == 3) {
-      CK(launch_pack((const PackSeg *)c->dpkR[k].p, (int)c->pk_R[k].size(), c->pk_R_rows, bufs, nullptr, c->bf16,
-                     c->st));
-      c->launches += 1;
-    }
+    if (stage == 3) CK(mix_pack(c, MP_R + k, nullptr));
     const TcTile *dt = (const TcTile *)(stage == 1 ? c->dtc1t[k].p : c->dtc3t[k].p);
     const TcTask *dk = (const TcTask *)(stage == 1 ? c->dtc1k[k].p : c->dtc3k[k].p);
     const int nt = (int)tiles[k].size();
@@ -1000,10 +1028,8 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
   const int64_t TA = 128 * 32;
   const int kblk = c->bf16 ? 64 : 32;
   auto cdiv = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
-  c->pk_L.clear();
+  c->pk.clear();
   for (int k = 0; k < MIX_NTN; ++k) {
-    c->pk_psi[k].clear();
-    c->pk_R[k].clear();
     c->tc1k[k].clear();
     c->tc1t[k].clear();
     c->tc3k[k].clear();
@@ -1012,11 +1038,11 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
   c->wtp.clear();
   c->wtpm.clear();
   c->wunits.clear();
-  c->pk_L_rows = c->pk_psi_rows = c->pk_R_rows = 0;
   double work1 = 0.0, work3 = 0.0;
   int64_t max_psi = 1;
-  auto seg = [&](std::vector<PackSeg> &v, int &mr, int sb, int dst_buf, int64_t dst_off, int src_buf,
-                 int64_t src_off, int row0, int k0, int rows, int ks, int ld, int trans, int KB, int G) {
+  // K: the packed matrix's; its last segment writes the padding of the K blocks
+  auto seg = [&](int list, int sb, int dst_buf, int64_t dst_off, int src_buf, int64_t src_off, int row0, int k0,
+                 int rows, int ks, int ld, int trans, int K, int G) {
     if (rows <= 0 || ks <= 0) return;
     PackSeg p{};
     p.dst_off = dst_off;
@@ -1027,14 +1053,14 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
     p.ks = ks;
     p.src_ld = ld;
     p.trans = trans;
-    p.KB = KB;
+    p.KB = (int)cdiv(K, kblk);
     p.G = G;
     p.sb = sb;
     p.src_buf = src_buf;
     p.dst_buf = dst_buf;
-    p.src_fp32 = 0;
-    v.push_back(p);
-    mr = std::max(mr, rows);
+    p.kpad = k0 + ks == K ? p.KB * kblk - K : 0;
+    p.alpha = 1.0;
+    c->pk.add(list, p);
   };
   for (int p = 0; p < P; ++p) {
     if (!c->owns(p)) continue;
@@ -1070,14 +1096,13 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
       for (int a = 0; a < wa; ++a) {
         if (rs1[si][a] < 0) continue;
         const int so = L.lay.so[a * SL + si];
-        seg(c->pk_L, c->pk_L_rows, p, BUF_PA1, pa1[si], BUF_L, L.lay.off[a * SL + si], rs1[si][a], 0,
-            BL.dim[so], K, K, 0, KB, GA);
+        seg(MP_L, p, BUF_PA1, pa1[si], BUF_L, L.lay.off[a * SL + si], rs1[si][a], 0, BL.dim[so], K, K, 0, K, GA);
       }
       for (int k = 0; k < MIX_NTN; ++k) {  // B (psi) layout, task and tiles per N tile
         const int TN = MIX_TNS[k], NT = (int)cdiv(N, TN);
         const int64_t pb = pb1n[k];
         pb1n[k] += (int64_t)NT * KB * 2 * TN * 32;
-        seg(c->pk_psi[k], c->pk_psi_rows, p, BUF_PB1, pb, BUF_IN, psi.roff[si], 0, 0, N, K, N, 1, KB, TN / 8);
+        seg(MP_PSI + k, p, BUF_PB1, pb, BUF_IN, psi.roff[si], 0, 0, N, K, N, 1, K, TN / 8);
         TcTask t{};
         t.a_off = pa1[si];
         t.b_off = pb;
@@ -1139,8 +1164,8 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
         for (int cc = 0; cc < wc; ++cc) {
           if (ks[cc] < 0) continue;
           const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
-          seg(c->pk_R[k], c->pk_R_rows, p, BUF_PB3, pb3[k], BUF_R, R.lay.off[cc * SR + jin], 0, ks[cc], N,
-              BR.dim[jin], BR.dim[jin], 0, KB, TN / 8);
+          seg(MP_R + k, p, BUF_PB3, pb3[k], BUF_R, R.lay.off[cc * SR + jin], 0, ks[cc], N, BR.dim[jin], BR.dim[jin], 0,
+              K, TN / 8);
         }
       }
       // W stage: T3[c](i,s,t) into rows rows_of(i,s,t), columns ks[c]
@@ -1178,6 +1203,7 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
                     term.k0 = ks[cc];
                     term.cols = BR.dim[jin];
                     term.coef = cf;
+                    term.coef32 = (float)cf;
                     c->wtpm.push_back(term);
                   }
               }
@@ -1216,13 +1242,11 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
           c->ensure(c->bT1F[p], 4 * std::max<int64_t>(t1fn, 4)) &&
           c->ensure(c->bPA3[p], 4 * std::max<int64_t>(pa3n, 4)) &&
           c->ensure(c->bPB3[p], 4 * std::max<int64_t>(pb3max, 4)) && c->upload(c->bRMAP[p], rmap));
-    // zero padding of every packed operand (only real elements are rewritten
-    // later; a K block's padding is zero in A, so B's padding only has to
-    // hold finite values, which a switch of B layouts leaves behind)
-    CK(cudaMemsetAsync(c->bPA1[p].p, 0, 4 * pa1n, c->st));
-    CK(cudaMemsetAsync(c->bPB1[p].p, 0, 4 * pb1max, c->st));
+    // zeros where the W stage has no term, and in the K padding (only real
+    // elements are rewritten later); the other operands' K padding is written
+    // with their last segment, and rows past M or N only reach outputs that are
+    // not stored
     CK(cudaMemsetAsync(c->bPA3[p].p, 0, 4 * pa3n, c->st));
-    CK(cudaMemsetAsync(c->bPB3[p].p, 0, 4 * pb3max, c->st));
     c->hbufs[p * NBUF + BUF_PA1] = c->dp(c->bPA1[p]);
     c->hbufs[p * NBUF + BUF_PB1] = c->dp(c->bPB1[p]);
     c->hbufs[p * NBUF + BUF_T1F] = c->dp(c->bT1F[p]);
@@ -1231,18 +1255,17 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
     c->hbufs[p * NBUF + BUF_RMAP] = c->dp(c->bRMAP[p]);
   }
   NOMEM(c->upload(c->dwunits, c->wunits));
-  NOMEM(c->upload(c->dpkL, c->pk_L) && c->upload(c->dwtp, c->wtp) && c->upload(c->dwtpm, c->wtpm));
+  c->pk.finish();
+  NOMEM(c->upload(c->pk.dsegs, c->pk.segs) && c->upload(c->pk.dunits, c->pk.all) && c->upload(c->dwtp, c->wtp) &&
+        c->upload(c->dwtpm, c->wtpm));
   for (int k = 0; k < MIX_NTN; ++k)
-    NOMEM(c->upload(c->dpkp[k], c->pk_psi[k]) && c->upload(c->dpkR[k], c->pk_R[k]) &&
-          c->upload(c->dtc1k[k], c->tc1k[k]) && c->upload(c->dtc1t[k], c->tc1t[k]) &&
+    NOMEM(c->upload(c->dtc1k[k], c->tc1k[k]) && c->upload(c->dtc1t[k], c->tc1t[k]) &&
           c->upload(c->dtc3k[k], c->tc3k[k]) && c->upload(c->dtc3t[k], c->tc3t[k]));
   NOMEM(c->upload(c->dbufs, c->hbufs));
   // split L once for this iteration
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
-  CK(launch_pack((const PackSeg *)c->dpkL.p, (int)c->pk_L.size(), c->pk_L_rows, (double *const *)c->dbufs.p,
-                 nullptr, c->bf16, c->st));
+  CK(mix_pack(c, MP_L, nullptr));
   c->kend(IDMRG_K_HEFF_WSTAGE);
-  c->launches += 1;
   // N tiles: tuned whenever a stage's work moved by more than 10 % since
   // its last tuning (every iteration while the blocks grow, rarely after)
   idmrg_status ts = tc_tune(c, c->tt1, 1, work1, max_psi);
@@ -1252,10 +1275,8 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
   // split R once for this iteration, in the chosen stage-3 layout
   const int k3 = c->tt3.choice;
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
-  CK(launch_pack((const PackSeg *)c->dpkR[k3].p, (int)c->pk_R[k3].size(), c->pk_R_rows,
-                 (double *const *)c->dbufs.p, nullptr, c->bf16, c->st));
+  CK(mix_pack(c, MP_R + k3, nullptr));
   c->kend(IDMRG_K_HEFF_WSTAGE);
-  c->launches += 1;
   return IDMRG_OK;
 }
 
@@ -1443,6 +1464,7 @@ idmrg_status plan_oz(idmrg_ctx *c) {
                     term.k0 = ks[cc];
                     term.cols = BR.dim[jin];
                     term.coef = cf;
+                    term.coef32 = (float)cf;
                     c->wtpm_oz.push_back(term);
                   }
               }
@@ -1594,8 +1616,7 @@ idmrg_status heff_launch_mixed(idmrg_ctx *c, const int *active_dev, const int *a
     }
   const int k1 = std::max(c->tt1.choice, 0), k3 = std::max(c->tt3.choice, 0);
   c->kbegin(IDMRG_K_HEFF_WSTAGE);
-  CK(launch_pack((const PackSeg *)c->dpkp[k1].p, (int)c->pk_psi[k1].size(), c->pk_psi_rows, bufs, active_dev,
-                 c->bf16, c->st));
+  CK(mix_pack(c, MP_PSI + k1, active_dev));
   c->kend(IDMRG_K_HEFF_WSTAGE, 0.0, pb);
   c->kbegin(IDMRG_K_HEFF_GEMM);
   CK(launch_tc_gemm((const TcTile *)c->dtc1t[k1].p, (int)c->tc1t[k1].size(), (const TcTask *)c->dtc1k[k1].p, bufs,
@@ -1609,7 +1630,7 @@ idmrg_status heff_launch_mixed(idmrg_ctx *c, const int *active_dev, const int *a
   CK(launch_tc_gemm((const TcTile *)c->dtc3t[k3].p, (int)c->tc3t[k3].size(), (const TcTask *)c->dtc3k[k3].p, bufs,
                     active_dev, (int *)c->derr.p, c->bf16, MIX_TNS[k3], c->st));
   c->kend(IDMRG_K_HEFF_GEMM, gf, by);
-  c->launches += 4;
+  c->launches += 3;
   c->mixed_matvecs += 1;
   return IDMRG_OK;
 }
@@ -3695,7 +3716,7 @@ void idmrg_destroy(idmrg_ctx *c) {
                     &c->ssv, &c->sjob0, &c->snjob, &c->skpj, &c->sperm, &c->slam, &c->seps, &c->sepsb, &c->skept,
                     &c->scj, &c->slamk, &c->siw, &c->sorder, &c->sorderq, &c->dsgk, &c->dsgs,
                     &c->dswk, &c->dsws, &c->dsxk, &c->dsxs, &c->dshk, &c->dshs, &c->dsrk, &c->dsrs, &c->dskk, &c->dsks,
-                    &c->dsvk, &c->dsvs, &c->dstk, &c->dsts, &c->dpkL, &c->dtune_out, &c->dmsb,
+                    &c->dsvk, &c->dsvs, &c->dstk, &c->dsts, &c->pk.dsegs, &c->pk.dunits, &c->dtune_out, &c->dmsb,
                     &c->dwtp, &c->dwtpm, &c->dwunits, &c->dtarget, &c->oz_step_w.dsegs, &c->oz_step_w.dunits, &c->oz_step_p.dsegs,
                     &c->oz_step_p.dunits, &c->oz_psi.dsegs, &c->oz_psi.dunits, &c->dozwu, &c->dozkeep,
                     &c->doz1k,
@@ -3704,7 +3725,7 @@ void idmrg_destroy(idmrg_ctx *c) {
                     &c->goz_exps})
     rel(*b);
   for (int k = 0; k < MIX_NTN; ++k)
-    for (DevBuf *b : {&c->dpkp[k], &c->dpkR[k], &c->dtc1k[k], &c->dtc1t[k], &c->dtc3k[k], &c->dtc3t[k]}) rel(*b);
+    for (DevBuf *b : {&c->dtc1k[k], &c->dtc1t[k], &c->dtc3k[k], &c->dtc3t[k]}) rel(*b);
   for (auto *t : {&c->tt1, &c->tt3})
     for (int k = 0; k < MIX_NTN; ++k) {
       if (t->e0[k]) cudaEventDestroy(t->e0[k]);

@@ -73,41 +73,167 @@ __device__ __forceinline__ int64_t packed_off_h(int row, int k, int KB, int G) {
   return ((int64_t)rt * KB + kb) * 2 * tile_h + (((int64_t)kc * G + (rr >> 3)) * 8 + (rr & 7)) * 8 + (k & 7);
 }
 
-// hi/lo split of x (given in FP64 or FP32) into the packed operand `dst` at
-// element (row, k): TF32 pair (bf16 = 0) or BF16 pair (bf16 = 1).
-__device__ __forceinline__ void put_split(float *dst, int row, int k, int KB, int G, int bf16, double x) {
+// hi/lo split of an FP32 value: hi its BF16 (bf16 = 1) or TF32 rounding, lo the
+// rest, which is exact
+__device__ __forceinline__ void split(float x, int bf16, float &hi, float &lo) {
+  hi = bf16 ? __bfloat162float(__float2bfloat16_rn(x)) : tf32_round(x);
+  lo = x - hi;
+}
+
+// The same of an FP64 value: hi from x rounded to FP32, lo = x - hi rounded to
+// FP32.  The FP64 pipe takes 4 operations per element for it (two narrowings, a
+// widening and the difference) at 2 lanes per clock and SM, which is more time
+// than the memory traffic; so integers round x to f, and x - hi = (f - hi) + r,
+// r = +-E 2^(e-52) with |E| <= 2^28, is formed in FP32 with one rounding: f - hi
+// and the part of E above its low 21 bits make 24 significant bits at most (hi
+// leaves 2^44 + 2^28 units at most), so the first fma is exact.  Values whose
+// rest could leave the normal FP32 range take the FP64 operations.
+__device__ __forceinline__ void split(double x, int bf16, float &hi, float &lo) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int e = (int)((h >> 20) & 2047u) - 1023;
+  if (((h << 1) | l) == 0) {
+    hi = __uint_as_float(h);
+    lo = 0.0f;
+    return;
+  }
+  if (e < -74 || e > 100) {
+    hi = bf16 ? __bfloat162float(__float2bfloat16_rn((float)x)) : tf32_round((float)x);
+    lo = (float)(x - (double)hi);
+    return;
+  }
+  const uint32_t trunc = ((uint32_t)(e + 127) << 23) | ((h & 0xFFFFFu) << 3) | (l >> 29);
+  const uint32_t rest = l & 0x1FFFFFFFu;
+  const bool up = rest > 0x10000000u || (rest == 0x10000000u && (trunc & 1u));
+  const float f = __uint_as_float((h & 0x80000000u) | (trunc + (up ? 1u : 0u)));
+  const int E = (int)rest - (up ? 0x20000000 : 0);
+  hi = bf16 ? __bfloat162float(__float2bfloat16_rn(f)) : tf32_round(f);
+  // integers below 2^23 to FP32 through the mantissa of 1.5 * 2^23
+  const float Eh = __int_as_float(0x4B400000 + (E >> 21)) - 12582912.0f;
+  const float El = __int_as_float(0x4B400000 + (E & 0x1FFFFF)) - 12582912.0f;
+  const float u = __uint_as_float((h & 0x80000000u) | ((uint32_t)(e - 52 + 127) << 23));
+  lo = fmaf(El, u, fmaf(Eh, u * 2097152.0f, f - hi));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // (exact for hi parts)
+  return (uint32_t)__bfloat16_as_ushort(v.x) | ((uint32_t)__bfloat16_as_ushort(v.y) << 16);
+}
+
+// one 16-byte group (8 BF16 or 4 TF32 elements from packed K kg on) of packed
+// row `row`
+template <class T>
+__device__ __forceinline__ void put_group(float *dst, int row, int kg, int KB, int G, int bf16, const T *v) {
+  float hi[8], lo[8];
   if (bf16) {
-    const __nv_bfloat16 hi = __float2bfloat16_rn((float)x);
-    const __nv_bfloat16 lo = __float2bfloat16_rn((float)(x - (double)__bfloat162float(hi)));
-    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst);
-    const int64_t o = packed_off_h(row, k, KB, G);
-    h[o] = hi;
-    h[o + (int64_t)8 * G * 64] = lo;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) split(v[j], 1, hi[j], lo[j]);
+    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst) + packed_off_h(row, kg, KB, G);
+    *reinterpret_cast<uint4 *>(h) = make_uint4(pack_bf16x2(hi[0], hi[1]), pack_bf16x2(hi[2], hi[3]),
+                                               pack_bf16x2(hi[4], hi[5]), pack_bf16x2(hi[6], hi[7]));
+    *reinterpret_cast<uint4 *>(h + (int64_t)8 * G * 64) =
+        make_uint4(pack_bf16x2(lo[0], lo[1]), pack_bf16x2(lo[2], lo[3]), pack_bf16x2(lo[4], lo[5]),
+                   pack_bf16x2(lo[6], lo[7]));
   } else {
-    const float hi = tf32_round((float)x);
-    const int64_t o = packed_off(row, k, KB, G);
-    dst[o] = hi;
-    dst[o + (int64_t)8 * G * 32] = (float)(x - (double)hi);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) split(v[j], 0, hi[j], lo[j]);
+    float *f = dst + packed_off(row, kg, KB, G);
+    *reinterpret_cast<float4 *>(f) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<float4 *>(f + (int64_t)8 * G * 32) = make_float4(lo[0], lo[1], lo[2], lo[3]);
   }
 }
 
-constexpr int PROWS = 16;
+// the elements of a group that fall into packed K [ka, kb), one by one: a group
+// that a neighbouring segment shares
+__device__ __forceinline__ void put_part(float *dst, int row, int kg, int ka, int kb, int KB, int G, int bf16,
+                                         const double *v) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = kg + j;
+    if (k < ka || k >= kb || (!bf16 && j >= 4)) continue;
+    float hi, lo;
+    split(v[j], bf16, hi, lo);
+    if (bf16) {
+      __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst) + packed_off_h(row, k, KB, G);
+      h[0] = __float2bfloat16_rn(hi);
+      h[(int64_t)8 * G * 64] = __float2bfloat16_rn(lo);
+    } else {
+      float *f = dst + packed_off(row, k, KB, G);
+      f[0] = hi;
+      f[(int64_t)8 * G * 32] = lo;
+    }
+  }
+}
 
-__global__ void pack_kernel(const PackSeg *__restrict__ segs, double *const *__restrict__ bufs,
-                            const int *__restrict__ active, int bf16) {
-  const PackSeg s = segs[blockIdx.x];
+// Packing runs through windows of 32 rows and 64 packed K columns (aligned to
+// 64) held in shared memory: read with the lanes along whatever is contiguous
+// in the source, written a 16-byte group of a row per thread with the lanes
+// along the rows, so that a warp fills 512 contiguous bytes.
+constexpr int OP_ROWS = PACK_ROWS, OP_K = PACK_K, OP_LD = OP_K + 2;
+
+// SCALED: alpha is not 1 (a multiplication is as long on the FP64 pipe as the
+// element's memory traffic)
+template <bool SCALED>
+__device__ __forceinline__ double pack_src(const PackSeg &s, const double *src, int r, int k) {
+  const double x = src[s.trans ? (int64_t)k * s.src_ld + r : (int64_t)r * s.src_ld + k];
+  return SCALED ? s.alpha * x : x;
+}
+
+// rows r0 .. r0 + nr - 1 of a segment, packed K columns kw .. kw + 63, zeros
+// where the segment has none (256 threads)
+template <bool SCALED>
+__device__ __forceinline__ void pack_load_window(const PackSeg &s, const double *src, int r0, int nr, int kw,
+                                                 double *tile) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k1 = s.k0 + s.ks;
+  if (s.trans) {
+#pragma unroll
+    for (int i = 0; i < OP_K / 8; ++i) {
+      const int kk = warp + 8 * i, k = kw + kk;
+      if (lane < nr)
+        tile[lane * OP_LD + kk] = k >= s.k0 && k < k1 ? pack_src<SCALED>(s, src, r0 + lane, k - s.k0) : 0.0;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < OP_ROWS / 8; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = warp + 8 * i, kk = lane + 32 * h, k = kw + kk;
+        if (r < nr)
+          tile[r * OP_LD + kk] = k >= s.k0 && k < k1 ? pack_src<SCALED>(s, src, r0 + r, k - s.k0) : 0.0;
+      }
+  }
+}
+
+// Split operands, one window per block: memory bound, 8 bytes in and 4 (BF16) or
+// 8 (TF32) out per element.  Measured (GB300, kagome cylinder at m = 1000, BF16,
+// under a profiler): R of all superblocks, 13 300 windows, 178 us by a thread per
+// element, its 16-bit stores and FP64 operations; 123 us through windows with the
+// split in integers; 99 us without the multiplication by alpha = 1.  What is left
+// are the rectangles' partly filled windows and the chain of loads in front of
+// each (unit, segment, data).
+__global__ void __launch_bounds__(256) pack_kernel(const int4 *__restrict__ units, const PackSeg *__restrict__ segs,
+                                                   double *const *__restrict__ bufs, const int *__restrict__ active,
+                                                   int bf16) {
+  __shared__ __align__(16) double tile[OP_ROWS * OP_LD];
+  const int4 u = units[blockIdx.x];  // segment, first row, first packed K column
+  const PackSeg s = segs[u.x];
   if (active && !active[s.sb]) return;
-  const int r0 = blockIdx.y * PROWS;
-  if (r0 >= s.rows) return;
-  const int r1 = min(s.rows, r0 + PROWS);
+  const int nr = min(OP_ROWS, s.rows - u.y), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pack_load_window<false>(s, bufs[s.sb * NBUF + s.src_buf] + s.src_off, u.y, nr, u.z, tile);
+  __syncthreads();
+  if (lane >= nr) return;
   float *dst = (float *)bufs[s.sb * NBUF + s.dst_buf] + s.dst_off;
-  const int n = (r1 - r0) * s.ks;
-  for (int e = threadIdx.x; e < n; e += blockDim.x) {
-    const int r = r0 + e / s.ks, k = e % s.ks;
-    const int64_t si = s.trans ? (int64_t)k * s.src_ld + r : (int64_t)r * s.src_ld + k;
-    const double x = s.src_fp32 ? (double)((const float *)bufs[s.sb * NBUF + s.src_buf])[s.src_off + si]
-                                : bufs[s.sb * NBUF + s.src_buf][s.src_off + si];
-    put_split(dst, s.row0 + r, s.k0 + k, s.KB, s.G, bf16, x);
+  const int gw = bf16 ? 8 : 4, ka = s.k0, kb = s.k0 + s.ks + s.kpad, row = s.row0 + u.y + lane;
+  for (int k = gw * warp; k < OP_K; k += 8 * gw) {
+    const int kg = u.z + k;
+    if (kg + gw <= ka || kg >= kb) continue;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2)
+      if (j < gw) *reinterpret_cast<double2 *>(v + j) = *reinterpret_cast<const double2 *>(tile + lane * OP_LD + k + j);
+    if (kg >= ka && kg + gw <= kb)
+      put_group(dst, row, kg, s.KB, s.G, bf16, v);
+    else
+      put_part(dst, row, kg, ka, kb, s.KB, s.G, bf16, v);
   }
 }
 
@@ -173,6 +299,21 @@ __device__ __forceinline__ void w_walk(const WUnit *__restrict__ units, int nuni
   }
 }
 
+template <class T>
+__device__ __forceinline__ T w_coef(const WTerm &w);
+template <>
+__device__ __forceinline__ float w_coef<float>(const WTerm &w) {
+  return w.coef32;
+}
+template <>
+__device__ __forceinline__ double w_coef<double>(const WTerm &w) {
+  return w.coef;
+}
+// comparisons that stay off the FP64 pipe, where one holds its unit for 64 cycles a warp
+__device__ __forceinline__ bool is_one(float x) { return x == 1.0f; }
+__device__ __forceinline__ bool is_one(double x) { return __double_as_longlong(x) == 0x3FF0000000000000ll; }
+__device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
+
 // The window's sums: warp w holds rows w, w + 8, w + 16, w + 24, lane l the
 // columns l and l + 32.  Most elements have one term of coefficient 1, which is
 // copied (an FMA in FP64 holds its unit for 64 cycles); halves of the window
@@ -196,7 +337,8 @@ __device__ __forceinline__ void w_accumulate(const WUnit &u, const WTerm *__rest
     for (int q = 0; q < n; ++q) {
       const WTerm w = st[q];
       const int k = u.k0 - w.k0;  // the window's first column in the rectangle
-      const bool copy = w.k0 != last && w.coef == 1.0;
+      const T cf = w_coef<T>(w);
+      const bool copy = w.k0 != last && is_one(cf);
       last = w.k0;
       const bool on[2] = {(unsigned)(k + lane) < (unsigned)w.cols, (unsigned)(k + lane + 32) < (unsigned)w.cols};
       const bool half[2] = {k + 31 >= 0 && k < w.cols, k + 32 < w.cols};  // (every term reaches the window)
@@ -223,7 +365,6 @@ __device__ __forceinline__ void w_accumulate(const WUnit &u, const WTerm *__rest
               if (on[h]) acc[i][h] = x[i][h];
           }
       } else {
-        const T cf = (T)w.coef;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           if (half[h]) {
@@ -235,38 +376,7 @@ __device__ __forceinline__ void w_accumulate(const WUnit &u, const WTerm *__rest
   }
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 a, __nv_bfloat16 b) {
-  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
 constexpr int WT_LD = W_K + 4;  // row stride of the tile (floats)
-
-// hi/lo split of one 16-byte group (8 BF16 or 4 TF32 elements from packed K kg
-// on) of packed row `row`
-__device__ __forceinline__ void put_group(float *dst, int row, int kg, int KB, int G, int bf16, const float *v) {
-  if (bf16) {
-    __nv_bfloat16 hi[8], lo[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      hi[j] = __float2bfloat16_rn(v[j]);
-      lo[j] = __float2bfloat16_rn(v[j] - __bfloat162float(hi[j]));
-    }
-    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(dst) + packed_off_h(row, kg, KB, G);
-    *reinterpret_cast<uint4 *>(h) = make_uint4(pack_bf16x2(hi[0], hi[1]), pack_bf16x2(hi[2], hi[3]),
-                                               pack_bf16x2(hi[4], hi[5]), pack_bf16x2(hi[6], hi[7]));
-    *reinterpret_cast<uint4 *>(h + (int64_t)8 * G * 64) =
-        make_uint4(pack_bf16x2(lo[0], lo[1]), pack_bf16x2(lo[2], lo[3]), pack_bf16x2(lo[4], lo[5]),
-                   pack_bf16x2(lo[6], lo[7]));
-  } else {
-    float hi[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) hi[j] = tf32_round(v[j]);
-    float *f = dst + packed_off(row, kg, KB, G);
-    *reinterpret_cast<float4 *>(f) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<float4 *>(f + (int64_t)8 * G * 32) =
-        make_float4(v[0] - hi[0], v[1] - hi[1], v[2] - hi[2], v[3] - hi[3]);
-  }
-}
 
 constexpr int W_TC_CTAS = 6;  // resident per SM
 __global__ void __launch_bounds__(256, W_TC_CTAS) wstage_tc_kernel(const WUnit *__restrict__ units, int nunits,
@@ -626,15 +736,12 @@ __device__ __forceinline__ void oz_digits8(const double *v, int e, uint4 (&out)[
     out[p] = make_uint4(oz_sub192(w[p][0]), oz_sub192(w[p][1]), oz_sub192(w[p][2]), oz_sub192(w[p][3]));
 }
 
-// Packing runs through windows of 32 rows and 64 packed K columns (aligned to
-// 64) held in shared memory: read with the lanes along whatever is contiguous
-// in the source, written with a row and eight K elements per thread, so that a
-// warp fills 512 contiguous bytes of every plane (128 of a B plane).  It is
-// memory bound: 8 bytes in, 16 out per element.  (Before, a thread per element
-// stored 16 bits per plane; environments and prediction of the kagome cylinder
-// at m = 1000 11.6 -> 8.2 ms a step with it.)
-static_assert(W_ROWS == PACK_ROWS && W_K == 64, "windows of oz_store_window");
-constexpr int OP_ROWS = PACK_ROWS, OP_K = 64, OP_LD = OP_K + 2;
+// Digit packing goes through the windows of pack_kernel, eight K elements of a
+// row per thread (a warp fills 512 contiguous bytes of every plane, 128 of a B
+// plane).  It is memory bound: 8 bytes in, 16 out per element.  (Before, a
+// thread per element stored 16 bits per plane; environments and prediction of
+// the kagome cylinder at m = 1000 11.6 -> 8.2 ms a step with it.)
+static_assert(W_ROWS == PACK_ROWS && W_K == PACK_K, "windows of oz_store_window");
 
 // The thread's share of a window: packed row row0 + lane (lane < nr), K group
 // kw + 8 warp; elements outside [ka, kb) belong to a neighbour.
@@ -669,13 +776,9 @@ __device__ __forceinline__ void oz_store_window(__nv_bfloat16 *dst, const double
   }
 }
 
-__device__ __forceinline__ double oz_src(const PackSeg &s, const double *src, int r, int k) {
-  const double x = src[s.trans ? (int64_t)k * s.src_ld + r : (int64_t)r * s.src_ld + k];
-  return s.alpha == 1.0 ? x : s.alpha * x;
-}
-
 // exponents of the rows r0 .. r0 + nr - 1 of a segment into rexp[32] (every
 // thread of the block takes part)
+template <bool SCALED>
 __device__ __forceinline__ void oz_row_exps(const PackSeg &s, const double *src, int r0, int nr, int *rexp) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x < OP_ROWS) rexp[threadIdx.x] = OZ_EXP_EMPTY;
@@ -686,8 +789,8 @@ __device__ __forceinline__ void oz_row_exps(const PackSeg &s, const double *src,
     if (lane < nr) {
 #pragma unroll 8
       for (int k = warp; k < s.ks; k += 8) {
-        const double x = oz_src(s, src, r0 + lane, k);
-        if (x != 0.0) m = max(m, oz_exp_of(x));
+        const double x = pack_src<SCALED>(s, src, r0 + lane, k);
+        if (!is_zero(x)) m = max(m, oz_exp_of(x));
       }
     }
     if (m != OZ_EXP_EMPTY) atomicMax(&rexp[lane], m);
@@ -697,8 +800,8 @@ __device__ __forceinline__ void oz_row_exps(const PackSeg &s, const double *src,
     for (int k = lane; k < s.ks; k += 32) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const double x = warp + 8 * i < nr ? oz_src(s, src, r0 + warp + 8 * i, k) : 0.0;
-        if (x != 0.0) m[i] = max(m[i], oz_exp_of(x));
+        const double x = warp + 8 * i < nr ? pack_src<SCALED>(s, src, r0 + warp + 8 * i, k) : 0.0;
+        if (!is_zero(x)) m[i] = max(m[i], oz_exp_of(x));
       }
     }
 #pragma unroll
@@ -719,7 +822,11 @@ __global__ void __launch_bounds__(256) oz_exp_kernel(const int2 *__restrict__ un
   const PackSeg s = segs[u.x];
   if (s.whole || (active && !active[s.sb])) return;
   const int nr = min(OP_ROWS, s.rows - u.y);
-  oz_row_exps(s, bufs[s.sb * NBUF + s.src_buf] + s.src_off, u.y, nr, rexp);
+  const double *src = bufs[s.sb * NBUF + s.src_buf] + s.src_off;
+  if (is_one(s.alpha))
+    oz_row_exps<false>(s, src, u.y, nr, rexp);
+  else
+    oz_row_exps<true>(s, src, u.y, nr, rexp);
   int *ex = (int *)bufs[s.sb * NBUF + s.exp_buf] + s.exp_off + s.row0 + u.y;
   if (threadIdx.x < nr && rexp[threadIdx.x] != OZ_EXP_EMPTY) atomicMax(ex + threadIdx.x, rexp[threadIdx.x]);
 }
@@ -741,29 +848,22 @@ __global__ void __launch_bounds__(256, 3) oz_pack_kernel(const int2 *__restrict_
   const double *src = bufs[s.sb * NBUF + s.src_buf] + s.src_off;
   __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(bufs[s.sb * NBUF + s.dst_buf]) + s.dst_off;
   if (s.whole) {
-    oz_row_exps(s, src, r0, nr, rexp);
+    if (is_one(s.alpha))
+      oz_row_exps<false>(s, src, r0, nr, rexp);
+    else
+      oz_row_exps<true>(s, src, r0, nr, rexp);
     if (threadIdx.x < nr) ex[threadIdx.x] = rexp[threadIdx.x];
   } else {
     if (threadIdx.x < nr) rexp[threadIdx.x] = ex[threadIdx.x];
   }
+  const bool scaled = !is_one(s.alpha);
   const int k1 = s.k0 + s.ks, kend = k1 + s.kpad;  // zeros up to the end of the last K block
   for (int kw = s.k0 & ~(OP_K - 1); kw < kend; kw += OP_K) {
     __syncthreads();
-    if (s.trans) {
-#pragma unroll
-      for (int i = 0; i < OP_K / 8; ++i) {
-        const int kk = warp + 8 * i, k = kw + kk;
-        if (lane < nr) tile[lane * OP_LD + kk] = k >= s.k0 && k < k1 ? oz_src(s, src, r0 + lane, k - s.k0) : 0.0;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < OP_ROWS / 8; ++i)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int r = warp + 8 * i, kk = lane + 32 * h, k = kw + kk;
-          if (r < nr) tile[r * OP_LD + kk] = k >= s.k0 && k < k1 ? oz_src(s, src, r0 + r, k - s.k0) : 0.0;
-        }
-    }
+    if (scaled)
+      pack_load_window<true>(s, src, r0, nr, kw, tile);
+    else
+      pack_load_window<false>(s, src, r0, nr, kw, tile);
     __syncthreads();
     oz_store_window(dst, tile, lane < nr ? rexp[lane] : 0, s.row0 + r0, nr, kw, s.k0, kend, s.KB, s.G);
   }
@@ -809,7 +909,7 @@ __global__ void __launch_bounds__(256, W_OZ_CTAS[PASS]) wstage_oz_kernel(const W
         int m = OZ_EXP_EMPTY;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          if (acc[i][h] != 0.0) m = max(m, oz_exp_of(acc[i][h]));
+          if (!is_zero(acc[i][h])) m = max(m, oz_exp_of(acc[i][h]));
           if (kept) kept[8 * i * W_K + 32 * h] = acc[i][h];
         }
         m = __reduce_max_sync(0xffffffffu, m);
@@ -1170,12 +1270,9 @@ cudaError_t launch_oz_sum(const int *ids, int n, int max_rows, const TcTask *tas
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(const PackSeg *segs, int nseg, int max_rows, double *const *bufs, const int *active,
+cudaError_t launch_pack(const int4 *units, int nunits, const PackSeg *segs, double *const *bufs, const int *active,
                         int bf16, cudaStream_t st) {
-  if (nseg > 0 && max_rows > 0) {
-    dim3 grid(nseg, (max_rows + PROWS - 1) / PROWS);
-    pack_kernel<<<grid, 256, 0, st>>>(segs, bufs, active, bf16);
-  }
+  if (nunits > 0) pack_kernel<<<nunits, 256, 0, st>>>(units, segs, bufs, active, bf16);
   return cudaGetLastError();
 }
 
