@@ -26,6 +26,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.h"
 
@@ -209,13 +210,25 @@ __global__ void __launch_bounds__(QR_THREADS) qrcp_kernel(const SvdJob *__restri
 // ------------------------------------------------------------ cluster QRCP
 // The same pivoted Householder QR over a cluster of C CTAs.  Column position
 // j lives in the shared memory of CTA j mod C (cyclic, so the trailing
-// columns stay spread as k grows).  Step k: the pivot is the largest
-// remaining column norm over the cluster (candidates gathered in rank 0's
-// shared memory, ties to the lower position as in qrcp_kernel); positions k
-// and p are swapped between their owners through distributed shared memory;
-// the owner of k forms the reflector and publishes it; every CTA applies it
-// to its own trailing columns.  The trailing update, which holds the
-// single-CTA kernel at one SM's FP64 rate, is spread over C SMs.
+// columns stay spread as k grows).  Two cluster barriers a step:
+//   every CTA pushes its largest remaining column norm to all of them; barrier;
+//   all choose the same pivot p (ties to the lower position as in qrcp_kernel);
+//   p's owner forms the reflector from its column as it stands and publishes it
+//   with the part above the diagonal, k's owner sends its column to p's; barrier;
+//   every CTA copies the reflector, k's owner keeps it as column k, p's owner
+//   takes the column that was there; every CTA applies H_k to its columns.
+// The application is bound by the FP64 units (an instruction holds one for 64
+// cycles a warp), so what is not an FMA of the update counts: a warp takes four
+// columns at a time, their four dot products share one 6-instruction tree
+// (5 each before), and the rest of the step's arithmetic (row k, the norm's
+// downdate) is done once for the four, a column per 8 lanes.  The norms need
+// only row k, so they are downdated, and the candidates on their way, before
+// the columns themselves are updated.
+// Measured (GB300, one step's QRs of the YC4 cylinder at m = 1024, sectors of up
+// to 566 columns): 13.3 -> 10.7 ms against three barriers a step and columns one
+// by one; kagome cylinder at m = 1000, 18.1 -> 14.5 ms; random chain at m = 256,
+// latency bound, 1.10 -> 1.07 ms.  The FMAs alone are 2.0 ms of the largest
+// sector's 2.6 on its 16 SMs.
 // Exponent and FP32 mantissa of a double, by integer operations only (an
 // FP64 instruction costs 64 cycles of its sub-partition's FP64 unit here):
 // x = m 2^e with |m| in [1, 2) (mantissa truncated to 23 bits); zero and
@@ -269,6 +282,19 @@ __device__ __forceinline__ double recip_signed(double x) {
 constexpr int QC_THREADS = 256;
 constexpr int QC_MAX_CLUSTER = 16;
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// sums over the warp of four values per lane; lane gets that of value lane / 8
+__device__ __forceinline__ double wsum4(const double (&a)[4], int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8;
+  const double b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h16 ? a[0] : a[2], 16);
+  const double b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h16 ? a[1] : a[3], 16);
+  double c = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
 // GCOLS: the columns stay in global memory (the job's A) instead of the
 // CTAs' shared memory, for sectors too large for a cluster's shared memory;
 // the algorithm and the cluster's division of labour are the same.
@@ -292,10 +318,14 @@ __global__ void __launch_bounds__(QC_THREADS)
   double *bcast = cols + (GCOLS ? (size_t)0 : (size_t)nloc * ld);  // [ld] reflector of the step
   double *swp = bcast + ld;                      // [ld] incoming column of a swap
   double *vn = swp + ld, *vref = vn + nloc;      // [nloc] squared norms
-  int *pl = (int *)(vref + nloc);                // [nloc] original column at each position
-  __shared__ double cand_v[QC_MAX_CLUSTER], red_v[QC_THREADS / 32], s_tau, s_beta, s_scale, s_swap_vn, s_swap_vref;
-  __shared__ int cand_i[QC_MAX_CLUSTER], s_piv, s_stop, s_swap_pl;
-  __shared__ double s_vp, s_stop2;
+  double *wl = vref + nloc;                      // [nloc] the step's multiples of the reflector
+  int *pl = (int *)(wl + nloc);                  // [nloc] original column at each position
+  __shared__ double red_v[QC_THREADS / 32], s_tau, s_beta, s_scale;
+  // written by other CTAs: candidates; tau of the step; column k's data for p's
+  // owner (in) and the pivot's original index for k's owner (out)
+  __shared__ longlong2 cand[QC_MAX_CLUSTER];  // (squared norm's bits, position)
+  __shared__ int s_in_pl, s_out_pl;
+  __shared__ double s_tk, s_in_vn, s_in_vref;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   auto pos = [&](int l) { return crank + C * l; };
   // column at local slot l: shared memory, or the job's A in global memory
@@ -322,17 +352,10 @@ __global__ void __launch_bounds__(QC_THREADS)
       pl[l] = j;
     }
   }
-  if (threadIdx.x == 0) s_stop2 = -1.0;
-  __syncthreads();
-  double *cand_v0 = cluster.map_shared_rank(cand_v, 0);
-  int *cand_i0 = cluster.map_shared_rank(cand_i, 0);
-  int rank = ca;
-  for (int k = 0; k < ca; ++k) {
-    // (a) pivot: local candidate, gathered in rank 0, the same choice
-    // everywhere.  The squared norms are non-negative, so they order like
-    // their bit patterns as 64-bit integers: the comparisons run on the
-    // integer units (an FP64 compare costs 64 cycles of the FP64 unit here).
-    // A CTA holds at most a few dozen columns: warp 0 scans them.
+  // The squared norms are non-negative, so they order like their bit patterns
+  // as 64-bit integers: the comparisons run on the integer units.  A CTA holds
+  // at most a few dozen columns: warp 0 scans them.
+  auto push_candidate = [&](int k) {
     if (warp == 0) {
       long long bv = -1;
       int bi = 0x7fffffff;
@@ -349,91 +372,52 @@ __global__ void __launch_bounds__(QC_THREADS)
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
       }
-      if (lane == 0) {
-        cand_v0[crank] = __longlong_as_double(bv);
-        cand_i0[crank] = bi;
-      }
+      if (lane < C) cluster.map_shared_rank(cand, lane)[crank] = make_longlong2(bv, bi);
     }
-    cluster.sync();
-    if (warp == 0) {  // one lane per CTA reads its candidate (remote loads in parallel)
-      long long v = lane < C ? __double_as_longlong(cand_v0[lane]) : -1;
-      int idx = lane < C ? cand_i0[lane] : 0x7fffffff;
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-      }
-      if (lane == 0) {
-        const double vd = __longlong_as_double(v);
-        s_piv = idx;
-        s_vp = vd;
-        if (k == 0) s_stop2 = vd * (0.01 * zero_rel * zero_rel / (double)ca);
-        s_stop = !(v >= 0 && v > __double_as_longlong(s_stop2));
-      }
+  };
+  __syncthreads();
+  cluster.sync();  // every CTA of the cluster runs before any is written to
+  push_candidate(0);
+  cluster_arrive();
+  int rank = ca;
+  long long stop2 = 0;
+  const int nl = max(0, (ca - crank + C - 1) / C);  // columns held here
+  for (int k = 0; k < ca; ++k) {
+    cluster_wait();
+    __syncthreads();  // (the columns' updates, which are not behind the cluster barrier)
+    // (a) the pivot, the same in every warp of every CTA
+    long long v = -1;
+    int p = 0x7fffffff;
+    if (lane < C) {
+      const longlong2 x = cand[lane];
+      v = x.x;
+      p = (int)x.y;
     }
-    __syncthreads();
-    if (s_stop) {  // the same decision in every CTA: numerical rank reached
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ov > v || (ov == v && oi < p)) { v = ov; p = oi; }
+    }
+    if (k == 0) stop2 = __double_as_longlong(__longlong_as_double(v) * (0.01 * zero_rel * zero_rel / (double)ca));
+    if (!(v >= 0 && v > stop2)) {  // numerical rank reached
       rank = k;
       break;
     }
-    const int p = s_piv;
     const int ok = k % C, op = p % C, lk = k / C, lp = p / C;
-    // (b) swap positions k and p
-    if (p != k) {
-      if (ok == op) {
-        if (crank == ok) {
-          double *ck = colp(lk), *cp = colp(lp);
-          for (int i = threadIdx.x; i < ra; i += blockDim.x) {
-            const double t = ck[i];
-            ck[i] = cp[i];
-            cp[i] = t;
-          }
-          if (threadIdx.x == 0) {
-            double t = vn[lk]; vn[lk] = vn[lp]; vn[lp] = t;
-            t = vref[lk]; vref[lk] = vref[lp]; vref[lp] = t;
-            const int ti = pl[lk]; pl[lk] = pl[lp]; pl[lp] = ti;
-          }
-        }
-        cluster.sync();  // every CTA passes the same barriers
-      } else {
-        // each owner writes its column into the other's swap buffer (with
-        // global columns the owner of k swaps both columns in place)
-        if (crank == ok || crank == op) {
-          const int mine = crank == ok ? lk : lp, other = crank == ok ? op : ok;
-          if (!GCOLS) {
-            double *dst = cluster.map_shared_rank(swp, other);
-            for (int i = threadIdx.x; i < ra; i += blockDim.x) dst[i] = cols[(size_t)mine * ld + i];
-          } else if (crank == ok) {
-            double *ck = A + (int64_t)k * ra, *cp = A + (int64_t)p * ra;
-            for (int i = threadIdx.x; i < ra; i += blockDim.x) {
-              const double t = ck[i];
-              ck[i] = cp[i];
-              cp[i] = t;
-            }
-          }
-          if (threadIdx.x == 0) {
-            *cluster.map_shared_rank(&s_swap_vn, other) = vn[mine];
-            *cluster.map_shared_rank(&s_swap_vref, other) = vref[mine];
-            *cluster.map_shared_rank(&s_swap_pl, other) = pl[mine];
-          }
-        }
-        cluster.sync();
-        if (crank == ok || crank == op) {
-          const int mine = crank == ok ? lk : lp;
-          if (!GCOLS)
-            for (int i = threadIdx.x; i < ra; i += blockDim.x) cols[(size_t)mine * ld + i] = swp[i];
-          if (threadIdx.x == 0) {
-            vn[mine] = s_swap_vn;
-            vref[mine] = s_swap_vref;
-            pl[mine] = s_swap_pl;
-          }
-        }
+    // (b) column k to the owner of p
+    if (p != k && crank == ok) {
+      const double *ck = colp(lk);
+      double *dst = cluster.map_shared_rank(swp, op);
+      for (int i = threadIdx.x; i < ra; i += blockDim.x) dst[i] = ck[i];
+      if (threadIdx.x == 0) {
+        *cluster.map_shared_rank(&s_in_vn, op) = vn[lk];
+        *cluster.map_shared_rank(&s_in_vref, op) = vref[lk];
+        *cluster.map_shared_rank(&s_in_pl, op) = pl[lk];
       }
-      __syncthreads();
     }
-    // (c) the owner of position k forms the reflector (rows k..ra-1)
-    if (crank == ok) {
-      double *ak = colp(lk);
+    // (c) the owner of p forms the reflector (rows k..ra-1)
+    if (crank == op) {
+      double *ak = colp(lp);
       double s2 = 0.0;
       for (int i = k + 1 + threadIdx.x; i < ra; i += blockDim.x) s2 = fma(ak[i], ak[i], s2);
       s2 = wsum(s2);
@@ -462,50 +446,120 @@ __global__ void __launch_bounds__(QC_THREADS)
       }
       __syncthreads();
       const double sc = s_scale;
-      if (s_tau != 0.0)
-        for (int i = k + 1 + threadIdx.x; i < ra; i += blockDim.x) ak[i] *= sc;
-      __syncthreads();
-      if (threadIdx.x == 0) ak[k] = s_beta;
-      for (int i = k + 1 + threadIdx.x; i < ra; i += blockDim.x) bcast[i] = ak[i];
+      const bool on = s_tau != 0.0;
+      // column k as it will be stored: R above the diagonal, beta, the reflector
+      for (int i = (p == k ? k : 0) + threadIdx.x; i < ra; i += blockDim.x) {
+        double x = ak[i];
+        if (i == k) x = s_beta;
+        if (i > k && on) x *= sc;
+        bcast[i] = x;
+        if (p == k) ak[i] = x;
+      }
+      if (threadIdx.x < C) *cluster.map_shared_rank(&s_tk, threadIdx.x) = s_tau;
+      if (threadIdx.x == 0 && p != k) *cluster.map_shared_rank(&s_out_pl, ok) = pl[lp];
     }
     cluster.sync();  // reflector published
-    // (d) every CTA applies H_k to its own trailing columns
-    const double tk = *cluster.map_shared_rank(&s_tau, ok);
-    if (tk != 0.0) {
-      if (crank != ok) {
-        const double *src = cluster.map_shared_rank(bcast, ok);
-        for (int i = k + 1 + threadIdx.x; i < ra; i += blockDim.x) bcast[i] = src[i];
-        __syncthreads();
-      }
-      for (int l = warp; l < nloc; l += nw) {
-        const int j = pos(l);
-        if (j <= k || j >= ca) continue;
-        double *aj = colp(l);
-        double w = 0.0;
-        for (int i = k + 1 + lane; i < ra; i += 32) w = fma(bcast[i], aj[i], w);
-        w = (wsum(w) + aj[k]) * tk;
-        __syncwarp();
-        if (lane == 0) aj[k] -= w;
-        for (int i = k + 1 + lane; i < ra; i += 32) aj[i] = fma(-w, bcast[i], aj[i]);
-      }
-      __syncthreads();
+    const double tk = s_tk;
+    // (d) the reflector here, the swapped columns in their places
+    {
+      const double *src = cluster.map_shared_rank(bcast, op);
+      const bool keep = p != k && crank == ok;
+      double *ck = keep ? colp(lk) : nullptr;
+      if (keep || crank != op)
+        for (int i = (keep ? 0 : k + 1) + threadIdx.x; i < ra; i += blockDim.x) {
+          const double x = src[i];
+          if (crank != op) bcast[i] = x;
+          if (keep) ck[i] = x;
+        }
+      if (keep && threadIdx.x == 0) pl[lk] = s_out_pl;
     }
-    // downdate the remaining column norms; recompute where cancellation hurts
-    for (int l = warp; l < nloc; l += nw) {
-      const int j = pos(l);
-      if (j <= k || j >= ca) continue;
-      const double *aj = colp(l);
-      double nv = vn[l] - aj[k] * aj[k];
-      if (!(nv > 1e-8 * vref[l])) {
-        double s2 = 0.0;
-        for (int i = k + 1 + lane; i < ra; i += 32) s2 = fma(aj[i], aj[i], s2);
-        nv = wsum(s2);
-        if (lane == 0) vref[l] = nv;
+    if (p != k && crank == op) {
+      double *cp = colp(lp);
+      for (int i = threadIdx.x; i < ra; i += blockDim.x) cp[i] = swp[i];
+      if (threadIdx.x == 0) {
+        vn[lp] = s_in_vn;
+        vref[lp] = s_in_vref;
+        pl[lp] = s_in_pl;
       }
-      if (lane == 0) vn[l] = fmax(nv, 0.0);
     }
     __syncthreads();
+    // (e) H_k on the columns after k: w_j = tau (a_kj + v . a_j), row k and the norms
+    const int l0 = max(0, (k - crank + C) / C);  // first slot with position > k
+    for (int lb = l0 + warp; lb < nl; lb += 4 * nw) {
+      const int n = min(4, (nl - lb + nw - 1) / nw);
+      const double *c0 = colp(lb);
+      const size_t cs = (size_t)nw * (GCOLS ? (size_t)C * ra : (size_t)ld);
+      auto dots = [&](auto tag) {
+        constexpr int NC = decltype(tag)::value;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        if (tk != 0.0) {
+          for (int i = k + 1 + lane; i < ra; i += 32) {
+            const double x = bcast[i];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c] = fma(x, c0[c * cs + i], acc[c]);
+          }
+        }
+        return NC == 1 ? wsum(acc[0]) : wsum4(acc, lane);
+      };
+      const double sum = n == 1   ? dots(std::integral_constant<int, 1>{})
+                         : n == 2 ? dots(std::integral_constant<int, 2>{})
+                         : n == 3 ? dots(std::integral_constant<int, 3>{})
+                                  : dots(std::integral_constant<int, 4>{});
+      const int l = lb + (lane >> 3) * nw;
+      const bool mine = (lane >> 3) < n;
+      double w = 0.0, r = 0.0, nv = 0.0;
+      bool again = false;
+      if (mine) {
+        const double ak = colp(l)[k];
+        w = (sum + ak) * tk;
+        r = ak - w;
+        nv = fma(-r, r, vn[l]);
+        // recompute where cancellation hurts (or nv is not a number)
+        const long long nb = __double_as_longlong(nv);
+        again = !(nb > __double_as_longlong(1e-8 * vref[l])) || nb > 0x7ff0000000000000ll;
+      }
+      __syncwarp();
+      if (mine && (lane & 7) == 0) {
+        colp(l)[k] = r;
+        wl[l] = w;
+        vn[l] = nv;
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, again);
+      __syncwarp();
+      while (todo) {  // (uniform)
+        const int c = (__ffs(todo) - 1) >> 3, lc = lb + c * nw;
+        todo &= ~(0xffu << (8 * c));
+        double *aj = colp(lc);
+        const double wc = wl[lc];
+        double s2 = 0.0;
+        for (int i = k + 1 + lane; i < ra; i += 32) {
+          const double x = fma(-wc, bcast[i], aj[i]);
+          aj[i] = x;
+          s2 = fma(x, x, s2);
+        }
+        s2 = wsum(s2);
+        __syncwarp();
+        if (lane == 0) {
+          vn[lc] = fmax(s2, 0.0);
+          vref[lc] = s2;
+          wl[lc] = 0.0;  // updated
+        }
+      }
+    }
+    __syncthreads();
+    push_candidate(k + 1);
+    cluster_arrive();
+    if (tk != 0.0) {
+      for (int l = l0 + warp; l < nl; l += nw) {
+        const double w = wl[l];
+        if ((__double_as_longlong(w) << 1) == 0) continue;
+        double *aj = colp(l);
+        for (int i = k + 1 + lane; i < ra; i += 32) aj[i] = fma(-w, bcast[i], aj[i]);
+      }
+    }
   }
+  if (rank == ca) cluster_wait();  // (the last step's arrival)
+  __syncthreads();
   // Householder vectors, R, the permutation, the rank; B = [R11 R12]^T
   for (int l = 0; l < nloc; ++l) {
     const int j = pos(l);
@@ -2917,14 +2971,14 @@ cudaError_t launch_svd_refine(SvdRefine part, const SvdJob *jobs, const int *ord
 
 size_t svd_qrc_smem(int rows, int cols, int csize) {
   const int64_t nloc = (cols + csize - 1) / csize, ld = (rows + 1) & ~1;
-  return (size_t)((nloc * ld + 2 * ld + 3 * nloc + 2) * sizeof(double));
+  return (size_t)((nloc * ld + 2 * ld + 4 * nloc + 2) * sizeof(double));
 }
 
 // the same with the columns in global memory (reflector, swap buffer and the
 // per-column norms in shared memory)
 static size_t svd_qrc_smem_global(int rows, int cols, int csize) {
   const int64_t nloc = (cols + csize - 1) / csize, ld = (rows + 1) & ~1;
-  return (size_t)((2 * ld + 3 * nloc + 2) * sizeof(double));
+  return (size_t)((2 * ld + 4 * nloc + 2) * sizeof(double));
 }
 
 // pivoted QR of the jobs order[0..njobs) in groups (as the Jacobi): groups
