@@ -2710,6 +2710,33 @@ size_t svd_block_smem(int cols, int csize) {
   return (size_t)(4 * (bw * (2 * pad + 2) + 1) * sizeof(double));
 }
 
+// Group 1 beside group 0: its cluster size.  The chip holds SVD_CLUSTERS_16
+// clusters of 16 CTAs that take a whole SM each (clusters stay inside a GPC) and
+// twice as many and one of 8; when groups 0 and 1 are more jobs than that, 8 CTAs
+// per job of group 1 use the SMs that no cluster of 16 fits on, and leave those
+// to group 0.  A job's time is largely its chain of barriers, so halving its SMs
+// costs it little.  Jacobi CTAs small enough to share an SM gain nothing from it
+// and keep 16.  Measured (GB300, ms of a step, all groups; before: 16 CTAs, group
+// 1 after group 0 on one stream): J1-J2 cylinder at m = 1024 QR 10.7 -> 9.5, FP32
+// Jacobi 21.7 -> 20.4, final Jacobi 7.4 -> 6.0; kagome at m = 1000 FP32 Jacobi
+// 31.0 -> 28.7; sectors of 148 columns (random chain, m = 256) QR 1.07 -> 1.01,
+// FP32 Jacobi 1.12 with 16 CTAs, 1.66 with 8.
+constexpr int SVD_CLUSTERS_16 = 7;
+constexpr size_t SVD_SHARED_SM = 64 * 1024;  // at least three such CTAs on an SM
+static int group1_csize(int jobs01, bool crowded, bool fits8) {
+  return jobs01 > SVD_CLUSTERS_16 && crowded && fits8 ? 8 : 16;
+}
+// the stream that runs group k (group 0: the caller's) and the event that ends it
+static int group_side(int k) { return k == 1 ? 3 : k - 2; }
+static cudaError_t join_groups(const int (&lo)[5], const int (&hi)[5], cudaStream_t st, const cudaEvent_t *ev) {
+  for (int k = 1; k < 5; ++k) {
+    if (hi[k] <= lo[k]) continue;
+    const cudaError_t e = cudaStreamWaitEvent(st, ev[k], 0);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaGetLastError();
+}
+
 // block kernel for jobs of at most `cols` columns on clusters of `csize`
 static cudaError_t launch_block_clusters(const SvdJob *jobs, const int *order, int njobs, int csize, int cols,
                                          double *work, int *iwork, double *sv, int *err, int jm_init,
@@ -2739,9 +2766,9 @@ static cudaError_t launch_block_clusters(const SvdJob *jobs, const int *order, i
 // [g[k-1], g[k]) (g[-1] = 0, g[4] = njobs): 0 Jacobi in global memory on
 // 16-CTA clusters (columns beyond the shared memory of the block kernel),
 // 1..4 block Jacobi on clusters of 16, 8, 4 and 1 CTAs; cols[k-1] is the
-// largest column count of block group k.  Groups 0 and 1 run on `st`, the others on the side
-// streams side[0..2], forked from and joined back to `st` by the events
-// ev[0..3].  pairs: group 0 in FP32-pair arithmetic (jacobi_scaled_kernel).
+// largest column count of block group k.  Group 0 runs on `st`, the others on
+// the side streams side[0..3], forked from and joined back to `st` by the events
+// ev[0..4].  pairs: group 0 in FP32-pair arithmetic (jacobi_scaled_kernel).
 cudaError_t launch_svd_jacobi(const SvdJob *jobs, const int *order, int njobs, const int *g, const int *cols,
                               double *work, int *iwork, double *sv, int *err, int jm_init, bool pairs,
                               cudaStream_t st, const cudaStream_t *side, const cudaEvent_t *ev) {
@@ -2753,19 +2780,9 @@ cudaError_t launch_svd_jacobi(const SvdJob *jobs, const int *order, int njobs, c
   if (e != cudaSuccess) return e;
   cudaGetLastError();
   const int lo[5] = {0, g[0], g[1], g[2], g[3]}, hi[5] = {g[0], g[1], g[2], g[3], njobs};
-  const int csz[5] = {16, 16, 8, 4, 1};
   e = cudaEventRecord(ev[0], st);
   if (e != cudaSuccess) return e;
-  for (int k = 2; k < 5; ++k) {
-    if (hi[k] <= lo[k]) continue;
-    e = cudaStreamWaitEvent(side[k - 2], ev[0], 0);
-    if (e != cudaSuccess) return e;
-    e = launch_block_clusters(jobs, order + lo[k], hi[k] - lo[k], csz[k], cols[k - 1], work, iwork, sv, err,
-                              jm_init, side[k - 2]);
-    if (e != cudaSuccess) return e;
-    e = cudaEventRecord(ev[k - 1], side[k - 2]);
-    if (e != cudaSuccess) return e;
-  }
+  // the largest sectors first: a cluster of theirs needs a GPC's SMs free
   if (hi[0] > lo[0]) {
     cudaFuncSetAttribute(jacobi_scaled_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(jacobi_scaled_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -2776,21 +2793,25 @@ cudaError_t launch_svd_jacobi(const SvdJob *jobs, const int *order, int njobs, c
     }
     if (e != cudaSuccess) return e;
   }
-  if (hi[1] > lo[1]) {
-    e = launch_block_clusters(jobs, order + lo[1], hi[1] - lo[1], 16, cols[0], work, iwork, sv, err, jm_init, st);
-    if (e != cudaSuccess) {
+  const int csz[5] = {16, group1_csize(hi[1], svd_block_smem(cols[0], 16) > SVD_SHARED_SM,
+                                           svd_block_smem(cols[0], 8) <= SVD_BLOCK_SMEM_MAX), 8, 4, 1};
+  for (int k = 1; k < 5; ++k) {
+    if (hi[k] <= lo[k]) continue;
+    const cudaStream_t sk = side[group_side(k)];
+    e = cudaStreamWaitEvent(sk, ev[0], 0);
+    if (e != cudaSuccess) return e;
+    e = launch_block_clusters(jobs, order + lo[k], hi[k] - lo[k], csz[k], cols[k - 1], work, iwork, sv, err,
+                              jm_init, sk);
+    if (e != cudaSuccess && k == 1) {
       // 16-CTA clusters not available: the global-memory kernel on 8
       cudaGetLastError();
-      e = launch_jacobi_clusters(jobs, order + lo[1], hi[1] - lo[1], 8, work, iwork, sv, err, jm_init, st);
+      e = launch_jacobi_clusters(jobs, order + lo[1], hi[1] - lo[1], 8, work, iwork, sv, err, jm_init, sk);
     }
     if (e != cudaSuccess) return e;
-  }
-  for (int k = 2; k < 5; ++k) {
-    if (hi[k] <= lo[k]) continue;
-    e = cudaStreamWaitEvent(st, ev[k - 1], 0);
+    e = cudaEventRecord(ev[k], sk);
     if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return join_groups(lo, hi, st, ev);
 }
 
 cudaError_t launch_svd_select(const SvdJob *jobs, const int *sb_job0, const int *sb_njob, int S, const double *sv,
@@ -2824,12 +2845,16 @@ cudaError_t launch_svd_compact(const SvdJob *jobs, const CompactJob *cj, int ncj
   return cudaGetLastError();
 }
 
+static size_t block32_smem(int cols, int csize) {
+  const int64_t bw = (cols + 2 * csize - 1) / (2 * csize), pad = 32 * (((int64_t)cols + 31) / 32);
+  return (size_t)(4 * ((bw * 2 * pad + 3) & ~(int64_t)3) * sizeof(float));
+}
 static cudaError_t launch_block32_clusters(const SvdJob *jobs, const int *order, int njobs, int csize, int cols,
                                            double *work, const int *iwork, cudaStream_t st) {
   const int bw = (cols + 2 * csize - 1) / (2 * csize);
   const int warps = std::min(BJ_THREADS / 32, std::max(2, bw));
   const int64_t pad = 32 * (((int64_t)cols + 31) / 32);
-  const size_t smem = (size_t)(4 * ((bw * 2 * pad + 3) & ~(int64_t)3) * sizeof(float));
+  const size_t smem = block32_smem(cols, csize);
   if (pad > 32 * BJ_REG || smem > SVD_BLOCK_SMEM_MAX) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(njobs * csize, 1, 1);
@@ -2888,21 +2913,11 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
                                        (int)SVD_BLOCK_SMEM_MAX);
   if (e != cudaSuccess) return e;
   const int lo[5] = {0, g[0], g[1], g[2], g[3]}, hi[5] = {g[0], g[1], g[2], g[3], njobs};
-  const int csz[5] = {16, 16, 8, 4, 1};
   e = cudaEventRecord(ev[0], st);
   if (e != cudaSuccess) return e;
-  for (int k = 2; k < 5; ++k) {
-    if (hi[k] <= lo[k]) continue;
-    e = cudaStreamWaitEvent(side[k - 2], ev[0], 0);
-    if (e != cudaSuccess) return e;
-    e = launch_block32_clusters(jobs, order + lo[k], hi[k] - lo[k], csz[k], cols[k - 1], work, iwork, side[k - 2]);
-    if (e != cudaSuccess) return e;
-    e = cudaEventRecord(ev[k - 1], side[k - 2]);
-    if (e != cudaSuccess) return e;
-  }
   // beyond the block kernels: the block tournament streamed through shared
   // memory; the all-global pair kernel if asked for, or if that launch is not
-  // possible (no 16-CTA clusters)
+  // possible (no 16-CTA clusters).  First: a cluster of 16 needs a GPC's SMs free
   if (hi[0] > lo[0]) {
     e = launch_jacobi32_stream(jobs, order, hi[0], cols0, 16, work, iwork, st);
     if (e != cudaSuccess) {
@@ -2916,16 +2931,19 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
     }
     if (e != cudaSuccess) return e;
   }
-  if (hi[1] > lo[1]) {
-    e = launch_block32_clusters(jobs, order + lo[1], hi[1] - lo[1], 16, cols[0], work, iwork, st);
-    if (e != cudaSuccess) return e;
-  }
-  for (int k = 2; k < 5; ++k) {
+  const int csz[5] = {16, group1_csize(hi[1], block32_smem(cols[0], 16) > SVD_SHARED_SM,
+                                           block32_smem(cols[0], 8) <= SVD_BLOCK_SMEM_MAX), 8, 4, 1};
+  for (int k = 1; k < 5; ++k) {
     if (hi[k] <= lo[k]) continue;
-    e = cudaStreamWaitEvent(st, ev[k - 1], 0);
+    const cudaStream_t sk = side[group_side(k)];
+    e = cudaStreamWaitEvent(sk, ev[0], 0);
+    if (e != cudaSuccess) return e;
+    e = launch_block32_clusters(jobs, order + lo[k], hi[k] - lo[k], csz[k], cols[k - 1], work, iwork, sk);
+    if (e != cudaSuccess) return e;
+    e = cudaEventRecord(ev[k], sk);
     if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return join_groups(lo, hi, st, ev);
 }
 
 cudaError_t launch_svd_elementwise(const SvdJob *jobs, int njobs, int max_cols, int mode, double *work, int *iwork,
@@ -2982,7 +3000,7 @@ static size_t svd_qrc_smem_global(int rows, int cols, int csize) {
 }
 
 // pivoted QR of the jobs order[0..njobs) in groups (as the Jacobi): groups
-// 0..4 on clusters of 16, 16, 8, 4, 1 CTAs; a group whose columns do not fit
+// 0..4 on clusters of 16, 16 or 8 (group1_csize), 8, 4, 1 CTAs; a group whose columns do not fit
 // in the shared memory of its cluster keeps them in global memory
 // (force_global_cols: every clustered group does), one that does not fit
 // either way runs on the single-CTA kernel; rows[k], cols[k] are the
@@ -2999,14 +3017,14 @@ cudaError_t launch_svd_qrcp_grouped(const SvdJob *jobs, const int *order, int nj
   }
   cudaError_t e = cudaSuccess;
   const int lo[5] = {0, g[0], g[1], g[2], g[3]}, hi[5] = {g[0], g[1], g[2], g[3], njobs};
-  const int csz[5] = {16, 16, 8, 4, 1};
-  // groups 2..4 on the side streams, concurrent with groups 0 and 1
+  const int csz[5] = {16, group1_csize(hi[1], true, svd_qrc_smem(rows[0], cols[0], 8) <= SVD_BLOCK_SMEM_MAX), 8, 4, 1};
+  // groups 1..4 on the side streams, concurrent with group 0
   e = cudaEventRecord(ev[0], st);
   if (e != cudaSuccess) return e;
   for (int k = 0; k < 5; ++k) {
     if (hi[k] <= lo[k]) continue;
-    const cudaStream_t sk = k >= 2 ? side[k - 2] : st;
-    if (k >= 2) {
+    const cudaStream_t sk = k >= 1 ? side[group_side(k)] : st;
+    if (k >= 1) {
       e = cudaStreamWaitEvent(sk, ev[0], 0);
       if (e != cudaSuccess) return e;
     }
@@ -3034,17 +3052,12 @@ cudaError_t launch_svd_qrcp_grouped(const SvdJob *jobs, const int *order, int nj
                                            zero_rel);
     }
     if (e != cudaSuccess) return e;
-    if (k >= 2) {
-      e = cudaEventRecord(ev[k - 1], sk);
+    if (k >= 1) {
+      e = cudaEventRecord(ev[k], sk);
       if (e != cudaSuccess) return e;
     }
   }
-  for (int k = 2; k < 5; ++k) {
-    if (hi[k] <= lo[k]) continue;
-    e = cudaStreamWaitEvent(st, ev[k - 1], 0);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  return join_groups(lo, hi, st, ev);
 }
 
 }  // namespace idmrg
