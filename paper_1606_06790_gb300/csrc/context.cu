@@ -61,7 +61,16 @@ struct SBPlan {
   int64_t t1size = 0, t3size = 0, xsize = 0, ysize = 0;
   std::vector<int64_t> t1off, t3off;
   std::vector<int> t3C, t3col;
-  std::vector<double> W12;  // [wa][wc][d*d][d*d]
+  // Non-zeros of the two-site MPO W12[a][c][(s,t)][(s',t')], one run per (c,
+  // (s,t)), in the order of a, then (s',t'): nine tenths of it and more are
+  // zeros, and three task lists go over it for every left sector.
+  struct W12Nz {
+    int a, st2;
+    double coef;
+  };
+  std::vector<W12Nz> w12;
+  std::vector<int> w12_run;  // [wc * d*d + 1] starts
+  std::vector<int> lsi;      // [wa][SL]: the in-sector of L_a's block with out-sector i, or -1
   std::vector<double> h2;   // centre bond operator [d*d][d*d]
   double heff_flops = 0, heff_bytes = 0;
   double gemm_flops = 0, w_flops = 0;
@@ -740,6 +749,7 @@ idmrg_status plan_iteration(idmrg_ctx *c) {
   c->rblocks.clear();
   c->rmax_rows = 0;
   const uint64_t state0 = c->o.seed;
+  std::vector<double> W12;
   for (int p = 0; p < P; ++p) {
     if (!c->owns(p)) continue;  // another worker's superblock
     SBPlan &S = c->plan[p];
@@ -755,7 +765,7 @@ idmrg_status plan_iteration(idmrg_ctx *c) {
       return c->fail(IDMRG_EINVAL, "MPO bond dimensions do not chain at superblock %d", p);
     // two-site MPO W12[a][c][(s,t)][(s',t')] = sum_b W_c1(a,b) W_c2(b,c)
     const int dd = d * d;
-    S.W12.assign((size_t)wa * wc * dd * dd, 0.0);
+    W12.assign((size_t)wa * wc * dd * dd, 0.0);
     for (int a = 0; a < wa; ++a)
       for (int b = 0; b < wb; ++b)
         for (int s = 0; s < d; ++s)
@@ -767,9 +777,26 @@ idmrg_status plan_iteration(idmrg_ctx *c) {
                 for (int t2 = 0; t2 < d; ++t2) {
                   const double w2 = c->Wat(S.c2, b, cc, t, t2);
                   if (w2 == 0.0) continue;
-                  S.W12[(((size_t)a * wc + cc) * dd + s * d + t) * dd + s2 * d + t2] += w1 * w2;
+                  W12[(((size_t)a * wc + cc) * dd + s * d + t) * dd + s2 * d + t2] += w1 * w2;
                 }
           }
+    S.w12.clear();
+    S.w12_run.assign(1, 0);
+    for (int cc = 0; cc < wc; ++cc)
+      for (int st = 0; st < dd; ++st) {
+        for (int a = 0; a < wa; ++a)
+          for (int st2 = 0; st2 < dd; ++st2) {
+            const double cf = W12[(((size_t)a * wc + cc) * dd + st) * dd + st2];
+            if (cf != 0.0) S.w12.push_back({a, st2, cf});
+          }
+        S.w12_run.push_back((int)S.w12.size());
+      }
+    S.lsi.assign((size_t)wa * BL.S(), -1);
+    for (int a = 0; a < wa; ++a)
+      for (int i = 0; i < BL.S(); ++i) {
+        const int si = BL.find(BL.q[i] - L.lay.chq[a]);
+        if (si >= 0 && L.lay.so[a * BL.S() + si] == i) S.lsi[a * BL.S() + i] = si;
+      }
     // centre-bond operator: channels opened on c1 and closed on c2
     S.h2.assign((size_t)dd * dd, 0.0);
     for (int b = 1; b < wb - 1; ++b)
@@ -827,17 +854,13 @@ idmrg_status plan_iteration(idmrg_ctx *c) {
             const int qsum = BL.q[i] + c->qp[s] + c->qp[t];
             const int jin = BR.find(target - qsum - R.lay.chq[cc]);
             c->wl.task(p, BUF_T3, S.t3off[cc * SL + i] + col, S.t3C[cc * SL + i], BUF_T1, BL.dim[i], BR.dim[jin]);
-            for (int a = 0; a < wa; ++a) {
-              const int si = BL.find(BL.q[i] - L.lay.chq[a]);
-              if (si < 0 || L.lay.so[a * SL + si] != i || S.t1off[a * SL + si] < 0) continue;
-              for (int s2 = 0; s2 < d; ++s2)
-                for (int t2 = 0; t2 < d; ++t2) {
-                  const double cf = S.W12[(((size_t)a * wc + cc) * dd + s * d + t) * dd + s2 * d + t2];
-                  if (cf == 0.0) continue;
-                  const int k = psi.sub(si, s2, t2);
-                  if (psi.sj[k] != jin) continue;
-                  c->wl.term(S.t1off[a * SL + si] + psi.scol[k], psi.C[si], cf);
-                }
+            for (int z = S.w12_run[cc * dd + s * d + t]; z < S.w12_run[cc * dd + s * d + t + 1]; ++z) {
+              const SBPlan::W12Nz &w = S.w12[z];
+              const int si = S.lsi[w.a * SL + i];
+              if (si < 0 || S.t1off[w.a * SL + si] < 0) continue;
+              const int k = psi.sub(si, w.st2 / d, w.st2 % d);
+              if (psi.sj[k] != jin) continue;
+              c->wl.term(S.t1off[w.a * SL + si] + psi.scol[k], psi.C[si], w.coef);
             }
           }
     // ---- stage 3: out = sum_c T3[c] R_c^T
@@ -1188,24 +1211,20 @@ idmrg_status plan_mixed(idmrg_ctx *c) {
               if (ks[cc] < 0) continue;
               const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
               const int term0 = (int)c->wtpm.size();
-              for (int a = 0; a < wa; ++a) {
-                const int si = BL.find(BL.q[i] - L.lay.chq[a]);
-                if (si < 0 || L.lay.so[a * SL + si] != i || rs1[si][a] < 0) continue;
-                for (int s2 = 0; s2 < d; ++s2)
-                  for (int t2 = 0; t2 < d; ++t2) {
-                    const double cf = S.W12[(((size_t)a * wc + cc) * dd + s * d + t) * dd + s2 * d + t2];
-                    if (cf == 0.0) continue;
-                    const int k2 = psi.sub(si, s2, t2);
-                    if (psi.sj[k2] != jin) continue;
-                    WTerm term{};
-                    term.in_off = t1f[si] + (int64_t)rs1[si][a] * psi.C[si] + psi.scol[k2];
-                    term.in_ld = psi.C[si];
-                    term.k0 = ks[cc];
-                    term.cols = BR.dim[jin];
-                    term.coef = cf;
-                    term.coef32 = (float)cf;
-                    c->wtpm.push_back(term);
-                  }
+              for (int z = S.w12_run[cc * dd + s * d + t]; z < S.w12_run[cc * dd + s * d + t + 1]; ++z) {
+                const SBPlan::W12Nz &nz = S.w12[z];
+                const int si = S.lsi[nz.a * SL + i];
+                if (si < 0 || rs1[si][nz.a] < 0) continue;
+                const int k2 = psi.sub(si, nz.st2 / d, nz.st2 % d);
+                if (psi.sj[k2] != jin) continue;
+                WTerm term{};
+                term.in_off = t1f[si] + (int64_t)rs1[si][nz.a] * psi.C[si] + psi.scol[k2];
+                term.in_ld = psi.C[si];
+                term.k0 = ks[cc];
+                term.cols = BR.dim[jin];
+                term.coef = nz.coef;
+                term.coef32 = (float)nz.coef;
+                c->wtpm.push_back(term);
               }
               const int nterm = (int)c->wtpm.size() - term0;  // without terms the packed rectangle stays zero
               if (nterm > 0) rects.push_back(WRect{ks[cc], BR.dim[jin], term0, nterm});
@@ -1449,24 +1468,20 @@ idmrg_status plan_oz(idmrg_ctx *c) {
               if (ks[cc] < 0) continue;
               const int jin = BR.find(BR.q[jo] - R.lay.chq[cc]);
               const int term0 = (int)c->wtpm_oz.size();
-              for (int a = 0; a < wa; ++a) {
-                const int si = BL.find(BL.q[i] - L.lay.chq[a]);
-                if (si < 0 || L.lay.so[a * SL + si] != i || rs1[si][a] < 0) continue;
-                for (int s2 = 0; s2 < d; ++s2)
-                  for (int t2 = 0; t2 < d; ++t2) {
-                    const double cf = S.W12[(((size_t)a * wc + cc) * dd + s * d + t) * dd + s2 * d + t2];
-                    if (cf == 0.0) continue;
-                    const int k2 = psi.sub(si, s2, t2);
-                    if (psi.sj[k2] != jin) continue;
-                    WTerm term{};
-                    term.in_off = t1f[si] + (int64_t)rs1[si][a] * psi.C[si] + psi.scol[k2];
-                    term.in_ld = psi.C[si];
-                    term.k0 = ks[cc];
-                    term.cols = BR.dim[jin];
-                    term.coef = cf;
-                    term.coef32 = (float)cf;
-                    c->wtpm_oz.push_back(term);
-                  }
+              for (int z = S.w12_run[cc * dd + s * d + t]; z < S.w12_run[cc * dd + s * d + t + 1]; ++z) {
+                const SBPlan::W12Nz &nz = S.w12[z];
+                const int si = S.lsi[nz.a * SL + i];
+                if (si < 0 || rs1[si][nz.a] < 0) continue;
+                const int k2 = psi.sub(si, nz.st2 / d, nz.st2 % d);
+                if (psi.sj[k2] != jin) continue;
+                WTerm term{};
+                term.in_off = t1f[si] + (int64_t)rs1[si][nz.a] * psi.C[si] + psi.scol[k2];
+                term.in_ld = psi.C[si];
+                term.k0 = ks[cc];
+                term.cols = BR.dim[jin];
+                term.coef = nz.coef;
+                term.coef32 = (float)nz.coef;
+                c->wtpm_oz.push_back(term);
               }
               const int nterm = (int)c->wtpm_oz.size() - term0;  // without terms the packed rectangle stays zero
               if (nterm > 0) rects.push_back(WRect{ks[cc], BR.dim[jin], term0, nterm});
