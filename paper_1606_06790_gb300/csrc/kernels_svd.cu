@@ -11,7 +11,11 @@
 //            columns of B orthogonal, B Jm = U~ S.  Parallel round-robin
 //            ordering, one warp per column pair, the pairs of a round spread
 //            over a cluster of CTAs that meet at the hardware cluster barrier.
-//            Then A = (Q Jm) S (P U~)^T.
+//            Then A = (Q Jm) S (P U~)^T.  An FP32 stage runs it to overlaps of
+//            1e-6; Newton-Schulz makes its rotations orthogonal in 64 bits.
+//  refine  : two corrections of those rotations from the Gram matrices of the
+//            rotated columns, by matrix products, and a check; the FP64 sweeps
+//            run on the sectors that the check finds unfinished.
 //  select  : per superblock, sorts all singular values in descending order
 //            (ties by |Q|, Q, index), drops values at or below zero_rel*max,
 //            cuts at D <= m without splitting values closer than tie_rel, and
@@ -229,6 +233,9 @@ __global__ void __launch_bounds__(QR_THREADS) qrcp_kernel(const SvdJob *__restri
 // by one; kagome cylinder at m = 1000, 18.1 -> 14.5 ms; random chain at m = 256,
 // latency bound, 1.10 -> 1.07 ms.  The FMAs alone are 2.0 ms of the largest
 // sector's 2.6 on its 16 SMs.
+// Columns in global memory go two at a time and are updated at once, while L1
+// holds them (kagome cylinder at m = 2048, up to 1126 columns: 91 ms a step,
+// 99 with four at a time and the update after all dot products).
 // Exponent and FP32 mantissa of a double, by integer operations only (an
 // FP64 instruction costs 64 cycles of its sub-partition's FP64 unit here):
 // x = m 2^e with |m| in [1, 2) (mantissa truncated to 23 bits); zero and
@@ -382,6 +389,8 @@ __global__ void __launch_bounds__(QC_THREADS)
   int rank = ca;
   long long stop2 = 0;
   const int nl = max(0, (ca - crank + C - 1) / C);  // columns held here
+  // columns in global memory: two at a time, updated while L1 still holds them
+  constexpr int NB = GCOLS ? 2 : 4;
   for (int k = 0; k < ca; ++k) {
     cluster_wait();
     __syncthreads();  // (the columns' updates, which are not behind the cluster barrier)
@@ -485,8 +494,17 @@ __global__ void __launch_bounds__(QC_THREADS)
     __syncthreads();
     // (e) H_k on the columns after k: w_j = tau (a_kj + v . a_j), row k and the norms
     const int l0 = max(0, (k - crank + C) / C);  // first slot with position > k
-    for (int lb = l0 + warp; lb < nl; lb += 4 * nw) {
-      const int n = min(4, (nl - lb + nw - 1) / nw);
+    // the warp's columns from slot `lb` on, n of them at most
+    auto update = [&](int lb, int n) {
+      for (int l = lb; l < nl && n > 0; l += nw, --n) {
+        const double w = wl[l];
+        if ((__double_as_longlong(w) << 1) == 0) continue;
+        double *aj = colp(l);
+        for (int i = k + 1 + lane; i < ra; i += 32) aj[i] = fma(-w, bcast[i], aj[i]);
+      }
+    };
+    for (int lb = l0 + warp; lb < nl; lb += NB * nw) {
+      const int n = min(NB, (nl - lb + nw - 1) / nw);
       const double *c0 = colp(lb);
       const size_t cs = (size_t)nw * (GCOLS ? (size_t)C * ra : (size_t)ld);
       auto dots = [&](auto tag) {
@@ -501,10 +519,10 @@ __global__ void __launch_bounds__(QC_THREADS)
         }
         return NC == 1 ? wsum(acc[0]) : wsum4(acc, lane);
       };
-      const double sum = n == 1   ? dots(std::integral_constant<int, 1>{})
-                         : n == 2 ? dots(std::integral_constant<int, 2>{})
-                         : n == 3 ? dots(std::integral_constant<int, 3>{})
-                                  : dots(std::integral_constant<int, 4>{});
+      const double sum = n == 1              ? dots(std::integral_constant<int, 1>{})
+                         : n == 2            ? dots(std::integral_constant<int, 2>{})
+                         : n == 3 && NB == 4 ? dots(std::integral_constant<int, NB == 4 ? 3 : 2>{})
+                                             : dots(std::integral_constant<int, NB>{});
       const int l = lb + (lane >> 3) * nw;
       const bool mine = (lane >> 3) < n;
       double w = 0.0, r = 0.0, nv = 0.0;
@@ -544,19 +562,14 @@ __global__ void __launch_bounds__(QC_THREADS)
           vref[lc] = s2;
           wl[lc] = 0.0;  // updated
         }
+        __syncwarp();
       }
+      if (GCOLS && tk != 0.0) update(lb, n);
     }
     __syncthreads();
     push_candidate(k + 1);
     cluster_arrive();
-    if (tk != 0.0) {
-      for (int l = l0 + warp; l < nl; l += nw) {
-        const double w = wl[l];
-        if ((__double_as_longlong(w) << 1) == 0) continue;
-        double *aj = colp(l);
-        for (int i = k + 1 + lane; i < ra; i += 32) aj[i] = fma(-w, bcast[i], aj[i]);
-      }
-    }
+    if (!GCOLS && tk != 0.0) update(l0 + warp, nl);
   }
   if (rank == ca) cluster_wait();  // (the last step's arrival)
   __syncthreads();
