@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "oz_order.h"
+
 namespace idmrg {
 
 // ---------------------------------------------------------------- buffers
@@ -332,7 +334,6 @@ cudaError_t launch_tc_gemm(const TcTile *tiles, int ntiles, const TcTask *tasks,
 // per element, exact integer accumulation per digit level).  K blocks are 16
 // elements; a tile sums at most OZ_MAX_K of K exactly, longer tasks have a tile
 // per K chunk (tile.chunk) and their chunks' results are added in FP64.
-constexpr int OZ_PLANES = 8;
 constexpr int OZ_KBLK = 16;
 constexpr int OZ_MAX_K = 768;
 constexpr int OZ_EXP_EMPTY = (int)0x80808080;  // byte-fill value: row without non-zeros

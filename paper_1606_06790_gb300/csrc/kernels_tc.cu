@@ -674,7 +674,7 @@ static_assert(OZ_KBLK == 16, "a K block is one kind::f16 MMA step");
 // is one M = 128 operand; B operands (G = 8) keep the planes of a K chunk one
 // after the other, so that consecutive planes read as one operand of 64 rows
 // each: A_p against B_q, B_q+1, ... is one MMA, and its output columns are the
-// consecutive levels p + q, p + q + 1, ...
+// consecutive levels p + q, p + q + 1, ... (see oz_order.h)
 __device__ __forceinline__ int64_t oz_off(int row, int k, int KB, int G, int p) {
   const int rows_per_tile = 8 * G;
   const int rt = row / rows_per_tile, rr = row - rt * rows_per_tile;
@@ -930,32 +930,35 @@ __global__ void __launch_bounds__(256, W_OZ_CTAS[PASS]) wstage_oz_kernel(const W
 
 constexpr int OZ_A_PLANE = TM * OZ_KBLK * 2;       // bytes of one A digit plane of a K block
 constexpr int OZ_B_PLANE = TC_TN * OZ_KBLK * 2;
-constexpr int OZ_STAGE = OZ_PLANES * (OZ_A_PLANE + OZ_B_PLANE);
-constexpr int OZ_STAGES = 4;
+constexpr int OZ_B_HALF = OZ_B_PLANE / 2;           // of it, one K chunk of 8
+constexpr int OZ_B_RUN = (OZ_ZERO + OZ_PLANES) * OZ_B_HALF;  // the stack of a K chunk: zero planes, then the digits
+constexpr int OZ_COPY = OZ_PLANES * (OZ_A_PLANE + OZ_B_PLANE);  // bytes copied per K block
+constexpr int OZ_STAGE = OZ_PLANES * OZ_A_PLANE + 2 * OZ_B_RUN;
+constexpr int OZ_STAGES = 3;
 constexpr int OZ_CH = OZ_MAX_K / OZ_KBLK;           // K blocks of one K chunk
 constexpr int OZ_TMEM_COLS = 512;                  // 8 levels x 64 columns
 constexpr int OZ_EPI_WARPS = 8;                    // two per TMEM lane quarter, 32 columns each
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_STG_LD = 17;                      // staging block of an epilogue warp: 32 rows x 16 columns
 constexpr int OZ_SMEM = OZ_STAGES * OZ_STAGE + OZ_EPI_WARPS * 32 * OZ_STG_LD * 8;
+static_assert(OZ_SMEM <= 227 * 1024, "shared memory of a CTA");
 
 // Persistent: one CTA per SM walks the tile list (128 x 64 outputs each, the
-// longest K first) with three roles, as tc_gemm_ps_kernel does.  What bounds
-// it is the tensor pipe: 36 digit products of 128 x 64 x 16 per K block, 1152
-// cycles.  They are issued as 12 MMAs of up to 256 columns (A_p against the
-// stacked planes of B, see oz_off), which read A from shared memory 12 times a
-// block instead of 36 and so stay below its bandwidth; 36 MMAs of 64 columns
-// were bound by it.  All 512 TMEM columns hold one tile, so the MMAs of the
-// next one wait until this one has been read: the epilogue warps first take
-// all eight levels into registers (integers, see below), release the
-// accumulators, and only then scale, round and store, beside the next tile's
-// MMAs.  Tasks longer than OZ_MAX_K have one tile per K chunk, so that few but
-// long outputs still fill the chip; these store into the task's partial
-// results, which oz_sum_kernel adds up in the order of K.
-// Measured (GB300; before: one CTA per tile of 32-element K blocks, the epilogue
-// in FP64 by the row): the two stages of the kagome cylinder's H_eff psi at
-// m = 1500 13.1 -> 4.2 ms (41 TFLOP/s FP64-accurate; 2.6 ms at the tensor pipe's
-// rate with all padding counted), of the J1-J2 cylinder at m = 500 0.81 -> 0.26 ms.
+// longest K first) with three roles, as tc_gemm_ps_kernel does.  A K block is 36
+// digit products of 128 x 64 x 16, issued as 15 MMAs of 128 or 192 columns in
+// fixed windows of levels (oz_order.h): 1376 cycles of the tensor pipe with the
+// zero planes, and 146 KB of operand reads beside 48 KB of copies, 1515 cycles
+// of shared memory; 36 MMAs of 64 columns read 216 KB.  All 512 TMEM columns
+// hold one tile, so the MMAs of the next one wait until this one has been read:
+// the epilogue warps first take all eight levels into registers (integers, see
+// below), release the accumulators, and only then scale, round and store, beside
+// the next tile's MMAs.  Tasks longer than OZ_MAX_K have one tile per K chunk, so
+// that few but long outputs still fill the chip; these store into the task's
+// partial results, which oz_sum_kernel adds up in the order of K.
+// Measured (GB300; before: one CTA per tile of 32-element K blocks, 36 MMAs of 64
+// columns per 16 of K, the epilogue in FP64 by the row): the two stages of the
+// kagome cylinder's H_eff psi at m = 1500 13.1 -> 4.4 ms (39 TFLOP/s
+// FP64-accurate), of the J1-J2 cylinder at m = 500 0.81 -> 0.28 ms.
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__restrict__ tiles, int ntiles,
                                                                 const TcTask *__restrict__ tasks,
                                                                 double *const *__restrict__ bufs,
@@ -980,6 +983,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__
     abort_flag = 0;
     tc::fence_mbar_init();
   }
+  // the zero planes of B: no copy touches them
+  for (int e = threadIdx.x; e < OZ_STAGES * 2 * OZ_ZERO * (OZ_B_HALF / 16); e += OZ_THREADS) {
+    const int run = e / (OZ_ZERO * (OZ_B_HALF / 16)), i = e - run * (OZ_ZERO * (OZ_B_HALF / 16));
+    *reinterpret_cast<uint4 *>(osm + (run >> 1) * OZ_STAGE + OZ_PLANES * OZ_A_PLANE + (run & 1) * OZ_B_RUN + 16 * i) =
+        make_uint4(0u, 0u, 0u, 0u);
+  }
+  tc::fence_async_smem();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -1007,10 +1017,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__
             break;
           }
           uint8_t *st = osm + s * OZ_STAGE;
-          tc::mbar_arrive_expect_tx(&full[s], (uint32_t)OZ_STAGE);
+          tc::mbar_arrive_expect_tx(&full[s], (uint32_t)OZ_COPY);
           tc::bulk_g2s(st, A + (int64_t)kb * OZ_PLANES * OZ_A_PLANE, OZ_PLANES * OZ_A_PLANE, &full[s]);
-          tc::bulk_g2s(st + OZ_PLANES * OZ_A_PLANE, B + (int64_t)kb * OZ_PLANES * OZ_B_PLANE, OZ_PLANES * OZ_B_PLANE,
-                       &full[s]);
+          for (int kc = 0; kc < 2; ++kc)
+            tc::bulk_g2s(st + OZ_PLANES * OZ_A_PLANE + kc * OZ_B_RUN + OZ_ZERO * OZ_B_HALF,
+                         B + ((int64_t)kb * 2 + kc) * OZ_PLANES * OZ_B_HALF, OZ_PLANES * OZ_B_HALF, &full[s]);
         }
       }
       if (!ok) {
@@ -1023,8 +1034,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ---- MMA issuer
-      constexpr uint32_t lboA = (TM / 8) * 128, lboB = OZ_PLANES * (TC_TN / 8) * 128, sbo = 128;
-      constexpr uint32_t bplane = (TC_TN / 8) * 128;  // bytes from one stacked B plane to the next
+      constexpr uint32_t lboA = (TM / 8) * 128, lboB = OZ_B_RUN, sbo = 128;
       long long it = 0;
       int v = 0;  // tiles so far
       bool ok = true;
@@ -1047,17 +1057,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__
           tc::fence_after_sync();
           const uint32_t sa = tc::smem_u32(osm + s * OZ_STAGE);
           const uint32_t sb = sa + OZ_PLANES * OZ_A_PLANE;
-#pragma unroll
-          for (int p = 0; p < OZ_PLANES; ++p) {
-            const uint64_t ad = tc::smem_desc(sa + p * OZ_A_PLANE, lboA, sbo);
-#pragma unroll
-            for (int q = 0; q < OZ_PLANES - p; q += 4) {  // planes q .. q + 3 (fewer at the end)
-              const int nq = OZ_PLANES - p - q < 4 ? OZ_PLANES - p - q : 4;
-              const uint64_t bd = tc::smem_desc(sb + q * bplane, lboB, sbo);
-              tc::mma_f16(tmem + (uint32_t)(TC_TN * (p + q)), ad, bd, tc::instr_desc(TM, nq * TC_TN, 1u),
-                          (kb > kc || p > 0) ? 1u : 0u);
-            }
-          }
+          oz_for_each_mma([&](int p, int q0, int level, int n) {
+            tc::mma_f16(tmem + (uint32_t)(TC_TN * level), tc::smem_desc(sa + p * OZ_A_PLANE, lboA, sbo),
+                        tc::smem_desc(sb + (OZ_ZERO + q0) * OZ_B_HALF, lboB, sbo), tc::instr_desc(TM, n * TC_TN, 1u),
+                        (kb > kc || p > 0) ? 1u : 0u);
+          });
           tc::mma_commit(&empty[s]);
         }
         if (!ok) break;
