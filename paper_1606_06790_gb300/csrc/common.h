@@ -123,11 +123,11 @@ struct SvdJob {
   int64_t x_off;    // rows_a x cols_a scratch for the back-transformation
   int64_t tau_off;  // cols_a Householder coefficients
   int64_t w_off;    // cols_a x cols_a scratch of the FP32-preconditioned Jacobi
-  int64_t t_off;    // cols_a x cols_a scratch of the refinement (refined jobs)
+  int64_t t_off;    // three cols_a x cols_a areas of the refinement (refined jobs): scratch, V and X before it
   int perm_off;     // cols_a column permutation of the pivoted QR (int work),
                     // then the numerical rank found by the QR, the sweeps of
                     // the final and of the FP32 Jacobi, and whether the final
-                    // Jacobi has anything to do (1: yes)
+                    // Jacobi has anything to do (0: no)
   int sv_off;       // singular values of this job
 };
 
@@ -240,16 +240,18 @@ cudaError_t launch_svd_jacobi(const SvdJob *jobs, const int *order, int njobs, c
 cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs, const int *g, const int *cols,
                                 int cols0, double *work, const int *iwork, cudaStream_t st,
                                 const cudaStream_t *side, const cudaEvent_t *ev);
-// per job over cols_a x cols_a elements: 0: V = I (and the final Jacobi is to
-// run); 1: V = 1.5 V - 0.5 W (Newton-Schulz step, W at w_off); 2: B = X (X at
-// w_off)
+// per job over cols_a x cols_a elements: 0: V = I; 1: V = 1.5 V - 0.5 W
+// (Newton-Schulz step, W at w_off); 2: B = X (X at w_off), and the final Jacobi
+// is to run on sectors that are not refined
 cudaError_t launch_svd_elementwise(const SvdJob *jobs, int njobs, int max_cols, int mode, double *work, int *iwork,
                                    cudaStream_t st);
 // The elementwise parts of the refinement between the Newton-Schulz steps and
-// the final Jacobi (see kernels_svd.cu), on the jobs order[0 .. njobs)
-enum SvdRefine { REF_SCALE, REF_BUILD, REF_BUILD_R, REF_FINISH, REF_PUT_V, REF_PUT_X, REF_CHECK };
-cudaError_t launch_svd_refine(SvdRefine part, const SvdJob *jobs, const int *order, int njobs, int max_cols,
-                              double *work, int *iwork, double *sv, cudaStream_t st);
+// the final Jacobi (see kernels_svd.cu), on the jobs order[0 .. njobs); round:
+// 0 .. SVD_REFINE_ROUNDS - 1
+enum SvdRefine { REF_SCALE, REF_BUILD, REF_FINISH, REF_ORTHO, REF_PUT_V, REF_PUT_X, REF_CHECK };
+constexpr int SVD_REFINE_ROUNDS = 2;
+cudaError_t launch_svd_refine(SvdRefine part, int round, const SvdJob *jobs, const int *order, int njobs,
+                              int max_cols, double *work, int *iwork, double *sv, cudaStream_t st);
 constexpr int SVD_REFINE_MIN = 64;  // columns from which sectors are refined
 struct SelectOut {
   int *kept_per_job;   // [njobs]

@@ -364,7 +364,7 @@ struct idmrg_ctx {
   int tiw = 0, tsv = 0, tentries_max = 1, tmaxcols = 0;
   // FP32-preconditioned Jacobi: G = V^T V, W = V G (Newton-Schulz), X = B V
   GemmList svdG, svdW, svdX;
-  // refinement (sectors of SVD_REFINE_MIN columns on): G = Xs^T Xs, V^T V, As^2, V T, Xs Ts
+  // refinement (sectors of SVD_REFINE_MIN columns on): G = Xs^T Xs, V^T V, Ks^2, V T, Xs Ts
   GemmList svdH, svdR, svdK, svdV, svdT;
   DevBuf dshk, dshs, dsrk, dsrs, dskk, dsks, dsvk, dsvs, dstk, dsts;
   DevBuf dsgk, dsgs, dswk, dsws, dsxk, dsxs;
@@ -2194,7 +2194,7 @@ idmrg_status trunc_plan(idmrg_ctx *c, int p) {
       J.w_off = work;
       work += (int64_t)J.cols_a * J.cols_a;
       J.t_off = work;
-      if (J.cols_a >= SVD_REFINE_MIN) work += (int64_t)J.cols_a * J.cols_a;
+      if (J.cols_a >= SVD_REFINE_MIN) work += 3 * (int64_t)J.cols_a * J.cols_a;
       J.perm_off = iw;
       iw += J.cols_a + 4;  // permutation, rank, FP64 and FP32 Jacobi sweeps, final Jacobi to run
       J.sv_off = sv;
@@ -2402,16 +2402,16 @@ void svd_stats_reset(idmrg_ctx *c) {
   c->svd_jobs32 = 0;
 }
 
-// Two correction steps for the sectors of SVD_REFINE_MIN columns on, and the
-// check that decides which of them the final Jacobi still has to sweep (see
-// the refinement in kernels_svd.cu).
+// Two rounds of correction and Newton-Schulz step for the sectors of
+// SVD_REFINE_MIN columns on, and the check that decides which of them the final
+// Jacobi still has to sweep (see the refinement in kernels_svd.cu).
 idmrg_status svd_refine(idmrg_ctx *c) {
   if (c->svdH.tasks.empty()) return IDMRG_OK;
   int nref = 0;  // torder lists the largest sectors first
   while (nref < (int)c->torder.size() && c->jobs[c->torder[nref]].cols_a >= SVD_REFINE_MIN) ++nref;
-  auto part = [&](SvdRefine what) {
+  auto part = [&](SvdRefine what, int round) {
     c->launches += 1;
-    return launch_svd_refine(what, (const SvdJob *)c->sjobs.p, (const int *)c->sorder.p, nref, c->tmaxcols,
+    return launch_svd_refine(what, round, (const SvdJob *)c->sjobs.p, (const int *)c->sorder.p, nref, c->tmaxcols,
                              c->dp(c->swork), (int *)c->siw.p, c->dp(c->ssv), c->st);
   };
 #define REF_GEMM(x, k, s)                                    \
@@ -2419,24 +2419,27 @@ idmrg_status svd_refine(idmrg_ctx *c) {
     const idmrg_status s_ = gemm_run(c, c->x, c->k, c->s, nullptr); \
     if (s_ != IDMRG_OK) return s_;                           \
   } while (0)
-  CK(part(REF_SCALE));
-  for (int step = 0; step < 2; ++step) {
+#define REF_APPLY(round)              \
+  do {                                \
+    REF_GEMM(gd_svdV, dsvk, dsvs);    \
+    CK(part(REF_PUT_V, round));       \
+    REF_GEMM(gd_svdT, dstk, dsts);    \
+    CK(part(REF_PUT_X, round));       \
+  } while (0)
+  CK(part(REF_SCALE, 0));
+  for (int round = 0; round < SVD_REFINE_ROUNDS; ++round) {
     REF_GEMM(gd_svdH, dshk, dshs);
-    if (step == 0) {
-      CK(part(REF_BUILD));
-    } else {
-      REF_GEMM(gd_svdR, dsrk, dsrs);
-      CK(part(REF_BUILD_R));
-    }
+    CK(part(REF_BUILD, round));
     REF_GEMM(gd_svdK, dskk, dsks);
-    CK(part(REF_FINISH));
-    REF_GEMM(gd_svdV, dsvk, dsvs);
-    CK(part(REF_PUT_V));
-    REF_GEMM(gd_svdT, dstk, dsts);
-    CK(part(REF_PUT_X));
+    CK(part(REF_FINISH, round));
+    REF_APPLY(round);
+    REF_GEMM(gd_svdR, dsrk, dsrs);
+    CK(part(REF_ORTHO, round));
+    REF_APPLY(round);
   }
   REF_GEMM(gd_svdH, dshk, dshs);
-  CK(part(REF_CHECK));
+  CK(part(REF_CHECK, 0));
+#undef REF_APPLY
 #undef REF_GEMM
   return IDMRG_OK;
 }

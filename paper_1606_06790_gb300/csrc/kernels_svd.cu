@@ -14,8 +14,9 @@
 //            Then A = (Q Jm) S (P U~)^T.  An FP32 stage runs it to overlaps of
 //            1e-6; Newton-Schulz makes its rotations orthogonal in 64 bits.
 //  refine  : two corrections of those rotations from the Gram matrices of the
-//            rotated columns, by matrix products, and a check; the FP64 sweeps
-//            run on the sectors that the check finds unfinished.
+//            rotated columns, by matrix products, each followed by a
+//            Newton-Schulz step, and a check; the FP64 sweeps run on the sectors
+//            that the check finds unfinished.
 //  select  : per superblock, sorts all singular values in descending order
 //            (ties by |Q|, Q, index), drops values at or below zero_rel*max,
 //            cuts at D <= m without splitting values closer than tie_rel, and
@@ -2259,7 +2260,7 @@ __global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *
                                        int *__restrict__ iwork, int mode) {
   const SvdJob J = jobs[blockIdx.y];
   const int ca = J.cols_a;
-  if (mode == 0 && blockIdx.x == 0 && threadIdx.x == 0) iwork[J.perm_off + ca + 3] = 1;
+  if (mode == 2 && blockIdx.x == 0 && threadIdx.x == 0) iwork[J.perm_off + ca + 3] = ca < SVD_REFINE_MIN;
   const int64_t tot = (int64_t)ca * ca;
   double *V = work + J.j_off, *W = work + J.w_off, *B = work + J.b_off;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
@@ -2278,50 +2279,65 @@ __global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *
 // X shows), and the final Jacobi would need two to three sweeps: one that
 // rotates by these overlaps, and one or two that find next to nothing left.
 // A correction takes all overlaps to second order at once, by matrix products
-// (Ogita and Aishima, "Iterative refinement for symmetric eigenvalue
+// (after Ogita and Aishima, "Iterative refinement for symmetric eigenvalue
 // decomposition", Japan J. Indust. Appl. Math. 35, 2018, for eigenvectors): with
-// D the column norms, X = Xs D, G = Xs^T Xs, b_i = D_i^2 G_ii, R = V^T V - 1 and
-//   A = K - R / 2,  K_ij = (G_ij D_i D_j - R_ij (b_i + b_j) / 2) / (b_j - b_i),
-// X' = X (1 + A + A^2 / 2) and V' = V (1 + A + A^2 / 2) have overlaps of order
-// K G, and with R = 0 the factor is orthogonal to K^4 / 4.  The first step (R is
-// rounding) takes pairs of |K| <= 2e-2: few sectors have nearer
-// singular values than that.  It leaves overlaps of 1e-8 at most and V
-// orthogonal to 4e-8; the second one, with R and |K| <= 1e-4, takes both to
-// rounding.  What they reach is then checked (REF_CHECK): a sector in which some
-// pair is still above the threshold of the FP64 Jacobi goes through the final
-// Jacobi's sweeps as before, the others only have their norms taken.
+// D the column norms, X = Xs D, G = Xs^T Xs, b_i = D_i^2 G_ii and
+//   K_ij = G_ij D_i D_j / (b_j - b_i), antisymmetric,
+// X' = X (1 + K + K^2 / 2) and V' = V (1 + K + K^2 / 2) have overlaps of order
+// K G.  The factor is orthogonal to K^4 / 4 (of the whole matrix K: in a group of
+// close values that is far more than of an entry), so each correction is
+// followed by a Newton-Schulz step for V, V' = V (1 - R / 2) with R = V^T V - 1,
+// and X' = X (1 - R / 2), which keeps X = B V.  Two such rounds: the first takes
+// pairs of |K| <= 2e-2 (few sectors have nearer singular values than that) and
+// leaves overlaps of 1e-8 at most and, before its Newton-Schulz step, V
+// orthogonal to 4e-8 in pairs, to 1e-4 in dense spectra; the second, of
+// |K| <= 1e-4, takes both to rounding.  K and R have to be applied one after the
+// other: a single factor 1 + A + A^2 / 2 with A = K - R / 2 leaves V^T V - 1 and
+// X - B V of order K R, measured at 1e-11 with quartets of values 1e-4 apart and
+// 5e-8 with 462 values within 2 %.
+// What the rounds reach is then checked (REF_CHECK): a sector in which some pair
+// is still above the threshold of the FP64 Jacobi goes through the final Jacobi's
+// sweeps, the others only have their norms taken.  The sweeps rotate V and so
+// keep what V^T V - 1 is: a sector whose last R had an entry above
+// sqrt(eps / n), beyond which R^2, which a Newton-Schulz step leaves, is not
+// rounding, gets back the V and X that it came with, and the sweeps do it all.
 // The spectra are graded over up to 13 decades, and overlaps must shrink
 // relative to their own columns: X is corrected in the scaled form
-// Xs' = Xs (1 + As + As^2 / 2), As = D A D^-1, whose entries are of the size of
+// Xs' = Xs (1 + Ks + Ks^2 / 2), Ks = D K D^-1, whose entries are of the size of
 // the overlaps (Ks_ij ~ -G_ij for D_i >> D_j, vanishing for D_i << D_j), so that
 // the products' rounding stays relative to every column; R, whose rounding would
-// not, is used where D_i and D_j are within a factor of 4, or of 64 if it stands
-// out of the rounding.
+// not, is used (for V as for X) where it stands out of the rounding, above 2e-15,
+// and on the diagonal.
 // All matrices lie transposed (row j belongs to column j of X): G and the
-// results in x_off, As^T and then (1 + As + As^2/2)^T in w_off, V^T V, (As^2)^T
-// and then (1 + A + A^2/2)^T in t_off, D in the job's singular values.
-// Measured (GB300, ms of a step; before -> now, the ten products included):
-// final Jacobi 39.8 -> 6.1 and Newton-Schulz to check 1.2 -> 4.1 for the J1-J2
-// cylinder at m = 1024, 55.8 -> 6.0 and 1.7 -> 5.6 for kagome at m = 1000, 13.2 ->
-// 0.8 and 0.5 -> 1.6 for J1-J2 at m = 500; sectors below SVD_REFINE_MIN columns
-// (2.7 -> 0.9 against 0.3 -> 1.0 for the chain at m = 256, half of whose sectors
+// results in x_off; Ks^T and then the factor of X in w_off; (Ks^2)^T or V^T V and
+// then the factor of V in t_off, followed by V and X as they came; D in the job's
+// singular values.
+// Measured (GB300, ms of a step; without -> with, the fifteen products included):
+// final Jacobi 39.8 -> 6.0 and Newton-Schulz to check 1.2 -> 5.3 for the J1-J2
+// cylinder at m = 1024, 55.8 -> 6.0 and 1.7 -> 7.2 for kagome at m = 1000, 13.2 ->
+// 0.9 and 0.5 -> 1.9 for J1-J2 at m = 500; sectors below SVD_REFINE_MIN columns
+// (2.7 -> 0.6 against 0.3 -> 1.2 for the chain at m = 256, half of whose sectors
 // are refined) gain less than the launches cost.
-constexpr float REF_KMAX = 2e-2f, REF_KMAX_R = 1e-4f;
+constexpr float REF_KMAX[SVD_REFINE_ROUNDS] = {2e-2f, 1e-4f};
 
 // column norms of X and Xs = X / D (rows of the transposed X at b_off, one
-// warp each; columns past the rank become zero)
+// warp each; columns past the rank become zero); X and V are kept as they came
 __global__ void __launch_bounds__(256) refine_scale_kernel(const SvdJob *__restrict__ jobs,
                                                            const int *__restrict__ order, double *__restrict__ work,
-                                                           int *__restrict__ iwork, double *__restrict__ sv) {
+                                                           const int *__restrict__ iwork, double *__restrict__ sv) {
   const SvdJob J = jobs[order[blockIdx.y]];
   const int ca = J.cols_a, n = iwork[J.perm_off + ca], lane = threadIdx.x & 31;
-  if (blockIdx.x == 0 && threadIdx.x == 0) iwork[J.perm_off + ca + 3] = 0;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (j >= ca) return;
-  double *x = work + J.b_off + (int64_t)j * ca;
+  const int64_t row = (int64_t)j * ca, nn = (int64_t)ca * ca;
+  double *x = work + J.b_off + row, *v0 = work + J.t_off + nn + row, *x0 = v0 + nn;
+  const double *v = work + J.j_off + row;
   double s = 0.0;
-  if (j < n)
-    for (int i = lane; i < ca; i += 32) s = fma(x[i], x[i], s);
+  for (int i = lane; i < ca; i += 32) {
+    x0[i] = x[i];
+    v0[i] = v[i];
+    if (j < n) s = fma(x[i], x[i], s);
+  }
   s = sqrt(wsum(s));
   const double inv = s > 0.0 ? 1.0 / s : 0.0;
   for (int i = lane; i < ca; i += 32) x[i] = s > 0.0 ? x[i] * inv : 0.0;
@@ -2331,14 +2347,14 @@ __global__ void __launch_bounds__(256) refine_scale_kernel(const SvdJob *__restr
 // The pairs (i, j), i <= j, of one 32 x 32 tile (rows j of the transposed
 // matrices, tile (tj, ti) with ti <= tj) and their mirror images: reads and
 // writes of both tiles coalesced, the mirrored one through shared memory.
-//   REF_BUILD  : G -> As^T (w), R = 0
-//   REF_BUILD_R: G, V^T V (t) -> As^T (w)
-//   REF_FINISH : As^T (w), (As^2)^T (t) -> the two correction factors
+//   REF_BUILD  : G -> Ks^T (w), entries with |K| <= kmax
+//   REF_FINISH : Ks^T (w), (Ks^2)^T (t) -> the factors of X (w) and V (t)
 //   REF_CHECK  : G -> is any overlap above the FP64 Jacobi's threshold
 template <int PART>
 __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restrict__ jobs,
                                                           const int *__restrict__ order, double *__restrict__ work,
-                                                          int *__restrict__ iwork, const double *__restrict__ sv) {
+                                                          int *__restrict__ iwork, const double *__restrict__ sv,
+                                                          float kmax) {
   __shared__ double m1[32][33], m2[32][33];
   const SvdJob J = jobs[order[blockIdx.y]];
   const int ca = J.cols_a, n = iwork[J.perm_off + ca];
@@ -2369,12 +2385,12 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
       const double Di = D[i], Dj = D[j];
       const double inv_i = Di > 0.0 ? 1.0 / Di : 0.0, inv_j = Dj > 0.0 ? 1.0 / Dj : 0.0;
       if (PART == REF_FINISH) {
-        // p, q: As at (i, j), (j, i); s, u: its square
+        // p, q: Ks at (i, j), (j, i); s, u: its square
         const double p = w[at(j, i)], q = m1[c][r], s = t[at(j, i)], u = m2[c][r];
         if (i == j) {
-          w[at(j, j)] = t[at(j, j)] = 1.0 + fma(0.5, s, p);
+          w[at(j, j)] = t[at(j, j)] = fma(0.5, s, 1.0);
         } else {
-          // A^2 from the triangle in which As^2 carries all digits
+          // K^2, symmetric, from the triangle in which Ks^2 carries all digits
           const double h = 0.5 * (Di >= Dj ? s * (Dj * inv_i) : u * (Di * inv_j));
           w[at(j, i)] = fma(0.5, s, p);
           a1 = fma(0.5, u, q);
@@ -2389,24 +2405,16 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
           bad |= !(fabsf((float)g) <= 0x1p-52f * sqrtf((float)ca)) &&
                  fabs(g) * Di * Dj > 4.0 * DBL_EPSILON * DBL_EPSILON * D[0] * D[0];
       } else {
-        double k = 0.0, h = 0.0;  // K_ij, R_ij / 2
-        if (j < n && Di > 0.0 && Dj > 0.0) {
-          if (PART == REF_BUILD_R) {
-            h = 0.5 * (i == j ? t[at(j, j)] - 1.0 : t[at(j, i)]);
-            const double hi = fmax(Di, Dj), lo = fmin(Di, Dj);
-            if (!(hi < 4.0 * lo) && !(hi < 64.0 * lo && fabs(h) > 0.5e-15)) h = 0.0;
-          }
-          if (i < j) {
-            const double bi = Di * Di * G[at(i, i)], bj = Dj * Dj * G[at(j, j)];
-            const double num = G[at(j, i)] * (Di * Dj) - h * (bi + bj);
-            // FP32 is enough for the angle (a relative error of K leaves that
-            // part of the overlap); both triangles use the same rounded value
-            const float kf = __fdividef((float)num, (float)(bj - bi));
-            if (fabsf(kf) <= (PART == REF_BUILD ? REF_KMAX : REF_KMAX_R)) k = (double)kf;
-          }
+        double k = 0.0;  // K_ij
+        if (i < j && j < n && Di > 0.0 && Dj > 0.0) {
+          const double bi = Di * Di * G[at(i, i)], bj = Dj * Dj * G[at(j, j)];
+          // FP32 is enough for the angle (a relative error of K leaves that
+          // part of the overlap); both triangles use the same rounded value
+          const float kf = __fdividef((float)(G[at(j, i)] * (Di * Dj)), (float)(bj - bi));
+          if (fabsf(kf) <= kmax) k = (double)kf;
         }
-        w[at(j, i)] = (k - h) * (Di * inv_j);
-        a1 = (-k - h) * (Dj * inv_i);
+        w[at(j, i)] = k * (Di * inv_j);
+        a1 = -k * (Dj * inv_i);
       }
     }
     if (PART != REF_CHECK) {  // (an element of the mirrored tile is read above by this thread only)
@@ -2415,7 +2423,7 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
     }
   }
   if (PART == REF_CHECK) {
-    if (bad) iwork[J.perm_off + ca + 3] = 1;
+    if (bad && iwork[J.perm_off + ca + 3] == 0) iwork[J.perm_off + ca + 3] = 1;
     return;
   }
   __syncthreads();
@@ -2428,17 +2436,51 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
   }
 }
 
-// mode REF_PUT_V: V = X (x_off); REF_PUT_X: Xs = X; REF_CHECK: X = Xs D
+// The Newton-Schulz step's factors from V^T V (t): of X, scaled, to w, of V to
+// t; a warp per row.  last: an entry of R too large for this step to leave
+// rounding marks the sector (2: V and X as they came).
+__global__ void __launch_bounds__(256) refine_ortho_kernel(const SvdJob *__restrict__ jobs,
+                                                           const int *__restrict__ order, double *__restrict__ work,
+                                                           int *__restrict__ iwork, const double *__restrict__ sv,
+                                                           bool last) {
+  const SvdJob J = jobs[order[blockIdx.y]];
+  const int ca = J.cols_a, n = iwork[J.perm_off + ca], lane = threadIdx.x & 31;
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= ca) return;
+  double *w = work + J.w_off + (int64_t)j * ca, *t = work + J.t_off + (int64_t)j * ca;
+  const double *D = sv + J.sv_off;
+  const double Dj = D[j], inv_j = Dj > 0.0 ? 1.0 / Dj : 0.0;
+  const float lim = sqrtf((float)DBL_EPSILON / (float)max(n, 1));
+  bool bad = false;
+  for (int i = lane; i < ca; i += 32) {
+    const double one = i == j ? 1.0 : 0.0, Di = D[i];
+    double h = 0.5 * (t[i] - one);
+    const float hf = fabsf((float)h);
+    if (i < n && j < n) bad |= !(2.0f * hf <= lim);
+    if (!(Di > 0.0) || !(Dj > 0.0) || (i != j && hf <= 1e-15f)) h = 0.0;
+    w[i] = fma(-h, Di * inv_j, one);
+    t[i] = one - h;
+  }
+  if (last && bad) iwork[J.perm_off + ca + 3] = 2;
+}
+
+// mode REF_PUT_V: V = X (x_off); REF_PUT_X: Xs = X; REF_CHECK: X = Xs D, or V
+// and X as they came
 __global__ void __launch_bounds__(256) refine_put_kernel(const SvdJob *__restrict__ jobs,
                                                          const int *__restrict__ order, double *__restrict__ work,
+                                                         const int *__restrict__ iwork,
                                                          const double *__restrict__ sv, int mode) {
   const SvdJob J = jobs[order[blockIdx.y]];
   const int ca = J.cols_a;
   const int64_t tot = (int64_t)ca * ca;
-  const double *from = work + (mode == REF_CHECK ? J.b_off : J.x_off);
-  double *to = work + (mode == REF_PUT_V ? J.j_off : J.b_off);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x)
-    to[e] = mode == REF_CHECK ? from[e] * sv[J.sv_off + e / ca] : from[e];
+  const bool back = mode == REF_CHECK && iwork[J.perm_off + ca + 3] == 2;
+  const double *v0 = work + J.t_off + tot;
+  const double *from = back ? v0 + tot : work + (mode == REF_CHECK ? J.b_off : J.x_off);
+  double *to = work + (mode == REF_PUT_V ? J.j_off : J.b_off), *V = work + J.j_off;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    to[e] = mode == REF_CHECK && !back ? from[e] * sv[J.sv_off + e / ca] : from[e];
+    if (back) V[e] = v0[e];
+  }
 }
 
 // ---------------------------------------------------------------- select
@@ -2968,33 +3010,27 @@ cudaError_t launch_svd_elementwise(const SvdJob *jobs, int njobs, int max_cols, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_svd_refine(SvdRefine part, const SvdJob *jobs, const int *order, int njobs, int max_cols,
-                              double *work, int *iwork, double *sv, cudaStream_t st) {
+cudaError_t launch_svd_refine(SvdRefine part, int round, const SvdJob *jobs, const int *order, int njobs,
+                              int max_cols, double *work, int *iwork, double *sv, cudaStream_t st) {
   if (njobs <= 0 || max_cols <= 0) return cudaGetLastError();
   const int nt = (max_cols + 31) / 32;
   const dim3 tiles((unsigned)(nt * (nt + 1) / 2), (unsigned)njobs);
   const dim3 elems((unsigned)std::min<int64_t>(((int64_t)max_cols * max_cols + 255) / 256, 64), (unsigned)njobs);
+  const dim3 rows((unsigned)((max_cols + 7) / 8), (unsigned)njobs);
   switch (part) {
-    case REF_SCALE:
-      refine_scale_kernel<<<dim3((unsigned)((max_cols + 7) / 8), (unsigned)njobs), 256, 0, st>>>(jobs, order, work,
-                                                                                                 iwork, sv);
-      break;
+    case REF_SCALE: refine_scale_kernel<<<rows, 256, 0, st>>>(jobs, order, work, iwork, sv); break;
     case REF_BUILD:
-      refine_pair_kernel<REF_BUILD><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+      refine_pair_kernel<REF_BUILD><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv, REF_KMAX[round]);
       break;
-    case REF_BUILD_R:
-      refine_pair_kernel<REF_BUILD_R><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
-      break;
-    case REF_FINISH:
-      refine_pair_kernel<REF_FINISH><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
+    case REF_FINISH: refine_pair_kernel<REF_FINISH><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv, 0.0f); break;
+    case REF_ORTHO:
+      refine_ortho_kernel<<<rows, 256, 0, st>>>(jobs, order, work, iwork, sv, round + 1 == SVD_REFINE_ROUNDS);
       break;
     case REF_PUT_V:
-    case REF_PUT_X:
-      refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, sv, part);
-      break;
+    case REF_PUT_X: refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, iwork, sv, part); break;
     case REF_CHECK:
-      refine_pair_kernel<REF_CHECK><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv);
-      refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, sv, part);
+      refine_pair_kernel<REF_CHECK><<<tiles, 256, 0, st>>>(jobs, order, work, iwork, sv, 0.0f);
+      refine_put_kernel<<<elems, 256, 0, st>>>(jobs, order, work, iwork, sv, part);
       break;
   }
   return cudaGetLastError();
