@@ -2321,10 +2321,11 @@ __global__ void svd_elementwise_kernel(const SvdJob *__restrict__ jobs, double *
 constexpr float REF_KMAX[SVD_REFINE_ROUNDS] = {2e-2f, 1e-4f};
 
 // column norms of X and Xs = X / D (rows of the transposed X at b_off, one
-// warp each; columns past the rank become zero); X and V are kept as they came
+// warp each; columns past the rank become zero); X and V are kept as they came,
+// and the sector gets them back if a column is not finite
 __global__ void __launch_bounds__(256) refine_scale_kernel(const SvdJob *__restrict__ jobs,
                                                            const int *__restrict__ order, double *__restrict__ work,
-                                                           const int *__restrict__ iwork, double *__restrict__ sv) {
+                                                           int *__restrict__ iwork, double *__restrict__ sv) {
   const SvdJob J = jobs[order[blockIdx.y]];
   const int ca = J.cols_a, n = iwork[J.perm_off + ca], lane = threadIdx.x & 31;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -2342,6 +2343,7 @@ __global__ void __launch_bounds__(256) refine_scale_kernel(const SvdJob *__restr
   const double inv = s > 0.0 ? 1.0 / s : 0.0;
   for (int i = lane; i < ca; i += 32) x[i] = s > 0.0 ? x[i] * inv : 0.0;
   if (lane == 0) sv[J.sv_off + j] = s;
+  if (lane == 0 && !isfinite(s)) iwork[J.perm_off + ca + 3] = 2;
 }
 
 // The pairs (i, j), i <= j, of one 32 x 32 tile (rows j of the transposed
@@ -2399,11 +2401,11 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
         }
       } else if (PART == REF_CHECK) {
         // bj_rotation's own test: relative overlap above sqrt(rows) 2^-52 (and
-        // g above its floor 4 eps^2 ||X||^2)
+        // g above its floor 4 eps^2 ||X||^2); not a number is above both
         const double g = G[at(j, i)];
         if (j < n && i < j)
           bad |= !(fabsf((float)g) <= 0x1p-52f * sqrtf((float)ca)) &&
-                 fabs(g) * Di * Dj > 4.0 * DBL_EPSILON * DBL_EPSILON * D[0] * D[0];
+                 !(fabs(g) * Di * Dj <= 4.0 * DBL_EPSILON * DBL_EPSILON * D[0] * D[0]);
       } else {
         double k = 0.0;  // K_ij
         if (i < j && j < n && Di > 0.0 && Dj > 0.0) {

@@ -1,0 +1,81 @@
+"""Not-a-numbers in the SVD refinement: the library refuses a non-finite
+wavefunction before the SVD, so the refinement's kernels are called on their own
+here.  A sector with a non-finite column, or with an overlap that is not a number,
+counts as unfinished (flag behind the job's permutation not 0: the final Jacobi
+sweeps it), and a non-finite column is handed on as it came; a sector of
+orthonormal columns is finished."""
+import ctypes as C
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_1606_06790_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+CSRC = os.path.join(os.path.dirname(pkg.__file__), "csrc")
+HEADER = open(os.path.join(CSRC, "common.h")).read()
+
+
+def _struct(name):
+    body = re.search(r"struct %s \{(.*?)\n\};" % name, HEADER, re.S).group(1)
+    fields = []
+    for kind, names in re.findall(r"^\s*(int64_t|int|float|double) ([^;]+);", body, re.M):
+        t = {"int64_t": C.c_int64, "int": C.c_int, "float": C.c_float, "double": C.c_double}[kind]
+        for n in names.split(","):
+            m = re.match(r"\s*(\w+)(?:\[(\d+)\])?\s*$", n)
+            fields.append((m.group(1), t * int(m.group(2)) if m.group(2) else t))
+    return type(name, (C.Structure,), {"_fields_": fields})
+
+
+def _launcher(name):
+    lib = pkg.load_library()
+    symbols = subprocess.run(["nm", "-D", lib._name], capture_output=True, text=True, check=True).stdout.split()
+    return getattr(lib, next(s for s in symbols if re.match(r"_ZN5idmrg%d%s" % (len(name), name), s)))
+
+
+PARTS = re.search(r"enum SvdRefine \{(.*?)\}", HEADER, re.S).group(1).replace(" ", "").split(",")
+CA = 80  # two rows of tiles and a ragged third
+
+
+@pytest.mark.parametrize("what", ["finite", "column", "overlap"])
+def test_not_a_number_is_unfinished(what):
+    import torch
+    nn = CA * CA
+    Job, refine = _struct("SvdJob"), _launcher("launch_svd_refine")
+    job = Job(r=CA, c=CA, rows_a=CA, cols_a=CA, a_off=0, j_off=nn, b_off=2 * nn, x_off=3 * nn, tau_off=4 * nn,
+              w_off=4 * nn + CA, t_off=5 * nn + CA, perm_off=0, sv_off=0)
+    work = torch.zeros(8 * nn + CA, device="cuda", dtype=torch.float64)
+    iwork = torch.zeros(CA + 4, device="cuda", dtype=torch.int32)
+    iwork[CA] = CA  # rank
+    sv = torch.zeros(CA, device="cuda", dtype=torch.float64)
+    jobs = torch.tensor(np.frombuffer(bytes(job), dtype=np.uint8).copy(), device="cuda")
+    order = torch.zeros(1, device="cuda", dtype=torch.int32)
+    X = torch.tensor(np.linalg.qr(np.random.default_rng(3).standard_normal((CA, CA)))[0], device="cuda")
+    X = X * torch.linspace(1.0, 0.1, CA, device="cuda", dtype=torch.float64)[:, None]  # row j: column j of X
+    if what == "column":
+        X[70, 5] = float("nan")
+    area = lambda off: work[off:off + nn].view(CA, CA)
+    area(job.b_off).copy_(X)
+    area(job.j_off).copy_(torch.eye(CA))
+
+    def part(name, stage=0):
+        s = refine(PARTS.index(name), stage, C.c_void_p(jobs.data_ptr()), C.c_void_p(order.data_ptr()), 1, CA,
+                   C.c_void_p(work.data_ptr()), C.c_void_p(iwork.data_ptr()), C.c_void_p(sv.data_ptr()),
+                   C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert s == 0
+        torch.cuda.synchronize()
+
+    part("REF_SCALE")
+    area(job.x_off).copy_(area(job.b_off) @ area(job.b_off).T)
+    if what == "overlap":
+        area(job.x_off)[70, 3] = float("nan")
+    part("REF_CHECK")
+    assert (iwork[CA + 3].item() != 0) == (what != "finite")
+    if what != "overlap":
+        got = area(job.b_off)
+        assert torch.equal(torch.isnan(got), torch.isnan(X))
+        assert (got - X).abs().nan_to_num().max().item() < 1e-15
