@@ -2400,11 +2400,12 @@ __global__ void __launch_bounds__(256) refine_pair_kernel(const SvdJob *__restri
           a2 = fma(q, Di * inv_j, h);
         }
       } else if (PART == REF_CHECK) {
-        // bj_rotation's own test: relative overlap above sqrt(rows) 2^-52 (and
-        // g above its floor 4 eps^2 ||X||^2); not a number is above both
+        // bj_rotation's own test: overlap above sqrt(rows) 2^-52 of the columns'
+        // norms as they are now (and g above its floor 4 eps^2 ||X||^2); not a
+        // number is above both
         const double g = G[at(j, i)];
         if (j < n && i < j)
-          bad |= !(fabsf((float)g) <= 0x1p-52f * sqrtf((float)ca)) &&
+          bad |= !(fabsf((float)g) <= 0x1p-52f * sqrtf((float)ca * (float)G[at(i, i)] * (float)G[at(j, j)])) &&
                  !(fabs(g) * Di * Dj <= 4.0 * DBL_EPSILON * DBL_EPSILON * D[0] * D[0]);
       } else {
         double k = 0.0;  // K_ij

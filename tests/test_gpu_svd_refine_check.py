@@ -1,9 +1,10 @@
-"""Not-a-numbers in the SVD refinement: the library refuses a non-finite
-wavefunction before the SVD, so the refinement's kernels are called on their own
-here.  A sector with a non-finite column, or with an overlap that is not a number,
-counts as unfinished (flag behind the job's permutation not 0: the final Jacobi
-sweeps it), and a non-finite column is handed on as it came; a sector of
-orthonormal columns is finished."""
+"""The check at the end of the SVD refinement, its kernels called on their own.
+
+Not-a-numbers: the library refuses a non-finite wavefunction before the SVD, so
+this is the second line of defence.  A sector with a non-finite column, or with an
+overlap that is not a number, counts as unfinished (flag behind the job's
+permutation not 0: the final Jacobi sweeps it), and a non-finite column is handed
+on as it came; a sector of orthonormal columns is finished."""
 import ctypes as C
 import os
 import re
@@ -41,8 +42,8 @@ PARTS = re.search(r"enum SvdRefine \{(.*?)\}", HEADER, re.S).group(1).replace(" 
 CA = 80  # two rows of tiles and a ragged third
 
 
-@pytest.mark.parametrize("what", ["finite", "column", "overlap"])
-def test_not_a_number_is_unfinished(what):
+def _sector():
+    """One sector of CA columns, norms 1 .. 0.1: job, arrays, call(part)."""
     import torch
     nn = CA * CA
     Job, refine = _struct("SvdJob"), _launcher("launch_svd_refine")
@@ -56,10 +57,7 @@ def test_not_a_number_is_unfinished(what):
     order = torch.zeros(1, device="cuda", dtype=torch.int32)
     X = torch.tensor(np.linalg.qr(np.random.default_rng(3).standard_normal((CA, CA)))[0], device="cuda")
     X = X * torch.linspace(1.0, 0.1, CA, device="cuda", dtype=torch.float64)[:, None]  # row j: column j of X
-    if what == "column":
-        X[70, 5] = float("nan")
     area = lambda off: work[off:off + nn].view(CA, CA)
-    area(job.b_off).copy_(X)
     area(job.j_off).copy_(torch.eye(CA))
 
     def part(name, stage=0):
@@ -69,6 +67,16 @@ def test_not_a_number_is_unfinished(what):
         assert s == 0
         torch.cuda.synchronize()
 
+    return job, X, area, iwork, part
+
+
+@pytest.mark.parametrize("what", ["finite", "column", "overlap"])
+def test_not_a_number_is_unfinished(what):
+    import torch
+    job, X, area, iwork, part = _sector()
+    if what == "column":
+        X[70, 5] = float("nan")
+    area(job.b_off).copy_(X)
     part("REF_SCALE")
     area(job.x_off).copy_(area(job.b_off) @ area(job.b_off).T)
     if what == "overlap":
@@ -79,3 +87,19 @@ def test_not_a_number_is_unfinished(what):
         got = area(job.b_off)
         assert torch.equal(torch.isnan(got), torch.isnan(X))
         assert (got - X).abs().nan_to_num().max().item() < 1e-15
+
+
+@pytest.mark.parametrize("norm2,overlap,finished", [(1.0, 0.9, True), (1.0, 1.1, False), (4.0, 3.9, True), (4.0, 4.1, False),
+                                                    (0.25, 0.24, True), (0.25, 0.26, False)])
+def test_overlaps_count_against_the_norms(norm2, overlap, finished):
+    """The threshold sqrt(columns) 2^-52 is of g / (|x_i| |x_j|), whatever the
+    corrections made of the norms."""
+    import torch
+    job, X, area, iwork, part = _sector()
+    area(job.b_off).copy_(X)
+    part("REF_SCALE")
+    G = norm2 * torch.eye(CA, device="cuda", dtype=torch.float64)
+    G[70, 3] = G[3, 70] = overlap * CA**0.5 * 2.0**-52
+    area(job.x_off).copy_(G)
+    part("REF_CHECK")
+    assert (iwork[CA + 3].item() == 0) == finished
