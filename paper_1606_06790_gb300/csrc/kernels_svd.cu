@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "common.h"
+#include "jacobi_rotation.h"
 
 namespace cg = cooperative_groups;
 
@@ -1944,22 +1945,6 @@ constexpr int JS_THREADS = 32 * JS_BW_MAX;
 __host__ __device__ constexpr int js_qld(int bw_cap) { return (2 * bw_cap + 7) & ~7; }
 __host__ __device__ constexpr int64_t js_smem_floats(int bw_cap, int ldb) {
   return 2 * (int64_t)bw_cap * ldb + (int64_t)js_qld(bw_cap) * 2 * bw_cap + 2 * bw_cap;
-}
-
-// The rotation that makes columns of squared norms a, b and overlap g
-// orthogonal, in FP32: false if their relative overlap is at most tol.
-__device__ __forceinline__ bool js_rotation(float a, float b, float g, float tol, float &ratio, float &t, float &c,
-                                            float &sn) {
-  if (!(a > 0.f) || !(b > 0.f)) return false;
-  ratio = fabsf(g) * rsqrtf(a) * rsqrtf(b);
-  if (!(ratio > tol)) return false;
-  const float z = __fdividef(b - a, 2.0f * g);
-  const float q = fmaf(z, z, 1.0f);
-  t = z == 0.f ? 1.0f : copysignf(__fdividef(1.0f, fabsf(z) + q * rsqrtf(q)), z);
-  if (!(fabsf(t) >= FLT_MIN) || !isfinite(t)) return false;
-  c = rsqrtf(fmaf(t, t, 1.0f));
-  sn = c * t;
-  return true;
 }
 
 // V's columns of blocks b0 (nv0 valid ones) and b1 times Q, whose 2 bw rows are
