@@ -410,10 +410,10 @@ idmrg_status idmrg_profile_read(idmrg_ctx *ctx, int kclass, double *ms, uint64_t
 
 /* Sector SVDs of the following truncations on the kernels for large sector
  * matrices only (global_only = 1: pivoted QR on thread-block clusters with
- * the columns in global memory, FP32 and FP64 cyclic Jacobi in global
- * memory), or on the size-dependent choice (0, the
- * default: sectors with at most 320 columns use the shared-memory block
- * kernels).  The results agree to rounding; this exists to test the
+ * the columns in global memory, FP32 block Jacobi streamed from global through
+ * shared memory, FP64 cyclic Jacobi in global memory), or on the size-dependent
+ * choice (0, the default: sectors with at most 320 columns use the
+ * shared-memory block kernels).  The results agree to rounding; this exists to test the
  * large-sector path on small problems. */
 idmrg_status idmrg_set_svd_path(idmrg_ctx *ctx, int global_only);
 

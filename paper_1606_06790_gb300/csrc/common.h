@@ -240,6 +240,10 @@ cudaError_t launch_svd_jacobi(const SvdJob *jobs, const int *order, int njobs, c
 cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs, const int *g, const int *cols,
                                 int cols0, double *work, const int *iwork, cudaStream_t st,
                                 const cudaStream_t *side, const cudaEvent_t *ev);
+// its large-sector stage on the jobs order[0 .. njobs) of at most `cols` columns,
+// a cluster of csize CTAs (16 or 8) each
+cudaError_t launch_jacobi32_stream(const SvdJob *jobs, const int *order, int njobs, int cols, int csize,
+                                   double *work, const int *iwork, cudaStream_t st);
 // per job over cols_a x cols_a elements: 0: V = I; 1: V = 1.5 V - 0.5 W
 // (Newton-Schulz step, W at w_off); 2: B = X (X at w_off), and the final Jacobi
 // is to run on sectors that are not refined

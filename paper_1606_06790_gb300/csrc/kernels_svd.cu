@@ -819,153 +819,11 @@ __device__ __forceinline__ void iwork32_sweeps(const int *iwork, const SvdJob &J
   const_cast<int *>(iwork)[J.perm_off + J.cols_a + 2] = sweep;
 }
 
-// FP32 stage (see jacobi32_block_kernel) for sector matrices too large for
-// the block kernels: the cyclic tournament of jacobi_kernel on FP32 copies
-// of B and of the rotations, kept in the job's x_off area (cols_a x cols_a
-// doubles, free until the Newton-Schulz step), one pair per warp, rounds
-// separated by the cluster barrier.  Ends by writing the rotations to V
-// (FP64, leading dimension cols_a) over the identity already there.
-// A pair's columns are read and written in batches of J32_BATCH elements per
-// lane whose loads are all issued before they are used: with the columns in
-// L2 or HBM, a plain strided loop waits on the load latency once per 32
-// elements of each column.
-constexpr int J32_BATCH = 8;
+// A pair's columns in global memory are read and written in batches of J64_BATCH
+// elements per lane whose loads are all issued before they are used: with the
+// columns in L2 or HBM, a plain strided loop waits on the load latency once per
+// 32 elements of each column.
 constexpr int J64_BATCH = 8;
-
-__device__ __forceinline__ void dots32(const float *xp, const float *xq, int len, int lane, float &a, float &b,
-                                       float &g) {
-  // two batches in flight; each lane adds its elements in index order
-  for (int i0 = 0; i0 < len; i0 += 64 * J32_BATCH) {
-    float u[2 * J32_BATCH], v[2 * J32_BATCH];
-#pragma unroll
-    for (int r = 0; r < 2 * J32_BATCH; ++r) {
-      const int i = i0 + lane + 32 * r;
-      u[r] = i < len ? xp[i] : 0.f;
-      v[r] = i < len ? xq[i] : 0.f;
-    }
-#pragma unroll
-    for (int r = 0; r < 2 * J32_BATCH; ++r) {
-      a = fmaf(u[r], u[r], a);
-      b = fmaf(v[r], v[r], b);
-      g = fmaf(u[r], v[r], g);
-    }
-  }
-}
-
-// the rotation of a pair of B columns (length len) and of the same pair of
-// rotation columns (length lenv <= len) in one pass
-__device__ __forceinline__ void rot32x2(float *xp, float *xq, int len, float *vp, float *vq, int lenv, int lane,
-                                        float c, float sn) {
-  for (int i0 = 0; i0 < len; i0 += 32 * J32_BATCH) {
-    float u[J32_BATCH], v[J32_BATCH], y[J32_BATCH], z[J32_BATCH];
-#pragma unroll
-    for (int r = 0; r < J32_BATCH; ++r) {
-      const int i = i0 + lane + 32 * r;
-      u[r] = i < len ? xp[i] : 0.f;
-      v[r] = i < len ? xq[i] : 0.f;
-      y[r] = i < lenv ? vp[i] : 0.f;
-      z[r] = i < lenv ? vq[i] : 0.f;
-    }
-#pragma unroll
-    for (int r = 0; r < J32_BATCH; ++r) {
-      const int i = i0 + lane + 32 * r;
-      if (i < len) {
-        xp[i] = c * u[r] - sn * v[r];
-        xq[i] = fmaf(sn, u[r], c * v[r]);
-      }
-      if (i < lenv) {
-        vp[i] = c * y[r] - sn * z[r];
-        vq[i] = fmaf(sn, y[r], c * z[r]);
-      }
-    }
-  }
-}
-
-__global__ void __launch_bounds__(JAC_THREADS, 2)
-    jacobi32_kernel(const SvdJob *__restrict__ jobs, const int *__restrict__ order, double *__restrict__ work,
-                    const int *__restrict__ iwork) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank();
-  const int csize = (int)cluster.num_blocks();
-  const SvdJob Jb = jobs[order[blockIdx.x / csize]];
-  const int nr = Jb.cols_a;
-  const int n = iwork[Jb.perm_off + Jb.cols_a];
-  float *B32 = reinterpret_cast<float *>(work + Jb.x_off);  // nr x n, then n x n rotations
-  float *V32 = B32 + (int64_t)nr * n;
-  const double *Bg = work + Jb.b_off;
-  double *Vg = work + Jb.j_off;
-  __shared__ int flag, local_changed, sweep_rmax, cl_rmax;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int gw = warp * csize + crank, gnw = csize * nw;
-  const int64_t stride = (int64_t)csize * blockDim.x, e0 = (int64_t)crank * blockDim.x + threadIdx.x;
-  if (n < 2) return;  // uniform over the cluster
-  for (int64_t e = e0; e < (int64_t)nr * n; e += stride) B32[e] = (float)Bg[e];
-  for (int64_t e = e0; e < (int64_t)n * n; e += stride) V32[e] = (e / n == e % n) ? 1.0f : 0.0f;
-  const float tol = sqrtf((float)nr) * FLT_EPSILON;
-  const int np = n + (n & 1);
-  int *flag0 = cluster.map_shared_rank(&flag, 0);
-  int *rmax0 = cluster.map_shared_rank(&cl_rmax, 0);
-  auto wsumf = [](float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  };
-  bool converged = false;
-  int sweep = 0;
-  for (; sweep < 15 && !converged; ++sweep) {
-    if (threadIdx.x == 0) {
-      local_changed = 0;
-      sweep_rmax = 0;
-    }
-    if (crank == 0 && threadIdx.x == 0) {
-      flag = 0;
-      cl_rmax = 0;
-    }
-    cluster.sync();
-    bool any = false;
-    float rmax = 0.f;
-    for (int rnd = 0; rnd < np - 1; ++rnd) {
-      for (int k = gw; k < np / 2; k += gnw) {
-        const int i1 = k, i2 = np - 1 - k;
-        const int p = i1 == 0 ? 0 : 1 + (i1 - 1 + rnd) % (np - 1);
-        const int q = i2 == 0 ? 0 : 1 + (i2 - 1 + rnd) % (np - 1);
-        if (p >= n || q >= n) continue;
-        float *xp = B32 + (int64_t)p * nr, *xq = B32 + (int64_t)q * nr;
-        float a = 0.f, b = 0.f, g = 0.f;
-        dots32(xp, xq, nr, lane, a, b, g);
-        a = wsumf(a);
-        b = wsumf(b);
-        g = wsumf(g);
-        if (!(a > 0.f) || !(b > 0.f)) continue;
-        const float ratio = fabsf(g) / sqrtf(a) / sqrtf(b);
-        if (!(ratio > tol)) continue;
-        const float z = (b - a) / (2.0f * g);
-        const float t = z == 0.f ? 1.0f : copysignf(1.0f, z) / (fabsf(z) + sqrtf(fmaf(z, z, 1.0f)));
-        if (!(fabsf(t) >= FLT_MIN) || !isfinite(t)) continue;
-        const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
-        rot32x2(xp, xq, nr, V32 + (int64_t)p * n, V32 + (int64_t)q * n, n, lane, c, sn);
-        any = true;
-        rmax = fmaxf(rmax, ratio);
-      }
-      cluster.sync();
-    }
-    if (any && lane == 0) local_changed = 1;
-    if (lane == 0) atomicMax(&sweep_rmax, __float_as_int(rmax));
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (local_changed) atomicOr(flag0, 1);
-      atomicMax(rmax0, sweep_rmax);
-    }
-    cluster.sync();
-    const float r = __int_as_float(*rmax0);
-    converged = (*flag0 == 0) || ((float)n * r * r < tol) || r < J32_PRECOND_R;
-    cluster.sync();
-  }
-  if (crank == 0 && threadIdx.x == 0) iwork32_sweeps(iwork, Jb, sweep);
-  for (int64_t e = e0; e < (int64_t)n * n; e += stride) {
-    const int64_t j = e / n, i = e - j * n;
-    Vg[j * nr + i] = (double)V32[e];
-  }
-}
 
 // ------------------------------------------------- block Jacobi (shared memory)
 // Same rotations as jacobi_kernel, ordered by blocks so that the columns stay
@@ -2727,23 +2585,6 @@ static cudaError_t launch_jacobi_clusters(const SvdJob *jobs, const int *order, 
   return cudaLaunchKernelEx(&cfg, jacobi_kernel, jobs, order, work, iwork, sv, err, jm_init);
 }
 
-static cudaError_t launch_jacobi32_clusters(const SvdJob *jobs, const int *order, int njobs, int csize,
-                                            double *work, const int *iwork, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(njobs * csize, 1, 1);
-  cfg.blockDim = dim3(JAC_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = csize;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, jacobi32_kernel, jobs, order, work, iwork);
-}
-
 // shared memory of the block kernel for a job of `cols` columns in clusters
 // of `csize` (the rank is at most cols): four blocks of B and Jm columns
 size_t svd_block_smem(int cols, int csize) {
@@ -2914,11 +2755,10 @@ static cudaError_t launch_block32_clusters(const SvdJob *jobs, const int *order,
   return cudaLaunchKernelEx(&cfg, jacobi32_block_kernel, jobs, order, work, iwork);
 }
 
-// jacobi32_stream_kernel on the jobs order[0 .. njobs) of at most `cols` columns
-static cudaError_t launch_jacobi32_stream(const SvdJob *jobs, const int *order, int njobs, int cols, int csize,
+cudaError_t launch_jacobi32_stream(const SvdJob *jobs, const int *order, int njobs, int cols, int csize,
                                           double *work, const int *iwork, cudaStream_t st) {
   const int ldb = 32 * ((cols + 31) / 32);
-  const int64_t budget = 200 * 1024 / (int)sizeof(float);
+  const int64_t budget = SVD_BLOCK_SMEM_MAX / sizeof(float);
   int bw_cap = std::min(JS_BW_MAX, (cols + 2 * csize - 1) / (2 * csize));
   while (bw_cap >= 1 && js_smem_floats(bw_cap, ldb) > budget) --bw_cap;
   if (bw_cap < 1) return cudaErrorInvalidValue;
@@ -2930,7 +2770,8 @@ static cudaError_t launch_jacobi32_stream(const SvdJob *jobs, const int *order, 
                             : jacobi32_stream_kernel<0>;
   const size_t smem = (size_t)js_smem_floats(bw_cap, ldb) * sizeof(float);
   cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit holds for the process: the same for every caller)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SVD_BLOCK_SMEM_MAX);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(njobs * csize, 1, 1);
@@ -2959,18 +2800,13 @@ cudaError_t launch_svd_jacobi32(const SvdJob *jobs, const int *order, int njobs,
   e = cudaEventRecord(ev[0], st);
   if (e != cudaSuccess) return e;
   // beyond the block kernels: the block tournament streamed through shared
-  // memory; the all-global pair kernel if asked for, or if that launch is not
-  // possible (no 16-CTA clusters).  First: a cluster of 16 needs a GPC's SMs free
+  // memory, on clusters of 16 CTAs, or of 8 where the device has none of 16.
+  // First: a cluster of 16 needs a GPC's SMs free
   if (hi[0] > lo[0]) {
     e = launch_jacobi32_stream(jobs, order, hi[0], cols0, 16, work, iwork, st);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      cudaFuncSetAttribute(jacobi32_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      e = launch_jacobi32_clusters(jobs, order, hi[0], 16, work, iwork, st);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        e = launch_jacobi32_clusters(jobs, order, hi[0], 8, work, iwork, st);
-      }
+      e = launch_jacobi32_stream(jobs, order, hi[0], cols0, 8, work, iwork, st);
     }
     if (e != cudaSuccess) return e;
   }

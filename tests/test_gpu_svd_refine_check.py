@@ -6,37 +6,14 @@ overlap that is not a number, counts as unfinished (flag behind the job's
 permutation not 0: the final Jacobi sweeps it), and a non-finite column is handed
 on as it came; a sector of orthonormal columns is finished."""
 import ctypes as C
-import os
 import re
-import subprocess
 
 import numpy as np
 import pytest
 
-import paper_1606_06790_gb300 as pkg
+from internal_calls import HEADER, launcher, struct
 
 pytestmark = pytest.mark.gpu
-
-CSRC = os.path.join(os.path.dirname(pkg.__file__), "csrc")
-HEADER = open(os.path.join(CSRC, "common.h")).read()
-
-
-def _struct(name):
-    body = re.search(r"struct %s \{(.*?)\n\};" % name, HEADER, re.S).group(1)
-    fields = []
-    for kind, names in re.findall(r"^\s*(int64_t|int|float|double) ([^;]+);", body, re.M):
-        t = {"int64_t": C.c_int64, "int": C.c_int, "float": C.c_float, "double": C.c_double}[kind]
-        for n in names.split(","):
-            m = re.match(r"\s*(\w+)(?:\[(\d+)\])?\s*$", n)
-            fields.append((m.group(1), t * int(m.group(2)) if m.group(2) else t))
-    return type(name, (C.Structure,), {"_fields_": fields})
-
-
-def _launcher(name):
-    lib = pkg.load_library()
-    symbols = subprocess.run(["nm", "-D", lib._name], capture_output=True, text=True, check=True).stdout.split()
-    return getattr(lib, next(s for s in symbols if re.match(r"_ZN5idmrg%d%s" % (len(name), name), s)))
-
 
 PARTS = re.search(r"enum SvdRefine \{(.*?)\}", HEADER, re.S).group(1).replace(" ", "").split(",")
 CA = 80  # two rows of tiles and a ragged third
@@ -46,7 +23,7 @@ def _sector():
     """One sector of CA columns, norms 1 .. 0.1: job, arrays, call(part)."""
     import torch
     nn = CA * CA
-    Job, refine = _struct("SvdJob"), _launcher("launch_svd_refine")
+    Job, refine = struct("SvdJob"), launcher("launch_svd_refine")
     job = Job(r=CA, c=CA, rows_a=CA, cols_a=CA, a_off=0, j_off=nn, b_off=2 * nn, x_off=3 * nn, tau_off=4 * nn,
               w_off=4 * nn + CA, t_off=5 * nn + CA, perm_off=0, sv_off=0)
     work = torch.zeros(8 * nn + CA, device="cuda", dtype=torch.float64)
