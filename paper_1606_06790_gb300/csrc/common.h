@@ -293,7 +293,7 @@ struct PackSeg {
   int kpad;               // zero columns to write after the segment
   int whole;              // digit form: the segment holds the whole K range of its rows
   int exp_buf;            // digit form: slot of the exponent array
-  double alpha;           // source values scaled by alpha
+  double alpha;           // digit form: source values scaled by alpha (split form: taken as they are)
 };
 struct WTaskP {           // rows of a packed stage-3 A matrix: one (left sector, s, t)
   int64_t dst_off;
