@@ -443,7 +443,7 @@ idmrg_status idmrg_svd_sweeps32(const idmrg_ctx *ctx, int *max_sweeps, double *m
 /* Milliseconds spent, since profiling was last enabled, in the phases of the
  * sector SVD of Step 4 (parts of IDMRG_K_SVD, event-timed on the context's
  * stream): ms[0] gather and pivoted QR, ms[1] FP32 Jacobi, ms[2]
- * Newton-Schulz orthogonalisation and X = B V, ms[3] FP64 Jacobi, ms[4]
+ * Newton-Schulz orthogonalisation, X = B V and refinement, ms[3] FP64 Jacobi, ms[4]
  * selection of the kept states, ms[5] compaction into U and V.  ms holds 6
  * entries. */
 idmrg_status idmrg_svd_phase_ms(idmrg_ctx *ctx, double *ms);

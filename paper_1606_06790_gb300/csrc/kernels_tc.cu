@@ -958,7 +958,10 @@ static_assert(OZ_SMEM <= 227 * 1024, "shared memory of a CTA");
 // Measured (GB300; before: one CTA per tile of 32-element K blocks, 36 MMAs of 64
 // columns per 16 of K, the epilogue in FP64 by the row): the two stages of the
 // kagome cylinder's H_eff psi at m = 1500 13.1 -> 4.4 ms (39 TFLOP/s
-// FP64-accurate), of the J1-J2 cylinder at m = 500 0.81 -> 0.28 ms.
+// FP64-accurate), of the J1-J2 cylinder at m = 500 0.81 -> 0.28 ms.  By ncu
+// (kagome, m = 1000) the tensor pipe is active 87 % of the cycles in stage 3 (long
+// K), close to what the operand reads allow (0.91), and 70 % in stage 1, whose
+// tiles have few K blocks beside their read-out (FP64 pipe 29 %); L2 at 26 %.
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const TcTile *__restrict__ tiles, int ntiles,
                                                                 const TcTask *__restrict__ tasks,
                                                                 double *const *__restrict__ bufs,
