@@ -157,9 +157,10 @@ def class_roofline(name: str, d: dict, prec: str, pk: dict):
     against the measured sustained bf16 peak (times the nominal tf32/bf16
     ratio for TF32): the split H_eff GEMMs (3 MMAs per product) and, in the
     mixed and FP64_TC forms, the FP64-accurate digit-slice GEMMs of the
-    environments, the prediction and the restart matvecs (36 BF16 MMAs per
-    FP64 product).  `executed_frac` is the same fraction with the MMAs the
-    pipe executes.  The W stage and psi split of the mixed H_eff and the
+    environments, the prediction and the restart matvecs (36 BF16 digit
+    products per FP64 product).  `executed_frac` is the same fraction with
+    these products counted (the zero planes that fill the digit GEMM's MMAs
+    are not).  The W stage and psi split of the mixed H_eff and the
     Lanczos vector kernels are HBM streams (algorithmic bytes booked by the
     library); the SVD (its R-SVD flop count at FP64 accuracy) and the FP64
     forms against the FP64 units: 152 SMs x 2 FMA/clk x 2.07 GHz.  In the
@@ -175,7 +176,7 @@ def class_roofline(name: str, d: dict, prec: str, pk: dict):
         achieved = d["flops"] / sec / 1e12 if sec > 0 else 0.0
         src = "sustained bf16" if bf else "sustained bf16 x nominal tf32/bf16 (1.1/2.25)"
         prod = 36 if digit else 3
-        what = ("FP64-accurate products counted once (36 BF16 digit MMAs each)" if digit
+        what = ("FP64-accurate products counted once (36 BF16 digit products each)" if digit
                 else "split products counted once (3 MMAs each)")
         out.update({"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "peak_source": f"{pk['src']} {src}; {what}", "products_per_flop": prod})
