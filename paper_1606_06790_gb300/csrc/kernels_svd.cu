@@ -1792,7 +1792,7 @@ __global__ void __launch_bounds__(BJ_THREADS, 2)
 // Measured (GB300; before: sectors of up to 640 columns on a kernel that held B
 // in shared memory and V's columns in L2, a round trip per pair): FP32 stage of
 // a step of the J1-J2 cylinder at m = 1024 (sectors of up to 566 columns) 49 ->
-// 23 ms, of the kagome cylinder at m = 1000 127 -> 30 ms.  A visit of 17 + 17
+// 23 ms, of the kagome cylinder at m = 1000 127 -> 31 ms.  A visit of 17 + 17
 // columns of 537 rows took 30 k cycles in its sub-rounds and 58 k in V Q (a
 // branch between any two loads of Q) before js_apply_q.
 constexpr int JS_BW_MAX = 20;  // columns per block: a row of the two blocks of V fits in registers
@@ -2603,8 +2603,10 @@ size_t svd_block_smem(int cols, int csize) {
 // and keep 16.  Measured (GB300, ms of a step, all groups; before: 16 CTAs, group
 // 1 after group 0 on one stream): J1-J2 cylinder at m = 1024 QR 10.7 -> 9.5, FP32
 // Jacobi 21.7 -> 20.4, final Jacobi 7.4 -> 6.0; kagome at m = 1000 FP32 Jacobi
-// 31.0 -> 28.7; sectors of 148 columns (random chain, m = 256) QR 1.07 -> 1.01,
-// FP32 Jacobi 1.12 with 16 CTAs, 1.66 with 8.
+// 31.0 -> 28.7 (22.5 and 31.0 since its rotations divide in full precision);
+// sectors of 148 columns (random chain, m = 256) QR 1.07 -> 1.01, FP32 Jacobi 1.12
+// with 16 CTAs, 1.66 with 8.  The count is that of the GB300s measured; on a part
+// that holds another number the choice costs time, never the result.
 constexpr int SVD_CLUSTERS_16 = 7;
 constexpr size_t SVD_SHARED_SM = 64 * 1024;  // at least three such CTAs on an SM
 static int group1_csize(int jobs01, bool crowded, bool fits8) {
